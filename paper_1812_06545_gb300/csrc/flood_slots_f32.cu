@@ -1,0 +1,6 @@
+// Flooding slot decoder: instances for FP32 messages.
+#include "flood_slots_kernel.cuh"
+
+namespace ldpc {
+template cudaError_t flood_slots_launch<float, false>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
+}  // namespace ldpc

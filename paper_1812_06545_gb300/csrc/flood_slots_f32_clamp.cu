@@ -1,0 +1,6 @@
+// Flooding slot decoder: instances for FP32 messages, upper clamp of |Q| at phi(X) applied.
+#include "flood_slots_kernel.cuh"
+
+namespace ldpc {
+template cudaError_t flood_slots_launch<float, true>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
+}  // namespace ldpc

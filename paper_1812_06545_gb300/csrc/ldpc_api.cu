@@ -214,17 +214,6 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
             if ((h.ent[b] >> 16) == j) h.colent[k++] = (b << 16) | (h.ent[b] & 0xffff);
     }
     h.colptr[nb] = k;
-    {
-        int n = 0;
-        for (int d = 2; d <= 9; d++) {
-            h.dbeg[d - 2] = n;
-            for (int l = 0; l < mb; l++) {
-                const int dl = h.rowptr[l + 1] - h.rowptr[l];
-                if (d < 9 ? dl == d : dl > 8) h.rord[n++] = l;
-            }
-        }
-        h.dbeg[8] = n;
-    }
     h.nnz = nnz;
     h.N = nb * Z;
     h.M = mb * Z;
@@ -232,9 +221,26 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
     h.E = nnz * Z;
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = ldpc::device_status_word(c->device, &h.status);
-    if (e == cudaSuccess) e = cudaMalloc(&c->dev, sizeof(CodeDev));
-    if (e == cudaSuccess) e = cudaMemcpy(c->dev, &h, sizeof(CodeDev), cudaMemcpyHostToDevice);
+    // one allocation: the code's description, then the flooding slot decoder's tables
+    c->n_ftab = h.dc_max <= 32 ? ldpc::flood_table_size(h) : 0;
+    const size_t head = (sizeof(CodeDev) + 255) & ~(size_t)255;
+    std::vector<char> img;
+    try {
+        img.resize(head + (size_t)4 * c->n_ftab * sizeof(int4));
+    } catch (const std::bad_alloc &) {
+        delete c;
+        return fail(LDPC_ENOMEM, "host allocation failed");
+    }
+    int4 *tab = reinterpret_cast<int4 *>(img.data() + head);
+    if (c->n_ftab)
+        for (int v = 0; v < 4; v++)
+            ldpc::flood_build_table(h, v < 2 ? LDPC_MSG_F32 : LDPC_MSG_F16, 1 + (v & 1), tab + (size_t)v * c->n_ftab);
+    memcpy(img.data(), &h, sizeof h);
+    if (e == cudaSuccess) e = cudaMalloc(&c->dev, img.size());
+    if (e == cudaSuccess) e = cudaMemcpy(c->dev, img.data(), img.size(), cudaMemcpyHostToDevice);
+    c->ftab = reinterpret_cast<int4 *>(reinterpret_cast<char *>(c->dev) + head);
     if (e != cudaSuccess) {
+        if (c->dev) cudaFree(c->dev);
         delete c;
         return cuda_fail(e, "device code tables");
     }

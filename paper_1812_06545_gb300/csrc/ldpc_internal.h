@@ -30,10 +30,8 @@ struct CodeDev {
     int32_t colptr[NB_MAX + 1];  // entries of block column j: [colptr[j], colptr[j+1])
     int32_t colent[NNZ_MAX];     // (b << 16) | s for those blocks
     unsigned int *status;        // the device's input status word (library-owned, one per device)
-    // block rows by degree: rord[dbeg[d - 2] .. dbeg[d - 1]) are the rows of degree d (2..8),
-    // rord[dbeg[7] .. dbeg[8]) those above degree 8 (for the flooding slot decoder)
-    int32_t rord[MB_MAX];
-    int32_t dbeg[12];
+    // block rows and columns in ascending degree: end of each degree class (flood_slots.h)
+    uint8_t rend[11], cend[5];
 };
 
 // Bits of the input status word: kernels that load channel LLRs set them (atomicOr, only
@@ -93,24 +91,6 @@ struct ReqDev {
     int64_t n_cw;
     int64_t item0;  // index of its first codeword in its group's work sequence
 };
-struct GroupDev {
-    const CodeDev *code;
-    int C;       // slots per CTA for this code
-    int K, TPG;  // thread slots per barrier group; threads per group (whole warps)
-    int req_begin, req_end;
-    int N, E, Z, mb, nb, nnz, dc_max;
-    int64_t n_items;
-    float cumw;  // cumulative share of the launch's work (initial CTA placement)
-    // single slots: thread groups of Z threads a slot's block rows and columns are spread over
-    // (1 unless a small batch leaves threads to spare).  Kept last: the field ahead of the
-    // others changed the slot decoder's parameter loads and cost it 2-3 % (measured).
-    int W;
-};
-struct MultiDesc {
-    int n_groups;
-    GroupDev groups[MULTI_MAX_GROUPS];
-    ReqDev reqs[MULTI_MAX_REQS];
-};
 struct HostReq {
     const ldpc_code *code;
     const void *llr;
@@ -141,6 +121,10 @@ cudaError_t flood_cluster_decode(const CodeDev &host, const CodeDev *dev, const 
 // Flooding SPA slot decoder: supported when one codeword of the code fits a CTA.
 int slots_supported(const CodeDev &host, int msg);
 int slots_pairable(const CodeDev &host, int msg);
+// Its tables of a code: their elements, and building those for V codewords per thread (also
+// sets the code's degree classes).
+int flood_table_size(const CodeDev &host);
+void flood_build_table(CodeDev &host, int msg, int V, int4 *tab);
 cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters,
                                cudaStream_t s);
 
@@ -159,6 +143,8 @@ struct ldpc_code {
     ldpc::CodeDev host;
     ldpc::CodeDev *dev;
     int device;
+    int4 *ftab;          // flooding slot decoder's tables: [2 * (F16) + V - 1][n_ftab] (flood_slots.h)
+    int n_ftab;
     int tuned_flood[2];  // per message type (F32, F16)
     int tuned_layered;
 };
