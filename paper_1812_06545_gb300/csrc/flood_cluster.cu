@@ -15,19 +15,32 @@
 //                      codeword has converged (its APP from that iteration is final)
 //   variable-node phase otherwise every owned variable: APP = L + sum of the new R
 // A finished codeword is written out and the cluster's leader takes the next codeword from
-// the global work counter.  Messages sit in check-row order, edge (b, r) of the owned block b
-// at (b - first owned block) * Z + r; posteriors at (j - first owned column) * Z + c.
+// the global work counter.  Messages are stored negated at the variable's position inside the
+// block, edge (b, r) of the owned block b at (b - first owned block) * Z + (r + s) mod Z;
+// posteriors at (place of column j) * Z + c.
+//
+// Threads: W row groups of whole warps; thread r of row group w owns row r of every W-th owned
+// block row and position r of every W-th owned column, both in ascending degree, so that a
+// warp runs one straight-line body at a time (flood_check.cuh).  The table entries hold
+// complete shared::cluster addresses (own CTA or the other), so an operand in either CTA costs one add.
+// Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB: 6727 -> 5430 us per launch,
+// 71 -> 55 warp instructions per edge update (bound by instruction issue, 65 %).
 #include <string.h>
 
 #include <cooperative_groups.h>
 
-#include "slot_common.cuh"
+#include "flood_check.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace ldpc {
 
 constexpr int CLUSTER_CTAS = 2;
+constexpr int CL_CLASSES = 11;  // row degree classes: 2..8 exact, then up to 12, 16, 24, 32
+__host__ __device__ constexpr int cl_class_degree(int c)
+{
+    return c < 7 ? c + 2 : c == 7 ? 12 : c == 8 ? 16 : c == 9 ? 24 : 32;
+}
 
 // One launch decodes every codeword of up to MULTI_MAX_REQS requests of one code: the codewords
 // are the items of one work sequence (request i's are items item0 .. item0 + n_cw - 1).
@@ -39,16 +52,20 @@ struct ClusterArgs {
     int ncols[CLUSTER_CTAS];          // block columns CTA q holds the posteriors of
     int col_owner[NB_MAX];            // owner of block column j
     int col_slot[NB_MAX];             // its place among the owner's columns
-    int col_list[CLUSTER_CTAS][NB_MAX];  // CTA q's columns in place order
+    // CTA q's rows and columns in ascending degree, the ends of their degree classes, the
+    // rows' first edge descriptors, and the elements of its table
+    uint8_t row_list[CLUSTER_CTAS][MB_MAX], col_list[CLUSTER_CTAS][NB_MAX];
+    uint8_t rend[CLUSTER_CTAS][CL_CLASSES], cend[CLUSTER_CTAS][5];
+    uint16_t row_e0[CLUSTER_CTAS][MB_MAX], col_x0[CLUSTER_CTAS][NB_MAX];
+    int n_edge[CLUSTER_CTAS], n_tab[CLUSTER_CTAS];
+    int off_app, off_r;  // posteriors and messages, bytes from the start of shared memory
     int max_iter, early_exit;
     float X;
     ReqDev reqs[MULTI_MAX_REQS];
 };
 
 // 32-bit shared::cluster addresses: the address of shared variable p in CTA `rank` of the
-// cluster, and loads through such an address (the CTA's own memory or the other's).  Posteriors
-// and messages are read this way, so an operand's address is one 32-bit add from a per-owner
-// base, whichever CTA holds it.
+// cluster, and loads through such an address (the CTA's own memory or the other's).
 __device__ __forceinline__ uint32_t cl_map(const void *p, unsigned rank)
 {
     uint32_t out;
@@ -69,6 +86,10 @@ __device__ __forceinline__ float cl_ld(const __half *, uint32_t addr)
     asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(addr));
     return __half2float(__ushort_as_half(v));
 }
+__device__ __forceinline__ void cl_st(uint32_t addr, int x)
+{
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
+}
 
 __host__ __device__ inline int cl_owner(const int *split, int x)
 {
@@ -77,149 +98,92 @@ __host__ __device__ inline int cl_owner(const int *split, int x)
     return q;
 }
 
-// An owned row of degree <= 8 in the product (tanh) domain (see slot_common.cuh): d_k = e^-a_k
-// with a_k = |Q_k| clamped to [phi(X), X], the other edges' maps combined from prefix and
-// suffix pairs, R_k = ln(alpha / beta); one ex2 and two lg2 per edge.
-template <int D, bool EXACT, typename MsgT>
-__device__ __forceinline__ uint32_t cl_check_tanh(int dc, const int4 *__restrict__ ed, MsgT *Rr, uint32_t app_0,
-                                                  uint32_t app_1, int r, int Z, float Xb, float Pb)
-{
-    constexpr uint32_t kSign = 0x80000000u;
-    float d[D];
-    uint32_t qs[D];
-    uint32_t sg = 0, par = 0;
-    const uint32_t rb = 4u * (uint32_t)r, ZA = 4u * (uint32_t)Z;
-#pragma unroll
-    for (int k = 0; k < D; k++) {
-        d[k] = 0.0f;  // a missing edge (k >= dc) is the identity map
-        qs[k] = 0;
-        if (EXACT || k < dc) {
-            const int4 e = ed[k];
-            const float ap = cl_ld((const float *)nullptr, (e.z ? app_1 : app_0) + e.x + rb - (r >= e.y ? ZA : 0u));
-            const float qv = ap - (float)Rr[k * Z];
-            par ^= __float_as_uint(ap);
-            qs[k] = __float_as_uint(qv) & kSign;
-            sg ^= qs[k];
-            d[k] = tanh_d<false>(qv, Xb, Pb);
-        }
-    }
-    float sa[D + 1], sb[D + 1];
-    sa[D] = 1.0f;
-    sb[D] = 0.0f;
-    sa[D - 1] = 1.0f;
-    sb[D - 1] = d[D - 1];
-#pragma unroll
-    for (int k = D - 2; k >= 1; k--) {
-        sa[k] = fmaf(d[k], sb[k + 1], sa[k + 1]);
-        sb[k] = fmaf(d[k], sa[k + 1], sb[k + 1]);
-    }
-    float pa = 1.0f, pb = 0.0f;
-#pragma unroll
-    for (int k = 0; k < D; k++) {
-        float al, be;
-        if (k == 0) {
-            al = sa[1];
-            be = sb[1];
-        } else if (k == D - 1) {
-            al = pa;
-            be = pb;
-        } else {
-            tanh_combine(pa, pb, sa[k + 1], sb[k + 1], al, be);
-        }
-        if (EXACT || k < dc) {
-            Rr[k * Z] = MsgT(__uint_as_float(__float_as_uint(tanh_mag<false>(al, be)) | (qs[k] ^ sg)));
-        }
-        if (k == 0) {
-            pb = d[0];
-        } else if (k < D - 1) {
-            const float t = fmaf(d[k], pb, pa);
-            pb = fmaf(d[k], pa, pb);
-            pa = t;
-        }
-    }
-    return par;
-}
-
-// One check of an owned row: Q = APP - R over its edges (posteriors wherever they live), the
-// check rule in the product (tanh) domain (slot_common.cuh), messages written in place;
-// returns the parity of the posteriors' sign bits.  Rows above degree 8 take the grouped
-// form, with Q formed from APP and R in both passes.
-template <int D, bool EXACT, typename MsgT>
-__device__ __forceinline__ uint32_t cl_check(int dc, const int4 *__restrict__ ed, MsgT *Rr, uint32_t app_0,
-                                             uint32_t app_1, int r, int Z, float Xb, float Pb)
-{
-    if constexpr (D <= 8) {
-        return cl_check_tanh<D, EXACT, MsgT>(dc, ed, Rr, app_0, app_1, r, Z, Xb, Pb);
-    } else {
-        uint32_t par = 0;
-        const uint32_t rb = 4u * (uint32_t)r, ZA = 4u * (uint32_t)Z;
-        auto qof = [&](int k, bool first) -> float {
-            const int4 e = ed[k];
-            const float ap = cl_ld((const float *)nullptr, (e.z ? app_1 : app_0) + e.x + rb - (r >= e.y ? ZA : 0u));
-            if (first) par ^= __float_as_uint(ap);
-            return ap - (float)Rr[k * Z];
-        };
-        auto put = [&](int k, float m, float) { Rr[k * Z] = MsgT(m); };
-        if constexpr (D <= 12)  // hold the factors (no second remote load) where that does not spill
-            tanh_check_wide_held<D, false>(dc, Xb, Pb, [&](int k) { return qof(k, true); },
-                                           [&](int k, float m) { put(k, m, 0.0f); });
-        else
-            tanh_check_wide<D, false>(dc, Xb, Pb, qof, put);
-        return par;
-    }
-}
-
-template <int D, int DMAX, typename MsgT>
-__device__ __forceinline__ uint32_t cl_check_dispatch(int dc, const int4 *__restrict__ ent, MsgT *Rr,
-                                                      uint32_t app_0, uint32_t app_1, int r, int Z, float Xb,
-                                                      float Pb)
-{
-    if constexpr (D >= DMAX) {
-        return cl_check<DMAX, false, MsgT>(dc, ent, Rr, app_0, app_1, r, Z, Xb, Pb);
-    } else if constexpr (D <= 8) {
-        if (dc == D) return cl_check<D, true, MsgT>(dc, ent, Rr, app_0, app_1, r, Z, Xb, Pb);
-        return cl_check_dispatch<next_degree(D), DMAX, MsgT>(dc, ent, Rr, app_0, app_1, r, Z, Xb, Pb);
-    } else {
-        if (dc <= D) return cl_check<D, false, MsgT>(dc, ent, Rr, app_0, app_1, r, Z, Xb, Pb);
-        return cl_check_dispatch<next_degree(D), DMAX, MsgT>(dc, ent, Rr, app_0, app_1, r, Z, Xb, Pb);
-    }
-}
-
-// Sum of the messages of variable position c of one block column (column degree dv; entry
-// descriptors cd, see the kernel) onto sum, in the order of the column lists: straight-line
-// bodies for the common degrees (every lane of a warp takes the same branch).
-template <int D, typename MsgT>
-__device__ __forceinline__ float cl_vn_sum(const int4 *__restrict__ cd, uint32_t r_0, uint32_t r_1, int c, int Z,
-                                           float sum)
-{
-    constexpr uint32_t SZ = sizeof(MsgT);
-#pragma unroll
-    for (int k = 0; k < D; k++) {
-        const int4 d = cd[k];
-        sum += cl_ld((const MsgT *)nullptr, (d.z ? r_1 : r_0) + d.x + SZ * (uint32_t)c + (c < d.y ? SZ * Z : 0u));
-    }
-    return sum;
-}
+// A check's operands: the posterior at a shared::cluster address, the message in the own CTA.
 template <typename MsgT>
-__device__ __forceinline__ float cl_vn_column(int dv, const int4 *__restrict__ cd, uint32_t r_0, uint32_t r_1, int c,
-                                              int Z, float sum)
+struct ClusterMem {
+    char *sm;
+    __device__ __forceinline__ float app(uint32_t o) const { return cl_ld((const float *)nullptr, o); }
+    __device__ __forceinline__ float msg(uint32_t o) const { return Sm<MsgT, 1>::ld(sm + o); }
+    __device__ __forceinline__ void put(uint32_t o, float x) const { Sm<MsgT, 1>::st(sm + o, x); }
+    __device__ __forceinline__ float word(uint32_t o) const { return Sm<float, 1>::ld(sm + o); }
+    __device__ __forceinline__ void put_word(uint32_t o, float x) const { Sm<float, 1>::st(sm + o, x); }
+};
+
+// Row r of every W-th owned block row from list position i, in ascending degree (see rows_of of
+// the slot decoder).
+template <int CLS, int DMAX, typename MsgT, bool HC>
+__device__ __forceinline__ void cl_rows(const uint8_t *rend, const int4 *__restrict__ tab,
+                                        const int32_t *__restrict__ rows, const ClusterMem<MsgT> mem,
+                                        const Place<1> &p, float Xb, float Pb, uint32_t (&pbad)[1], int i, int step,
+                                        int W2)
 {
-    constexpr uint32_t SZ = sizeof(MsgT);
-    switch (dv) {
-    case 2: return cl_vn_sum<2, MsgT>(cd, r_0, r_1, c, Z, sum);
-    case 3: return cl_vn_sum<3, MsgT>(cd, r_0, r_1, c, Z, sum);
-    case 4: return cl_vn_sum<4, MsgT>(cd, r_0, r_1, c, Z, sum);
-    default:
-        for (int k = 0; k < dv; k++) {
-            const int4 d = cd[k];
-            sum += cl_ld((const MsgT *)nullptr, (d.z ? r_1 : r_0) + d.x + SZ * (uint32_t)c + (c < d.y ? SZ * Z : 0u));
+    constexpr int D = cl_class_degree(CLS);
+    if constexpr (D <= DMAX) {
+        const int end = rend[CLS];
+        for (; i < end; i += step, step = W2 - step) {
+            const int hd = rows[i];
+            if constexpr (D <= 8)
+                check_narrow<D, 1, MsgT, false, HC>(tab + (hd >> 8), mem, p, Xb, Pb, pbad);
+            else if constexpr (D == 12)
+                check_12<1, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
+            else
+                check_wide<D / 8, 1, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
         }
-        return sum;
+        if constexpr (CLS + 1 < CL_CLASSES)
+            cl_rows<CLS + 1, DMAX, MsgT, HC>(rend, tab, rows, mem, p, Xb, Pb, pbad, i, step, W2);
     }
 }
 
-// Shared memory ahead of the posterior array: flags and codeword (16 bytes), the block-row
-// and block-column pointers, then two descriptors (int4) per block.
+// Position r of every W-th owned column from list position i, in ascending degree: APP = L + the
+// column's messages in block-row order.  Lr: channel values at position r of block column 0;
+// rb: the thread's byte offset in a block of messages; A: its place in the posteriors.
+constexpr int kClChunk = 4;  // columns whose channel values a thread requests at once
+template <int DV, typename MsgT>
+__device__ __forceinline__ void cl_cols(const uint8_t *cend, const int4 *__restrict__ ctab,
+                                        const int4 *__restrict__ tab, const int32_t *__restrict__ cols,
+                                        const float *__restrict__ Lr, uint32_t rb, float *A, int Z, bool own, int i,
+                                        int W)
+{
+    const int end = cend[DV - 1];
+    auto add = [&](float s, int addr) { return s - cl_ld((const MsgT *)nullptr, rb + (uint32_t)addr); };
+    for (; i < end;) {
+        float lv[kClChunk];
+        int jc[kClChunk];
+#pragma unroll
+        for (int c = 0; c < kClChunk; c++) {
+            lv[c] = 0.0f;
+            jc[c] = 0;
+            if (c == 0 || i + c * W < end) {
+                jc[c] = cols[i + c * W];
+                lv[c] = __ldg(Lr + (jc[c] & 255) * Z);
+            }
+        }
+#pragma unroll
+        for (int c = 0; c < kClChunk; c++) {
+            if (c == 0 || i < end) {
+                const int4 o = ctab[i];
+                float s = add(lv[c], o.x);
+                if constexpr (DV > 1) s = add(s, o.y);
+                if constexpr (DV > 2) s = add(s, o.z);
+                if constexpr (DV == 4) s = add(s, o.w);
+                if constexpr (DV == 5) {
+                    const int4 *m = tab + (o.w >> 8);
+                    for (int k = o.w & 255; k > 0; k -= 4, m++) {
+                        s = add(s, m->x);
+                        if (k > 1) s = add(s, m->y);
+                        if (k > 2) s = add(s, m->z);
+                        if (k > 3) s = add(s, m->w);
+                    }
+                }
+                if (own) A[(jc[c] >> 8) * Z] = s + 0.0f;  // -0 -> +0: the sign bit is the decision
+                i += W;
+            }
+        }
+    }
+    if constexpr (DV < 5) cl_cols<DV + 1, MsgT>(cend, ctab, tab, cols, Lr, rb, A, Z, own, i, W);
+}
+
+// Shared memory ahead of the posterior array (flags, codeword, tables; see the kernel).
 __host__ __device__ inline size_t cl_tables_bytes(int nnz)
 {
     return (((size_t)16 + 4 * (MB_MAX + 1 + NB_MAX + 1) + 15) & ~(size_t)15) + (size_t)32 * nnz;
@@ -227,76 +191,71 @@ __host__ __device__ inline size_t cl_tables_bytes(int nnz)
 
 // threads per CTA: higher check degrees keep more values live per thread
 template <int DMAX>
-constexpr int cl_threads() { return DMAX <= 8 ? 1024 : (DMAX <= 16 ? 768 : 512); }
+constexpr int cl_threads() { return DMAX <= 12 ? 768 : 512; }
 
-template <int DMAX, typename MsgT>
+template <int DMAX, typename MsgT, bool HC>
 __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_threads<DMAX>(), 1)
     k_flood_cluster(const CodeDev *__restrict__ cd, const __grid_constant__ ClusterArgs a)
 {
     constexpr uint32_t kSign = 0x80000000u;
+    constexpr int SR = (int)sizeof(MsgT);
     extern __shared__ __align__(16) unsigned char smem[];
     cg::cluster_group cluster = cg::this_cluster();
     const int q = (int)cluster.block_rank();
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int Z = cd->Z, mb = cd->mb, nb = cd->nb, nnz = cd->nnz;
+    const int Z = cd->Z;
     const float Xb = a.X * kSLog2e, Pb = s_phi_b2(a.X);  // the clamp [phi(X), X] in base-2 units
 
-    // bookkeeping: [0] bad flags (2, alternating by round), [2] the codeword being decoded
-    // (int64 at 8: request << 32 | request-local index, -1 when the work is done)
+    // bookkeeping: [0] bad flags (2, alternating by round; a check of either CTA sets both
+    // CTAs' flag), [2] the codeword being decoded (int64 at 8: request << 32 | request-local
+    // index, -1 when the work is done)
     int32_t *flags = reinterpret_cast<int32_t *>(smem);
     int64_t *cwp = reinterpret_cast<int64_t *>(smem + 8);
-    int32_t *t_rowptr = reinterpret_cast<int32_t *>(smem + 16);  // [mb + 1]
-    int32_t *t_colptr = t_rowptr + MB_MAX + 1;                    // [nb + 1]
-    // check-node descriptor of block b = (row l, column j, shift s): .x = the posterior
-    // index of position s of column j in its owner, .y = Z - s, .z = the owner; check row r
-    // reads .x + r, less Z when r >= .y.  Variable-node descriptor of the i-th entry of the
-    // column lists (block b, shift s): .x = the index of b's message row in its owner, less
-    // s, .y = s, .z = the owner; variable position c reads .x + c, plus Z when c < .y
-    // (message row (c - s) mod Z, which holds the edge of variable c).
-    int4 *t_ed = reinterpret_cast<int4 *>(smem + (((size_t)16 + 4 * (MB_MAX + 1 + NB_MAX + 1) + 15) & ~(size_t)15));
-    int4 *t_cd = t_ed + nnz;
-    const int row0 = a.row_split[q], row1 = a.row_split[q + 1];
-    // block b's owner of posteriors and its base there; column entry's owner of messages
-    for (int i = tid; i <= mb; i += nth) t_rowptr[i] = cd->rowptr[i];
-    for (int i = tid; i <= nb; i += nth) t_colptr[i] = cd->colptr[i];
-    __syncthreads();
-    const int blk0 = t_rowptr[row0], blk1 = t_rowptr[row1];
-    for (int b = tid; b < nnz; b += nth) {
-        const int e = cd->ent[b];
-        const int j = e >> 16, s = e & 0xffff;
-        t_ed[b] = make_int4(4 * (a.col_slot[j] * Z + s), Z - s, a.col_owner[j], 0);
-    }
-    for (int i = tid; i < nnz; i += nth) {
-        const int ce = cd->colent[i];
-        const int b = ce >> 16, s = ce & 0xffff;
-        int l = 0;
-        while (l < mb - 1 && b >= cd->rowptr[l + 1]) l++;
-        const int qo = cl_owner(a.row_split, l);
-        t_cd[i] = make_int4((int)sizeof(MsgT) * ((b - cd->rowptr[a.row_split[qo]]) * Z - s), s, qo, 0);
-    }
-    const size_t off_app = cl_tables_bytes(nnz);
-    float *app = reinterpret_cast<float *>(smem + off_app);
+    // tables: the owned rows' edge descriptors (.x = shared::cluster address of the posterior of
+    // position s of column j, .y = offset of the message of position s, .z = Z - s), the owned
+    // columns' message addresses (position 0; four, or three and in .w the element and number
+    // of the others << 8), then per row its first descriptor << 8 | degree and per column its
+    // place << 8 | number
+    int4 *tab = reinterpret_cast<int4 *>(smem + 16), *ctab = tab + a.n_edge[q];
+    int32_t *rows = reinterpret_cast<int32_t *>(tab + a.n_tab[q]);
+    const int n_rows = a.row_split[q + 1] - a.row_split[q], n_cols = a.ncols[q];
+    int32_t *cols = rows + n_rows;
+    float *app = reinterpret_cast<float *>(smem + a.off_app);
     // R starts at the same offset in every CTA (after the largest posterior share), so that
     // mapping an address into another CTA of the cluster finds that CTA's messages
-    int napp_max = 0;
-#pragma unroll
-    for (int k = 0; k < CLUSTER_CTAS; k++) napp_max = a.ncols[k] * Z > napp_max ? a.ncols[k] * Z : napp_max;
-    MsgT *R = reinterpret_cast<MsgT *>(smem + off_app + (((size_t)napp_max * 4 + 15) & ~(size_t)15));
-    // the cluster's posterior and message arrays, by owning CTA (generic pointers; the own
-    // CTA's are plain shared memory)
-    static_assert(CLUSTER_CTAS == 2, "the owner selects below assume two CTAs");
-    const uint32_t app_0 = cl_map(app, 0), app_1 = cl_map(app, 1);
-    const uint32_t r_0 = cl_map(R, 0), r_1 = cl_map(R, 1);
-    const int n_var = a.ncols[q] * Z;
-    // The check and variable loops without a division per item: thread tid works on position
-    // tid mod Z of block rows / columns tid / Z, tid / Z + RS, ... (RS = nth / Z rows per pass;
-    // threads beyond RS * Z idle there).  When Z exceeds the thread count (RS = 0), thread tid
-    // works on positions tid, tid + nth, ... of every block row / column instead.
-    const int RS = nth / Z;
-    const int p0 = RS > 0 ? tid % Z : tid, ps = RS > 0 ? Z : nth;     // positions
-    const int l0 = RS > 0 ? tid / Z : 0, ls = RS > 0 ? RS : 1;        // block rows / columns
-    const bool works = RS == 0 || tid / Z < RS;
-    const int *my_cols = a.col_list[q];
+    MsgT *R = reinterpret_cast<MsgT *>(smem + a.off_r);
+    const int blk0 = cd->rowptr[a.row_split[q]], blk1 = cd->rowptr[a.row_split[q + 1]];
+    for (int i = tid; i < n_rows; i += nth) {
+        const int l = a.row_list[q][i], b0 = cd->rowptr[l], dc = cd->rowptr[l + 1] - b0, e0 = a.row_e0[q][i];
+        rows[i] = (e0 << 8) | dc;
+        for (int k = 0; k < dc; k++) {
+            const int e = cd->ent[b0 + k], j = e >> 16, s = e & 0xffff;
+            tab[e0 + k] = make_int4((int)(cl_map(app, a.col_owner[j]) + 4 * (a.col_slot[j] * Z + s)),
+                                    a.off_r + SR * ((b0 + k - blk0) * Z + s), Z - s, 0);
+        }
+    }
+    for (int i = tid; i < n_cols; i += nth) {
+        const int j = a.col_list[q][i], i0 = cd->colptr[j], dv = cd->colptr[j + 1] - i0;
+        cols[i] = (a.col_slot[j] << 8) | j;
+        auto addr = [&](int k) -> int {
+            if (k >= dv) return 0;
+            const int b = cd->colent[i0 + k] >> 16;
+            int l = 0;
+            while (l < cd->mb - 1 && b >= cd->rowptr[l + 1]) l++;
+            const int qo = cl_owner(a.row_split, l);
+            return (int)(cl_map(R, qo) + SR * ((b - cd->rowptr[a.row_split[qo]]) * Z));
+        };
+        int x = a.col_x0[q][i];
+        ctab[i] = make_int4(addr(0), addr(1), addr(2), dv > 4 ? (x << 8) | (dv - 3) : addr(3));
+        for (int k = 3; dv > 4 && k < dv; k += 4) tab[x++] = make_int4(addr(k), addr(k + 1), addr(k + 2), addr(k + 3));
+    }
+    const uint32_t flag_0 = cl_map(flags, 0), flag_1 = cl_map(flags, 1);
+    // row groups of WT threads; when a row needs more threads than the CTA has, one group whose
+    // threads take positions ru, ru + nth, ...
+    const int wt = (Z + 31) & ~31, W = wt <= nth ? nth / wt : 1, WT = wt <= nth ? wt : nth;
+    const int w0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT));  // (said to be warp-uniform)
+    const int ru = tid - w0 * WT;
+    const bool works = w0 < W;
     int64_t *cw0 = cluster.map_shared_rank(cwp, 0);
     cluster.sync();  // tables built in every CTA before any remote access
 
@@ -312,20 +271,21 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             }
             cwp[0] = v;
         }
-        cluster.sync();  // also: no CTA still reads another's flags of the previous codeword
+        cluster.sync();
         const int64_t item = *cw0;
         if (item < 0) break;
         const ReqDev &req = a.reqs[(int)(item >> 32)];
         const int64_t cw = item & 0xffffffffll;
         if (tid == 0) flags[0] = flags[1] = 0;
-        // load: APP = L (+0: no -0) for owned variables, R = 0 for owned edges
+        // load: APP = L (+0: no -0) for owned variables, messages 0 for owned edges
         const float *L = static_cast<const float *>(req.llr) + cw * cd->N;
-        for (int i = tid; i < n_var; i += nth) {
-            const int jl = i / Z, c = i - jl * Z;
-            const float v = __ldg(L + my_cols[jl] * Z + c);
-            if (!isfinite(v)) atomicOr(cd->status, IN_NONFINITE);
-            app[i] = v + 0.0f;
-        }
+        for (int r = ru; works && r < Z; r += WT)
+            for (int i = w0; i < n_cols; i += W) {
+                const int jw = cols[i];
+                const float v = __ldg(L + (jw & 255) * Z + r);
+                if (!isfinite(v)) atomicOr(cd->status, IN_NONFINITE);
+                app[(jw >> 8) * Z + r] = v + 0.0f;
+            }
         for (int i = tid; i < (blk1 - blk0) * Z; i += nth) R[i] = MsgT(0.0f);
         cluster.sync();
         int t = 0;
@@ -333,62 +293,61 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
         while (!done) {
             const int tr = t;  // this round's flag is flags[tr & 1]
             // ---------------- check-node phase over the owned checks
-            bool pbad = false;
-            auto check_row = [&](int lr, int r) {
-                const int l = row0 + lr;
-                const int b0 = t_rowptr[l];
-                const uint32_t par = cl_check_dispatch<2, DMAX, MsgT>(t_rowptr[l + 1] - b0, t_ed + b0,
-                                                                      R + (b0 - blk0) * Z + r, app_0, app_1, r, Z,
-                                                                      Xb, Pb);
-                pbad |= (par & kSign) != 0;
-            };
-            for (int r = p0; works && r < Z; r += ps)
-                for (int lr = l0; lr < row1 - row0; lr += ls) check_row(lr, r);
-            if (pbad) flags[tr & 1] = 1;
+            uint32_t bad = 0;
+            if (works)
+                for (int rr = 0; rr < wt; rr += WT) {
+                    Place<1> p;
+                    const int r = rr + ru;
+                    p.own = r < Z;
+                    p.r = p.own ? r : Z - 1;
+                    p.a0 = 4u * (uint32_t)p.r;
+                    p.a1 = p.a0 - 4u * (uint32_t)Z;
+                    p.r0 = (uint32_t)SR * (uint32_t)p.r;
+                    p.r1 = p.r0 - (uint32_t)SR * (uint32_t)Z;
+                    uint32_t pbad[1] = {0};
+                    cl_rows<0, DMAX, MsgT, HC>(a.rend[q], tab, rows, ClusterMem<MsgT>{reinterpret_cast<char *>(smem)},
+                                               p, Xb, Pb, pbad, w0, 2 * (W - w0) - 1, 2 * W);
+                    if (p.own) bad |= pbad[0];
+                }
+            if (__any_sync(0xffffffffu, (bad & kSign) != 0) && (tid & 31) == 0) {
+                cl_st(flag_0 + 4 * (tr & 1), 1);
+                cl_st(flag_1 + 4 * (tr & 1), 1);
+            }
             cluster.sync();
-            // ---------------- decision (the same in every CTA: all flags are read after the barrier)
-            bool any_bad = false;
-#pragma unroll
-            for (int k = 0; k < CLUSTER_CTAS; k++) any_bad |= cluster.map_shared_rank(flags, k)[tr & 1] != 0;
-            const bool conv = tr >= 1 && a.early_exit && !any_bad;
-            if (!conv) {
+            // ---------------- decision (the same in every CTA)
+            const bool conv = tr >= 1 && a.early_exit && flags[tr & 1] == 0;
+            if (!__any_sync(0xffffffffu, conv)) {
                 // ---------------- variable-node phase over the owned variables
-                auto var_col = [&](int jl, int c) {
-                    const int j = my_cols[jl];
-                    const int e0 = t_colptr[j];
-                    const float sum = cl_vn_column<MsgT>(t_colptr[j + 1] - e0, t_cd + e0, r_0, r_1, c, Z,
-                                                         __ldg(L + j * Z + c));
-                    app[jl * Z + c] = sum + 0.0f;  // -0 -> +0: the sign bit is the decision
-                };
-                for (int c = p0; works && c < Z; c += ps)
-                    for (int jl = l0; jl < a.ncols[q]; jl += ls) var_col(jl, c);
+                if (works)
+                    for (int rr = 0; rr < wt; rr += WT) {
+                        const int r = rr + ru, rc = r < Z ? r : Z - 1;
+                        cl_cols<1, MsgT>(a.cend[q], ctab, tab, cols, L + rc, (uint32_t)(SR * rc), app + rc, Z, r < Z,
+                                         w0, W);
+                    }
                 t++;
             }
-            done = conv || t >= a.max_iter;
-            // the other flag was read by every CTA in the previous round (before this round's
-            // first barrier): clear it for the next round, which writes it after the barrier below
+            done = __any_sync(0xffffffffu, conv || t >= a.max_iter);
+            // the other flag was last read before this round's first barrier: clear it for the
+            // next round, which writes it after the barrier below
             if (tid == 0) flags[(tr + 1) & 1] = 0;
             cluster.sync();
         }
         // output: each CTA writes its variables
         uint8_t *Bo = req.bits + cw * cd->N;
         float *Ao = req.app ? req.app + cw * cd->N : nullptr;
-        for (int i = tid; i < n_var; i += nth) {
-            const int jl = i / Z, c = i - jl * Z;
-            const int n = my_cols[jl] * Z + c;
-            const float v = app[i];
-            Bo[n] = v < 0.0f ? 1 : 0;
-            if (Ao) Ao[n] = v;
-        }
+        for (int r = ru; works && r < Z; r += WT)
+            for (int i = w0; i < n_cols; i += W) {
+                const int jw = cols[i], n = (jw & 255) * Z + r;
+                const float v = app[(jw >> 8) * Z + r];
+                Bo[n] = v < 0.0f ? 1 : 0;
+                if (Ao) Ao[n] = v;
+            }
         if (q == 0 && tid == 0) req.iters[cw] = t;
     }
     cluster.sync();  // no CTA leaves while another may still read its shared memory
 }
 
-
 // ------------------------------------------------------------------ host side
-
-// bytes of the table area ahead of APP (the kernel's layout)
 
 // Split the block rows between the cluster's CTAs in contiguous ranges of about equal block
 // counts, then give each block column to the CTA that owns most of its blocks' rows (its
@@ -447,14 +406,42 @@ static size_t cl_plan(const CodeDev &h, int msg, ClusterArgs &a, size_t limit)
         }
     }
     for (int q = 0; q < CLUSTER_CTAS; q++) a.ncols[q] = 0;
-    for (int j = 0; j < h.nb; j++) {
-        const int q = a.col_owner[j];
-        a.col_slot[j] = a.ncols[q];
-        a.col_list[q][a.ncols[q]++] = j;
-    }
+    for (int j = 0; j < h.nb; j++) a.col_slot[j] = a.ncols[a.col_owner[j]]++;
     int nmax = 0;
     for (int q = 0; q < CLUSTER_CTAS; q++) nmax = a.ncols[q] > nmax ? a.ncols[q] : nmax;
-    return cl_tables_bytes(h.nnz) + (((size_t)nmax * h.Z * 4 + 15) & ~(size_t)15) + nr * msz;
+    // the CTAs' lists in ascending degree, and the size of their tables
+    size_t tables = cl_tables_bytes(h.nnz);
+    for (int q = 0; q < CLUSTER_CTAS; q++) {
+        int ne = 0, nr = 0, nc = 0;
+        for (int c = 0; c < CL_CLASSES; c++) {
+            for (int d = (c ? cl_class_degree(c - 1) : 0) + 1; d <= cl_class_degree(c); d++)
+                for (int l = a.row_split[q]; l < a.row_split[q + 1]; l++)
+                    if (h.rowptr[l + 1] - h.rowptr[l] == d) {
+                        a.row_e0[q][nr] = (uint16_t)ne;
+                        a.row_list[q][nr++] = (uint8_t)l;
+                        ne += d;
+                    }
+            a.rend[q][c] = (uint8_t)nr;
+        }
+        int nx = ne + a.ncols[q];
+        for (int c = 1; c <= 5; c++) {
+            for (int d = c; d <= (c < 5 ? c : h.mb); d++)
+                for (int j = 0; j < h.nb; j++)
+                    if (a.col_owner[j] == q && h.colptr[j + 1] - h.colptr[j] == d) {
+                        a.col_x0[q][nc] = (uint16_t)nx;
+                        a.col_list[q][nc++] = (uint8_t)j;
+                        if (d > 4) nx += d / 4;
+                    }
+            a.cend[q][c - 1] = (uint8_t)nc;
+        }
+        a.n_edge[q] = ne;
+        a.n_tab[q] = nx;
+        const size_t need = ((size_t)16 + (size_t)nx * 16 + (size_t)(nr + nc) * 4 + 15) & ~(size_t)15;
+        tables = need > tables ? need : tables;
+    }
+    a.off_app = (int)tables;
+    a.off_r = (int)(tables + (((size_t)nmax * h.Z * 4 + 15) & ~(size_t)15));
+    return (size_t)a.off_r + nr * msz;
 }
 
 static size_t cl_limit()
@@ -476,10 +463,10 @@ int cluster_supported(const CodeDev &h, int msg)
     return need > 0 && need <= cl_limit();
 }
 
-template <int DMAX, typename MsgT>
+template <int DMAX, typename MsgT, bool HC>
 static cudaError_t launch_cluster(const ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d, cudaStream_t s)
 {
-    cudaError_t e = ensure_smem<k_flood_cluster<DMAX, MsgT>>(smem);
+    cudaError_t e = ensure_smem<k_flood_cluster<DMAX, MsgT, HC>>(smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CLUSTER_CTAS, 1, 1);
@@ -494,7 +481,7 @@ static cudaError_t launch_cluster(const ClusterArgs &a, size_t smem, int64_t n_c
     if (dev < 0 || dev >= 64) dev = 0;
     int clusters = __atomic_load_n(&cached[dev], __ATOMIC_RELAXED);
     if (clusters < 1 || __atomic_load_n(&cached_smem[dev], __ATOMIC_RELAXED) != smem) {
-        e = cudaOccupancyMaxActiveClusters(&clusters, k_flood_cluster<DMAX, MsgT>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&clusters, k_flood_cluster<DMAX, MsgT, HC>, &cfg);
         if (e != cudaSuccess || clusters < 1) {
             cudaGetLastError();
             int nsm = 2;
@@ -506,8 +493,17 @@ static cudaError_t launch_cluster(const ClusterArgs &a, size_t smem, int64_t n_c
     }
     if ((int64_t)clusters > n_cw) clusters = (int)n_cw;
     LaunchScope ls(F_SLOTS, s);
-    k_flood_cluster<DMAX, MsgT><<<(unsigned)(clusters * CLUSTER_CTAS), cl_threads<DMAX>(), smem, s>>>(d, a);
+    k_flood_cluster<DMAX, MsgT, HC><<<(unsigned)(clusters * CLUSTER_CTAS), cl_threads<DMAX>(), smem, s>>>(d, a);
     return cudaGetLastError();
+}
+
+template <typename MsgT, bool HC>
+static cudaError_t launch_cluster_d(int dmax, const ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d,
+                                    cudaStream_t s)
+{
+    if (dmax <= 8) return launch_cluster<8, MsgT, HC>(a, smem, n_cw, d, s);
+    if (dmax <= 12) return launch_cluster<12, MsgT, HC>(a, smem, n_cw, d, s);
+    return launch_cluster<32, MsgT, HC>(a, smem, n_cw, d, s);
 }
 
 cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_decode_params &p, const HostReq *reqs,
@@ -538,12 +534,12 @@ cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     a.X = p.phi_clamp;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    const bool f16 = p.msg == LDPC_MSG_F16;
-    if (h.dc_max <= 8)
-        return f16 ? launch_cluster<8, __half>(a, smem, items, d, s) : launch_cluster<8, float>(a, smem, items, d, s);
-    if (h.dc_max <= 16)
-        return f16 ? launch_cluster<16, __half>(a, smem, items, d, s) : launch_cluster<16, float>(a, smem, items, d, s);
-    return f16 ? launch_cluster<32, __half>(a, smem, items, d, s) : launch_cluster<32, float>(a, smem, items, d, s);
+    const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
+    if (p.msg == LDPC_MSG_F16)
+        return hc ? launch_cluster_d<__half, true>(h.dc_max, a, smem, items, d, s)
+                  : launch_cluster_d<__half, false>(h.dc_max, a, smem, items, d, s);
+    return hc ? launch_cluster_d<float, true>(h.dc_max, a, smem, items, d, s)
+              : launch_cluster_d<float, false>(h.dc_max, a, smem, items, d, s);
 }
 
 }  // namespace ldpc

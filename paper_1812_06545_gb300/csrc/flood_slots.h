@@ -73,10 +73,6 @@ struct FloodBook {
 // Named barriers thread slots can have (barrier 0 is the CTA's).
 constexpr int FLOOD_BARRIERS = 15;
 
-// From this X on the upper clamp phi(X) <= |Q| changes nothing in FP32: phi(X) < 2^-50, and
-// e^-phi(X) and e^0 are both 1.
-constexpr float FLOOD_CLAMP_X = 40.0f;
-
 // Threads per CTA of an instance (rows of degree <= 8, or up to 32; message type).
 __host__ __device__ constexpr int flood_threads_max(int dmax, int V, bool f16)
 {

@@ -112,6 +112,10 @@ cudaError_t layered_spa_decode(const CodeDev &host, const CodeDev *dev, const ld
                                int64_t n_cw, uint8_t *bits, int32_t *iters, float *app_out, void *counter,
                                cudaStream_t s);
 
+// From this X on the upper clamp phi(X) <= |Q| changes nothing in FP32: phi(X) < 2^-50, and
+// e^-phi(X) and e^0 are both 1.
+constexpr float FLOOD_CLAMP_X = 40.0f;
+
 // Flooding SPA cluster decoder (flood_cluster.cu): one codeword per two-SM cluster, for codes
 // whose codeword does not fit one CTA; every codeword of n requests of one code in one launch.
 int cluster_supported(const CodeDev &host, int msg);
