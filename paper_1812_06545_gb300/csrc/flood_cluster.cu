@@ -23,15 +23,11 @@
 // block row and position r of every W-th owned column, both in ascending degree, so that a
 // warp runs one straight-line body at a time (flood_check.cuh).  The table entries hold
 // complete shared::cluster addresses (own CTA or the other), so an operand in either CTA costs one add.
-// Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB: 6727 -> 5430 us per launch,
+// Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB: 6727 -> 5378 us per launch,
 // 71 -> 55 warp instructions per edge update (bound by instruction issue, 65 %).
 #include <string.h>
 
-#include <cooperative_groups.h>
-
 #include "flood_check.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace ldpc {
 
@@ -46,6 +42,9 @@ __host__ __device__ constexpr int cl_class_degree(int c)
 // are the items of one work sequence (request i's are items item0 .. item0 + n_cw - 1).
 struct ClusterArgs {
     int n_req;
+    // from here (neither loaded nor divided in the kernel) these are known to be warp-uniform: the
+    // code's sizes, and W row groups of WT threads
+    int Z, N, W, WT;
     int64_t n_items;
     unsigned long long *next;
     int row_split[CLUSTER_CTAS + 1];  // block rows [row_split[q], row_split[q+1]) belong to CTA q
@@ -89,6 +88,13 @@ __device__ __forceinline__ float cl_ld(const __half *, uint32_t addr)
 __device__ __forceinline__ void cl_st(uint32_t addr, int x)
 {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
+}
+
+// The cluster barrier, in its aligned form (all threads of a warp together): the compiler then
+// knows that warps leave it converged, which uniform branches after it need.
+__device__ __forceinline__ void cl_sync()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 __host__ __device__ inline int cl_owner(const int *split, int x)
@@ -200,10 +206,9 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
     constexpr uint32_t kSign = 0x80000000u;
     constexpr int SR = (int)sizeof(MsgT);
     extern __shared__ __align__(16) unsigned char smem[];
-    cg::cluster_group cluster = cg::this_cluster();
-    const int q = (int)cluster.block_rank();
+    const int q = (int)(blockIdx.x % CLUSTER_CTAS);  // the rank in the cluster (one-dimensional grid)
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int Z = cd->Z;
+    const int Z = a.Z, N = a.N;
     const float Xb = a.X * kSLog2e, Pb = s_phi_b2(a.X);  // the clamp [phi(X), X] in base-2 units
 
     // bookkeeping: [0] bad flags (2, alternating by round; a check of either CTA sets both
@@ -252,12 +257,12 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
     const uint32_t flag_0 = cl_map(flags, 0), flag_1 = cl_map(flags, 1);
     // row groups of WT threads; when a row needs more threads than the CTA has, one group whose
     // threads take positions ru, ru + nth, ...
-    const int wt = (Z + 31) & ~31, W = wt <= nth ? nth / wt : 1, WT = wt <= nth ? wt : nth;
-    const int w0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT));  // (said to be warp-uniform)
+    const int wt = (Z + 31) & ~31, W = a.W, WT = a.WT;
+    const int w0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT));  // (a warp reduction: known to be uniform)
     const int ru = tid - w0 * WT;
     const bool works = w0 < W;
-    int64_t *cw0 = cluster.map_shared_rank(cwp, 0);
-    cluster.sync();  // tables built in every CTA before any remote access
+    const uint32_t cw0 = cl_map(cwp, 0);
+    cl_sync();  // tables built in every CTA before any remote access
 
     for (;;) {
         // the leader (CTA 0, thread 0) takes the next codeword; every CTA reads it
@@ -271,14 +276,15 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             }
             cwp[0] = v;
         }
-        cluster.sync();
-        const int64_t item = *cw0;
-        if (item < 0) break;
+        cl_sync();
+        int64_t item;
+        asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(item) : "r"(cw0));
+        if (__any_sync(0xffffffffu, item < 0)) break;  // (a vote: known to be warp-uniform, as the loops below need)
         const ReqDev &req = a.reqs[(int)(item >> 32)];
         const int64_t cw = item & 0xffffffffll;
         if (tid == 0) flags[0] = flags[1] = 0;
         // load: APP = L (+0: no -0) for owned variables, messages 0 for owned edges
-        const float *L = static_cast<const float *>(req.llr) + cw * cd->N;
+        const float *L = static_cast<const float *>(req.llr) + cw * N;
         for (int r = ru; works && r < Z; r += WT)
             for (int i = w0; i < n_cols; i += W) {
                 const int jw = cols[i];
@@ -287,7 +293,7 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
                 app[(jw >> 8) * Z + r] = v + 0.0f;
             }
         for (int i = tid; i < (blk1 - blk0) * Z; i += nth) R[i] = MsgT(0.0f);
-        cluster.sync();
+        cl_sync();
         int t = 0;
         bool done = false;
         while (!done) {
@@ -313,7 +319,7 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
                 cl_st(flag_0 + 4 * (tr & 1), 1);
                 cl_st(flag_1 + 4 * (tr & 1), 1);
             }
-            cluster.sync();
+            cl_sync();
             // ---------------- decision (the same in every CTA)
             const bool conv = tr >= 1 && a.early_exit && flags[tr & 1] == 0;
             if (!__any_sync(0xffffffffu, conv)) {
@@ -330,11 +336,11 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             // the other flag was last read before this round's first barrier: clear it for the
             // next round, which writes it after the barrier below
             if (tid == 0) flags[(tr + 1) & 1] = 0;
-            cluster.sync();
+            cl_sync();
         }
         // output: each CTA writes its variables
-        uint8_t *Bo = req.bits + cw * cd->N;
-        float *Ao = req.app ? req.app + cw * cd->N : nullptr;
+        uint8_t *Bo = req.bits + cw * N;
+        float *Ao = req.app ? req.app + cw * N : nullptr;
         for (int r = ru; works && r < Z; r += WT)
             for (int i = w0; i < n_cols; i += W) {
                 const int jw = cols[i], n = (jw & 255) * Z + r;
@@ -344,7 +350,7 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             }
         if (q == 0 && tid == 0) req.iters[cw] = t;
     }
-    cluster.sync();  // no CTA leaves while another may still read its shared memory
+    cl_sync();  // no CTA leaves while another may still read its shared memory
 }
 
 // ------------------------------------------------------------------ host side
@@ -464,7 +470,7 @@ int cluster_supported(const CodeDev &h, int msg)
 }
 
 template <int DMAX, typename MsgT, bool HC>
-static cudaError_t launch_cluster(const ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d, cudaStream_t s)
+static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d, cudaStream_t s)
 {
     cudaError_t e = ensure_smem<k_flood_cluster<DMAX, MsgT, HC>>(smem);
     if (e != cudaSuccess) return e;
@@ -492,13 +498,16 @@ static cudaError_t launch_cluster(const ClusterArgs &a, size_t smem, int64_t n_c
         __atomic_store_n(&cached[dev], clusters, __ATOMIC_RELAXED);
     }
     if ((int64_t)clusters > n_cw) clusters = (int)n_cw;
+    const int wt = (a.Z + 31) & ~31, nth = cl_threads<DMAX>();
+    a.W = wt <= nth ? nth / wt : 1;
+    a.WT = wt <= nth ? wt : nth;
     LaunchScope ls(F_SLOTS, s);
     k_flood_cluster<DMAX, MsgT, HC><<<(unsigned)(clusters * CLUSTER_CTAS), cl_threads<DMAX>(), smem, s>>>(d, a);
     return cudaGetLastError();
 }
 
 template <typename MsgT, bool HC>
-static cudaError_t launch_cluster_d(int dmax, const ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d,
+static cudaError_t launch_cluster_d(int dmax, ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d,
                                     cudaStream_t s)
 {
     if (dmax <= 8) return launch_cluster<8, MsgT, HC>(a, smem, n_cw, d, s);
@@ -528,6 +537,8 @@ cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     }
     if (items == 0) return cudaSuccess;
     a.n_items = items;
+    a.Z = h.Z;
+    a.N = h.N;
     a.next = static_cast<unsigned long long *>(counter);
     a.max_iter = p.max_iter;
     a.early_exit = p.early_exit;
