@@ -1,18 +1,15 @@
 // Horizontal layered sum-product decoding with the decoder state on chip (Sec. II
 // "Algorithm 2" schedule with the sum-product check rule of Sec. I).
 //
-// A persistent grid of one CTA per SM.  Each CTA holds C codeword slots; a slot keeps its
-// posterior APP [N] (fp32) and its check-to-variable messages R [E] (fp32 or fp16) in
-// shared memory for the whole decode of one codeword.  The slots form barrier groups of K:
-// a group's threads cover its K*Z check rows packed into whole warps, and thread u of a
-// group owns check row u mod Z of slot u / Z, for every block row (layer).  The Z checks of
-// a QC layer touch disjoint variables (each block is one circulant), so the row threads
-// update a layer at once and the group's own barrier (a named barrier, or the warp itself
-// when the group is one warp) separates consecutive layers: the slots of a group run in
-// lock-step, the groups independently, with no CTA-wide barrier.  K trades the idle lanes
-// of a warp-aligned slot (Z not a multiple of 32) against waiting for a group's slowest slot.
-// Messages are stored in check-row order, edge (b, r) at b*Z + r: the layered schedule has
-// no variable-node pass, so the row threads of a warp read and write them contiguously.
+// A persistent grid of one CTA per SM.  Each CTA holds thread slots of V codewords (two, packed in
+// float2 operands, where the messages are FP16, or one); a thread slot keeps its codewords'
+// posteriors APP [N] (fp32) and check-to-variable messages R [E] (fp32 or fp16, stored negated)
+// in shared memory for their whole decode.  Thread r of a thread slot's warps owns check row r
+// of every block row (layer): the Z checks of a QC layer touch disjoint variables (each block
+// is one circulant), so the row threads update a layer at once, and the thread slot's own
+// barrier (a named barrier, or the warp itself) separates consecutive layers; the thread slots
+// of a CTA run independently.  Messages are in check-row order, edge (b, r) at b*Z + r: the
+// layered schedule has no variable-node pass, so a warp reads and writes them contiguously.
 // Per check (the arithmetic of the flooding slot decoder, only the schedule differs):
 //   Q_k   = APP_n - R_k                                   over the check's edges
 //   R'_k  = prod_{other} sgn Q * min(X, phi( sum_{other} phi(clampX |Q|) ))
@@ -20,370 +17,465 @@
 //           messages are half precision
 //   APP_n = Q_k + R'_k   with R'_k the stored value, so that the next Q = APP - R removes
 //                        exactly what was added
-// After every full iteration each slot's hard decisions are checked against all of its
-// checks; a slot that converged (early exit) or reached max_iter writes its outputs and
-// takes the next codeword from the global work counter at its group's next iteration.
+// After every full iteration each slot's hard decisions are checked against its checks, layer
+// by layer until every codeword has shown an unsatisfied one; a codeword that converged (early
+// exit) or reached max_iter is written out and the slot takes the next one from the global
+// work counter.
+//
+// What bounds it (GB300): instruction issue (71-83 %).  8192 codewords of the N = 1944 rate-1/2
+// code, FP32, 2.0 dB: 605 -> 502 us per launch, 45 -> 39 warp instructions per edge update;
+// 7281 codewords of the N = 2304 code, FP16, 5 fixed iterations: 355 -> 298 us.  What went: the
+// syndrome pass over all layers in every iteration (15 % of the instructions; most codewords
+// show an unsatisfied check in the first layer), divergent control, one barrier of two per
+// iteration's end, the upper clamp of |Q| where it cannot bind.
 //
 // APP is never -0: the refill adds +0 to the (scaled) channel value and Q + R' is -0 only when both
 // are -0, which cannot happen while APP is not -0 (then Q = APP - R is not -0).  The sign
 // bit therefore is the hard decision [APP < 0] and sgn(0) = +1, as the oracle reads it.
-#include "slot_common.cuh"
+#include "flood_check.cuh"
 
 namespace ldpc {
-
-#ifndef LDPC_LSPA_REFILL_CHUNK
-#define LDPC_LSPA_REFILL_CHUNK 1  // channel values a thread requests at once when a slot takes a codeword
-#endif
-#ifndef LDPC_LSPA_KMAX
-#define LDPC_LSPA_KMAX 64  // most slots in one barrier group
-#endif
 
 // The FP32-message form keeps APP, Q and R in base-2 units (LLR x log2 e, set at the refill
 // and undone at the output), which spares the check rule its scaling multiplies; the
 // FP16-message form stays in natural units, so that its stored binary16 message is the
 // natural-unit value rounded, as the oracle's binary16 mode rounds it.
 // (Measured on the 8192-codeword N = 1944 rate-1/2 sweep: base-2 units 9.22 info Gbit/s,
-// natural units 8.98; the flooding slot decoder measured the other way round.)
-#ifndef LDPC_LSPA_B2
-#define LDPC_LSPA_B2 1
-#endif
+// natural units 8.98.)
 template <typename MsgT>
-constexpr bool kBase2 = LDPC_LSPA_B2 && sizeof(MsgT) == 4;
+constexpr bool kBase2 = sizeof(MsgT) == 4;
+
+// Bookkeeping of one slot in shared memory.
+struct LspaBook {
+    int64_t cw;      // its next codeword (-1: none)
+    int32_t bad[2];  // unsatisfied check seen, by iteration parity
+};
 
 struct LayeredSpaArgs {
     const float *llr;
     int64_t n_cw;
-    int C, strideA, strideR;  // slots per CTA; per-slot APP and R strides (elements)
-    int K, TPG;               // slots per barrier group; threads per group (whole warps)
-    int max_iter, early_exit;
-    float X;
     uint8_t *bits;
     int32_t *iters;
     float *app_out;
     unsigned long long *next;
+    // sizes and layer lists from here, not from the code's device tables: known to be warp-uniform
+    int N, Z, mb, nb, nnz;
+    int G, TPG;        // thread slots per CTA, threads of one (whole warps)
+    int tab0, slots0;  // tables and first slot, bytes from the start of shared memory
+    int strA, strR, offR;  // bytes from one thread slot's posteriors / messages to the next one's; first messages
+    int max_iter, early_exit;
+    float X;
+    uint8_t deg[MB_MAX];    // degree of each layer
+    uint16_t first[MB_MAX]; // its first block
 };
 
-template <typename MsgT>
-struct MsgIO;
-template <>
-struct MsgIO<float> {
-    // store the message; return the value as stored
-    static __device__ __forceinline__ float st(float *p, float x)
-    {
-        *p = x;
-        return x;
-    }
-    static __device__ __forceinline__ float ld(const float *p) { return *p; }
-};
-template <>
-struct MsgIO<__half> {
-    static __device__ __forceinline__ float st(__half *p, float x)
-    {
-        const __half h = __float2half_rn(x);
-        *p = h;
-        return __half2float(h);
-    }
-    static __device__ __forceinline__ float ld(const __half *p) { return __half2float(*p); }
-};
-
-// Edge descriptor of block b = (row l, column j, shift s) for the layered slots: .x = byte
-// offset of the posterior j*Z + s, .y = byte offset of the message row b*Z, .z = Z - s.
-// Check row r reaches variable position (r + s) mod Z: .x from the thread's posterior base
-// (position r), less one block (ZA bytes) when r >= .z; its message is .y from its message
-// base (row r), with no wrap.
-__device__ __forceinline__ int lspa_app_off(const int4 d, int r, int ZA) { return d.x - (r >= d.z ? ZA : 0); }
-
-// One check of row r (degree <= 8) in the product (tanh) domain: with d_k = e^-a_k,
-// a_k = |Q_k| clamped to [phi(X), X], the pair (alpha, beta) of the other edges' maps
-// (alpha, beta) <- (alpha + d beta, beta + d alpha) from (1, 0) gives
-// R'_k = ln(alpha / beta) = phi(sum_{other} phi(a)) (slot_common.cuh); one ex2 and two lg2
-// per edge.  The FP32 form holds Q per edge; the FP16 form (1024 threads, 64 registers)
-// forms it again from APP and R, neither of which is written before its own edge is.
-template <int D, bool EXACT, typename MsgT>
-__device__ __forceinline__ void layer_check_tanh(int dc, const int4 *__restrict__ ed, char *Ar, char *Rr, int r, int ZA,
-                                                 float Xb, float Pb)
+// Edge descriptor of block b = (row l, column j, shift s): .x = byte offset of the posterior
+// j*Z + s, .y of the message row b*Z, .z = Z - s.  Check row r reaches variable position
+// (r + s) mod Z: .x from the thread's posterior base (position r), less one block when r >= .z;
+// its message is .y from its message base (row r), with no wrap.
+template <int V>
+__device__ __forceinline__ void lspa_at(const int4 &e, const Place<V> &p, uint32_t &ao, uint32_t &ro)
 {
+    ao = (p.r >= e.z ? p.a1 : p.a0) + (uint32_t)e.x;
+    ro = p.r0 + (uint32_t)e.y;
+}
+
+// Store the negated message n of an edge and the posterior Q - n, with n as stored.
+template <typename MsgT>
+__device__ __forceinline__ void lspa_put(char *sm, bool own, uint32_t ao, uint32_t ro, float q, float n)
+{
+    if constexpr (sizeof(MsgT) == 2) {
+        const __half h = __float2half_rn(n);
+        if (own) *reinterpret_cast<__half *>(sm + ro) = h;
+        n = __half2float(h);
+    } else {
+        if (own) *reinterpret_cast<float *>(sm + ro) = n;
+    }
+    if (own) *reinterpret_cast<float *>(sm + ao) = q - n;
+}
+template <typename MsgT>
+__device__ __forceinline__ void lspa_put(char *sm, bool own, uint32_t ao, uint32_t ro, float2 q, float2 n)
+{
+    if constexpr (sizeof(MsgT) == 2) {
+        const __half2 h = __floats2half2_rn(n.x, n.y);
+        if (own) *reinterpret_cast<__half2 *>(sm + ro) = h;
+        n = __half22float2(h);
+    } else {
+        if (own) *reinterpret_cast<float2 *>(sm + ro) = n;
+    }
+    const float2 a = __ffma2_rn(n, make_float2(-1.0f, -1.0f), q);
+    if (own) *reinterpret_cast<float2 *>(sm + ao) = a;
+}
+
+// One check of degree D <= 8: every edge's state in registers.
+template <int D, int V, typename MsgT, bool HC>
+__device__ __forceinline__ void layer_narrow(const int4 *__restrict__ ed, char *sm, const Place<V> &p, float Xb, float Pb)
+{
+    constexpr bool B2 = kBase2<MsgT>;
     constexpr uint32_t kSign = 0x80000000u;
-    constexpr bool B2 = kBase2<MsgT>, kHoldQ = sizeof(MsgT) == 4;
-    MsgT *Rl = at<MsgT>(Rr, ed[0].y);
-    const int Zm = ZA / (int)sizeof(float);
-    float d[D];
-    int ao[D];
-    float q[kHoldQ ? D : 1];
-    uint32_t sg = 0;
+    using T = VT<V>;
+    const T one = vset(T(), 1.0f), zero = vset(T(), 0.0f);
+    T d[D], q[D];
+    uint32_t ao[D], sg[V];
+#pragma unroll
+    for (int v = 0; v < V; v++) sg[v] = 0;
 #pragma unroll
     for (int k = 0; k < D; k++) {
-        d[k] = 0.0f;  // a missing edge (k >= dc) is the identity map
-        ao[k] = 0;
-        if (EXACT || k < dc) {
-            ao[k] = lspa_app_off(ed[k], r, ZA);
-            const float qk = *at<float>(Ar, ao[k]) - MsgIO<MsgT>::ld(Rl + k * Zm);
-            if constexpr (kHoldQ) q[k] = qk;
-            sg ^= __float_as_uint(qk);
-            d[k] = tanh_d<B2>(qk, Xb, Pb);
-        }
+        uint32_t ro;
+        lspa_at<V>(ed[k], p, ao[k], ro);
+        q[k] = vadd(Sm<float, V>::ld(sm + ao[k]), Sm<MsgT, V>::ld(sm + ro));
+        each(q[k], [&](float x, int v) { sg[v] ^= __float_as_uint(x); });
+        d[k] = form_d<B2, HC>(q[k], Xb, Pb);
     }
-    float sa[D + 1], sb[D + 1];
-    sa[D] = 1.0f;
-    sb[D] = 0.0f;
-    sa[D - 1] = 1.0f;
+    T sa[D + 1], sb[D + 1];
+    sa[D - 1] = one;
     sb[D - 1] = d[D - 1];
 #pragma unroll
     for (int k = D - 2; k >= 1; k--) {
-        sa[k] = fmaf(d[k], sb[k + 1], sa[k + 1]);
-        sb[k] = fmaf(d[k], sa[k + 1], sb[k + 1]);
+        sa[k] = vfma(d[k], sb[k + 1], sa[k + 1]);
+        sb[k] = vfma(d[k], sa[k + 1], sb[k + 1]);
     }
-    float pa = 1.0f, pb = 0.0f;
+    T pa = one, pb = zero;
 #pragma unroll
     for (int k = 0; k < D; k++) {
-        float al, be;
+        T al, be;
         if (k == 0) {
             al = sa[1];
             be = sb[1];
         } else if (k == D - 1) {
             al = pa;
             be = pb;
+        } else if (k == D - 2) {  // the suffix is one edge's map (1, d): one rounding less
+            al = vfma(pb, sb[D - 1], pa);
+            be = vfma(pa, sb[D - 1], pb);
         } else {
-            tanh_combine(pa, pb, sa[k + 1], sb[k + 1], al, be);
+            al = vfma(pb, sb[k + 1], vmul(pa, sa[k + 1]));
+            be = vfma(pb, sa[k + 1], vmul(pa, sb[k + 1]));
         }
-        if (EXACT || k < dc) {
-            const float mag = tanh_mag<B2>(al, be);
-            float qk;
-            if constexpr (kHoldQ)
-                qk = q[k];
-            else
-                qk = *at<float>(Ar, ao[k]) - MsgIO<MsgT>::ld(Rl + k * Zm);
-            const float out = __uint_as_float(__float_as_uint(mag) | ((__float_as_uint(qk) ^ sg) & kSign));
-            *at<float>(Ar, ao[k]) = qk + MsgIO<MsgT>::st(Rl + k * Zm, out);
-        }
+        T n = neg_mag<B2>(al, be);
+        T qk = q[k];
+        each(qk, [&](float x, int v) {
+            float &y = reinterpret_cast<float *>(&n)[v];
+            y = __uint_as_float(__float_as_uint(y) & ~((__float_as_uint(x) ^ sg[v]) & kSign));
+        });
+        lspa_put<MsgT>(sm, p.own, ao[k], p.r0 + (uint32_t)ed[k].y, q[k], n);
         if (k == 0) {
             pb = d[0];
         } else if (k < D - 1) {
-            const float t = fmaf(d[k], pb, pa);
-            pb = fmaf(d[k], pa, pb);
+            const T t = vfma(d[k], pb, pa);
+            pb = vfma(d[k], pa, pb);
             pa = t;
         }
     }
 }
 
-// One check of row r in the layer whose blocks start at descriptor `ed`, computed from and
-// written back to the slot's APP (thread base Ar) and R (thread base Rr): rows up to degree 8
-// hold their state per edge, wider rows take the grouped form (see slot_common.cuh), with Q
-// formed from APP and R in both passes (neither is written before its own edge is) and
-// APP = Q + R' at the store.
-template <int D, bool EXACT, typename MsgT>
-__device__ __forceinline__ void layer_check(int dc, const int4 *__restrict__ ed, char *Ar, char *Rr, int r, int ZA,
-                                            float Xb, float Pb)
+// One check of degree 9..32 in groups of 8 edges (see flood_check.cuh): pass 1 forms each
+// group's pair, pass 2 each group's messages; Q is formed from APP and N in both (neither is
+// written before its own edge is).
+template <int G, int V, typename MsgT, bool HC>
+__device__ __forceinline__ void layer_wide(int dc, const int4 *__restrict__ ed, char *sm, const Place<V> &p, float Xb,
+                                           float Pb)
 {
-    if constexpr (D <= 8) {
-        layer_check_tanh<D, EXACT, MsgT>(dc, ed, Ar, Rr, r, ZA, Xb, Pb);
-    } else {
-        MsgT *Rl = at<MsgT>(Rr, ed[0].y);
-        const int Zm = ZA / (int)sizeof(float);
-        auto qof = [&](int k, bool) -> float {
-            return *at<float>(Ar, lspa_app_off(ed[k], r, ZA)) - MsgIO<MsgT>::ld(Rl + k * Zm);
-        };
-        auto put = [&](int k, float m, float q) {
-            *at<float>(Ar, lspa_app_off(ed[k], r, ZA)) = q + MsgIO<MsgT>::st(Rl + k * Zm, m);
-        };
-        tanh_check_wide<D, kBase2<MsgT>>(dc, Xb, Pb, qof, put);
-    }
-}
-
-template <int D, int DMAX, typename MsgT>
-__device__ __forceinline__ void layer_check_dispatch(int dc, const int4 *__restrict__ ed, char *Ar, char *Rr, int r,
-                                                     int ZA, float Xb, float Pb)
-{
-    if constexpr (D >= DMAX) {
-        layer_check<DMAX, false, MsgT>(dc, ed, Ar, Rr, r, ZA, Xb, Pb);
-    } else if constexpr (D <= 8) {
-        if (dc == D)
-            layer_check<D, true, MsgT>(dc, ed, Ar, Rr, r, ZA, Xb, Pb);
-        else
-            layer_check_dispatch<next_degree(D), DMAX, MsgT>(dc, ed, Ar, Rr, r, ZA, Xb, Pb);
-    } else {
-        if (dc <= D)
-            layer_check<D, false, MsgT>(dc, ed, Ar, Rr, r, ZA, Xb, Pb);
-        else
-            layer_check_dispatch<next_degree(D), DMAX, MsgT>(dc, ed, Ar, Rr, r, ZA, Xb, Pb);
-    }
-}
-
-// XOR of the posterior sign bits of check row r of one block row (degree dc): straight-line
-// bodies for the common degrees (every lane of a warp takes the same branch).
-template <int D>
-__device__ __forceinline__ uint32_t lspa_parity(const int4 *__restrict__ ed, const char *Ar, int r, int ZA)
-{
-    uint32_t par = 0;
+    constexpr bool B2 = kBase2<MsgT>;
+    using T = VT<V>;
+    const T one = vset(T(), 1.0f), zero = vset(T(), 0.0f);
+    T ga[G], gb[G];
+    uint32_t sg[V];
 #pragma unroll
-    for (int k = 0; k < D; k++) par ^= __float_as_uint(*at<float>(Ar, lspa_app_off(ed[k], r, ZA)));
-    return par;
+    for (int v = 0; v < V; v++) sg[v] = 0;
+#pragma unroll
+    for (int g = 0; g < G; g++) {
+        ga[g] = one;
+        gb[g] = zero;
+    }
+    auto q_of = [&](int k, uint32_t &ao, uint32_t &ro) -> T {
+        lspa_at<V>(ed[k], p, ao, ro);
+        return vadd(Sm<float, V>::ld(sm + ao), Sm<MsgT, V>::ld(sm + ro));
+    };
+    auto pass1 = [&](int k0, auto full) {
+        constexpr bool FULL = decltype(full)::value;
+        T a = one, b = zero;
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            if (!FULL && k0 + i >= dc) break;
+            uint32_t ao, ro;
+            T q = q_of(k0 + i, ao, ro);
+            each(q, [&](float x, int v) { sg[v] = __funnelshift_l(__float_as_uint(x), sg[v], 1); });
+            const T d = form_d<B2, HC>(q, Xb, Pb);
+            if (i == 0) {
+                b = d;
+            } else {
+                const T t = vfma(d, b, a);
+                b = vfma(d, a, b);
+                a = t;
+            }
+        }
+#pragma unroll
+        for (int g = 0; g < G; g++)
+            if (k0 == 8 * g) {
+                ga[g] = a;
+                gb[g] = b;
+            }
+    };
+    auto pass2 = [&](int k0, auto full) {
+        constexpr bool FULL = decltype(full)::value;
+        T pa = one, pb = zero;  // the other groups' product (its first factor is taken exactly)
+#pragma unroll
+        for (int h = 0; h < G; h++) {
+            if (k0 == 8 * h || 8 * h >= dc) continue;
+            const T a1 = pa, b1 = pb;
+            pa = vfma(b1, gb[h], vmul(a1, ga[h]));
+            pb = vfma(b1, ga[h], vmul(a1, gb[h]));
+        }
+        T d[8], q[8];
+        uint32_t ao[8], ro[8];
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            d[i] = q[i] = zero;
+            ao[i] = ro[i] = 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; i++) {
+            if (!FULL && k0 + i >= dc) break;
+            q[i] = q_of(k0 + i, ao[i], ro[i]);
+            d[i] = form_d<B2, HC>(q[i], Xb, Pb);
+        }
+        group_out<FULL, B2, V>(dc - k0, d, pa, pb, sg,
+                               [&](int i, T n) { lspa_put<MsgT>(sm, p.own, ao[i], ro[i], q[i], n); });
+#pragma unroll
+        for (int v = 0; v < V; v++) sg[v] <<= 8;
+    };
+#pragma unroll
+    for (int g = 0; g < G - 1; g++) pass1(8 * g, Const<true>());
+    pass1(8 * (G - 1), Const<false>());
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        sg[v] ^= 0u - (__popc(sg[v]) & 1u);  // the product of the other edges' signs
+        sg[v] <<= 32 - dc;
+    }
+#pragma unroll
+    for (int g = 0; g < G - 1; g++) pass2(8 * g, Const<true>());
+    pass2(8 * (G - 1), Const<false>());
 }
-__device__ __forceinline__ uint32_t lspa_row_parity(int dc, const int4 *__restrict__ ed, const char *Ar, int r,
-                                                    int ZA)
+
+// One layer (the degree is warp-uniform).
+template <int DMAX, int V, typename MsgT, bool HC>
+__device__ __forceinline__ void layer_check(int dc, const int4 *__restrict__ ed, char *sm, const Place<V> &p, float Xb,
+                                            float Pb)
 {
     switch (dc) {
-    case 4: return lspa_parity<4>(ed, Ar, r, ZA);
-    case 5: return lspa_parity<5>(ed, Ar, r, ZA);
-    case 6: return lspa_parity<6>(ed, Ar, r, ZA);
-    case 7: return lspa_parity<7>(ed, Ar, r, ZA);
-    case 8: return lspa_parity<8>(ed, Ar, r, ZA);
-    default: {
-        uint32_t par = 0;
-        for (int k = 0; k < dc; k++) par ^= __float_as_uint(*at<float>(Ar, lspa_app_off(ed[k], r, ZA)));
-        return par;
+    case 2: layer_narrow<2, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    case 3: layer_narrow<3, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    case 4: layer_narrow<4, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    case 5: layer_narrow<5, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    case 6: layer_narrow<6, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    case 7: layer_narrow<7, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    case 8: layer_narrow<8, V, MsgT, HC>(ed, sm, p, Xb, Pb); break;
+    default:
+        if constexpr (DMAX > 8) {
+            if (dc <= 16)
+                layer_wide<2, V, MsgT, HC>(dc, ed, sm, p, Xb, Pb);
+            else if (dc <= 24)
+                layer_wide<3, V, MsgT, HC>(dc, ed, sm, p, Xb, Pb);
+            else
+                layer_wide<4, V, MsgT, HC>(dc, ed, sm, p, Xb, Pb);
+        }
     }
+}
+
+// XOR of the posterior sign bits of the thread's check row of one layer, per codeword.
+template <int V>
+__device__ __forceinline__ void lspa_parity(int dc, const int4 *__restrict__ ed, const char *sm, const Place<V> &p,
+                                            uint32_t (&par)[V])
+{
+#pragma unroll
+    for (int v = 0; v < V; v++) par[v] = 0;
+    auto take = [&](int k) {
+        uint32_t ao, ro;
+        lspa_at<V>(ed[k], p, ao, ro);
+        VT<V> a = Sm<float, V>::ld(sm + ao);
+        each(a, [&](float x, int v) { par[v] ^= __float_as_uint(x); });
+    };
+    int k = 0;
+    for (; k + 4 <= dc; k += 4) {
+        take(k);
+        take(k + 1);
+        take(k + 2);
+        take(k + 3);
     }
+    for (; k < dc; k++) take(k);
 }
 
-// Table space (ints) ahead of the slots: four per block for its edge descriptor, then the
-// block-row pointers.
-__host__ __device__ inline int lspa_tables_ints(int nnz, int mb) { return 4 * nnz + mb + 1; }
-
-// Threads per CTA for an instance: high-degree checks keep more values live per thread.
-// fp32 slots are limited to a few per CTA by shared memory, so their threads get more
-// registers (672 = 7 slots of three warps at 96 registers); fp16 slots are twice as many
-// and run the register-lean check form.
-template <int DMAX, typename MsgT>
-constexpr int lspa_threads_max()
+// Threads per CTA for an instance.
+__host__ __device__ constexpr int lspa_threads(int dmax, int V, bool f16)
 {
-    return sizeof(MsgT) == 4 ? (DMAX <= 16 ? 672 : 512) : (DMAX <= 8 ? 1024 : (DMAX <= 16 ? 768 : 512));
+    if (V == 2) return 640;
+    return f16 ? (dmax <= 8 ? 1024 : 768) : 672;
 }
 
-// The barrier of one slot group: its warps only (named barrier group + 1; barrier 0 is the
-// CTA's), or nothing beyond the warp itself when the group is one warp.
-__device__ __forceinline__ void group_sync(int grp, int tpg)
+template <int DMAX, int V, typename MsgT, bool HC>
+__global__ void __launch_bounds__(lspa_threads(DMAX, V, sizeof(MsgT) == 2), 1)
+    k_layered_spa(const CodeDev *__restrict__ cd, const __grid_constant__ LayeredSpaArgs a)
 {
-    if (tpg == 32)
-        __syncwarp();
-    else
-        asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(tpg) : "memory");
-}
-
-template <int DMAX, typename MsgT>
-__global__ void __launch_bounds__(lspa_threads_max<DMAX, MsgT>(), 1) k_layered_spa(const CodeDev *__restrict__ cd,
-                                                                                    const LayeredSpaArgs a)
-{
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int N = cd->N, Z = cd->Z, mb = cd->mb, nb = cd->nb, nnz = cd->nnz;
-    const int C = a.C, K = a.K, TPG = a.TPG;
-    int32_t *bad = reinterpret_cast<int32_t *>(smem);                 // [SLOTS_MAX] unsatisfied check seen
-    int32_t *gany = bad + SLOTS_MAX;                                   // [SLOTS_MAX / 2][2] group vote
-    int64_t *fresh = reinterpret_cast<int64_t *>(gany + SLOTS_MAX);    // [SLOTS_MAX] the slot's codeword
-    int4 *t_ed = reinterpret_cast<int4 *>(fresh + SLOTS_MAX);         // edge descriptor per block
-    int32_t *t_rowptr = reinterpret_cast<int32_t *>(t_ed + nnz);
-    float *APPs = reinterpret_cast<float *>(smem + slots_smem_head(lspa_tables_ints(nnz, mb)));
-    MsgT *Rs = reinterpret_cast<MsgT *>(APPs + (size_t)C * a.strideA);
-
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    char *sm = reinterpret_cast<char *>(smem_raw);
+    LspaBook *books = reinterpret_cast<LspaBook *>(sm);
+    int4 *tab = reinterpret_cast<int4 *>(sm + a.tab0);
+    constexpr int SA = (int)sizeof(float) * V, SR = (int)sizeof(MsgT) * V;
+    constexpr uint32_t kSign = 0x80000000u;
+    const int N = a.N, Z = a.Z, mb = a.mb, nb = a.nb, nnz = a.nnz, TPG = a.TPG;
     const int tid = threadIdx.x, nth = blockDim.x;
     const float Xb = a.X * kSLog2e, Pb = s_phi_b2(a.X);  // the clamp [phi(X), X] in base-2 units
     for (int i = tid; i < nnz; i += nth) {
         const int e = cd->ent[i], sh = e & 0xffff;
-        t_ed[i] = make_int4((int)sizeof(float) * ((e >> 16) * Z + sh), (int)sizeof(MsgT) * i * Z, Z - sh, 0);
+        tab[i] = make_int4(SA * ((e >> 16) * Z + sh), SR * i * Z, Z - sh, 0);
     }
-    const int ZA = (int)sizeof(float) * Z;
-    for (int i = tid; i <= mb; i += nth) t_rowptr[i] = cd->rowptr[i];
-    const int g = tid / TPG, u = tid - (tid / TPG) * TPG;
-    const int c = g * K + u / Z, r = u - (u / Z) * Z;
-    const bool mine = u < K * Z && c < C;  // a row of a slot (else an idle lane of the group)
-    if (tid == 0)
-        for (int i = 0; i < SLOTS_MAX; i++) gany[i] = 0;
-    if (mine && r == 0) {
+    // thread slot g (a warp reduction: known to be warp-uniform), row ru of its layers
+    const int g = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / TPG)), ru = tid - g * TPG;
+    const bool own = ru < Z, lead = ru == 0;  // (idle lanes of the last warp repeat row Z - 1 and store nothing)
+    LspaBook *book = books + g * V;
+    auto grab = [&](int v) {
         const unsigned long long k = atomicAdd(a.next, 1ull);
-        fresh[c] = k < (unsigned long long)a.n_cw ? (int64_t)k : -1;
-        bad[c] = 0;
+        book[v].cw = k < (unsigned long long)a.n_cw ? (int64_t)k : -1;
+    };
+    if (lead) {
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            grab(v);
+            book[v].bad[0] = book[v].bad[1] = 0;
+        }
     }
     __syncthreads();
-    if (g * K >= C) return;  // whole warps beyond the last group
-    float *A = APPs + (size_t)(mine ? c : 0) * a.strideA;
-    MsgT *Rc = Rs + (size_t)(mine ? c : 0) * a.strideR;
-    char *Ar = reinterpret_cast<char *>(A + r), *Rr = reinterpret_cast<char *>(Rc + r);
-    int ph = 0;
-    // OR of a predicate over the group (every thread of the group calls it at the same
-    // point; the vote alternates between two words so that clearing the next one races with
-    // nothing)
-    auto group_any = [&](bool pred) {
-        if (pred) gany[2 * g + ph] = 1;
-        group_sync(g, TPG);
-        const bool any = gany[2 * g + ph] != 0;
-        if (u == 0) gany[2 * g + (ph ^ 1)] = 0;
-        ph ^= 1;
-        return any;
+    Place<V> p;
+    p.own = own;
+    p.r = own ? ru : Z - 1;
+    p.a0 = (uint32_t)(a.slots0 + g * a.strA + p.r * SA);
+    p.a1 = p.a0 - (uint32_t)(Z * SA);
+    p.r0 = (uint32_t)(a.slots0 + a.offR + g * a.strR + p.r * SR);
+    p.r1 = p.r0;
+    const int r = p.r;
+    float *A = reinterpret_cast<float *>(sm + p.a0);
+    MsgT *R = reinterpret_cast<MsgT *>(sm + p.r0);
+    auto gsync = [&]() {
+        if (TPG == 32)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(TPG) : "memory");
     };
 
-    // a slot given codeword k loads APP = L (+0: no -0 in APP) and clears its messages; the
-    // channel values of a chunk are all requested before any is used
-    auto refill = [&](int64_t k) {
-        const float *L = a.llr + k * N;
-        constexpr int CH = LDPC_LSPA_REFILL_CHUNK;
+    // lane v takes codeword k: APP = L (+0: no -0 in APP), messages 0; the channel values of a chunk
+    // are all requested before any is used
+    auto refill = [&](int v, int64_t k) {
+        const float *L = a.llr + k * N + r;
+        constexpr int CH = 4;
         for (int j0 = 0; j0 < nb; j0 += CH) {
-            float v[CH];
+            float x[CH];
 #pragma unroll
             for (int w = 0; w < CH; w++)
-                if (j0 + w < nb) v[w] = __ldg(L + (j0 + w) * Z + r);
+                if (j0 + w < nb) x[w] = __ldg(L + (j0 + w) * Z);
 #pragma unroll
             for (int w = 0; w < CH; w++)
                 if (j0 + w < nb) {
-                    if (!isfinite(v[w])) atomicOr(cd->status, IN_NONFINITE);
-                    A[(j0 + w) * Z + r] = kBase2<MsgT> ? fmaf(v[w], kSLog2e, 0.0f) : v[w] + 0.0f;
+                    if (!isfinite(x[w])) atomicOr(cd->status, IN_NONFINITE);
+                    A[(j0 + w) * Z * V + v] = kBase2<MsgT> ? fmaf(x[w], kSLog2e, 0.0f) : x[w] + 0.0f;
                 }
         }
-        for (int b = 0; b < nnz; b++) Rc[b * Z + r] = MsgT(0.0f);
+        for (int b = 0; b < nnz; b++) R[b * Z * V + v] = MsgT(0.0f);
     };
 
-    int64_t cw = mine ? fresh[c] : -1;
-    int t = 0;
-    if (cw >= 0) refill(cw);
-    if (!group_any(cw >= 0)) return;
+    int64_t cw[V];
+    int t[V];
+    bool any = false;
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        cw[v] = book[v].cw;
+        t[v] = 0;
+        if (cw[v] >= 0 && own) refill(v, cw[v]);
+        any |= cw[v] >= 0;
+    }
+    any = __any_sync(0xffffffffu, any);  // (votes: conditions known to be warp-uniform)
+    gsync();
 
-    for (;;) {
-        const bool busy = cw >= 0;
+    for (int ph = 0; any; ph ^= 1) {
+#pragma unroll 1
         for (int l = 0; l < mb; l++) {
-            if (busy) {
-                const int b0 = t_rowptr[l];
-                layer_check_dispatch<2, DMAX, MsgT>(t_rowptr[l + 1] - b0, t_ed + b0, Ar, Rr, r, ZA, Xb, Pb);
-            }
-            group_sync(g, TPG);
+            layer_check<DMAX, V, MsgT, HC>(a.deg[l], tab + a.first[l], sm, p, Xb, Pb);
+            gsync();
         }
-        if (busy) t++;
-        // syndrome of the hard decisions (APP sign bits): row r of every layer
-        if (busy && a.early_exit) {
-            uint32_t par_any = 0;
+        bool busy[V], done[V];
+        bool anydone = false;
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            busy[v] = cw[v] >= 0;
+            t[v] += busy[v];
+        }
+        if (a.early_exit) {
+            // syndrome of the hard decisions (APP sign bits), until each codeword of the slot has
+            // shown this warp an unsatisfied check
+            bool seen[V];
+#pragma unroll
+            for (int v = 0; v < V; v++) seen[v] = !busy[v];
+#pragma unroll 1
             for (int l = 0; l < mb; l++) {
-                const int b0 = t_rowptr[l];
-                par_any |= lspa_row_parity(t_rowptr[l + 1] - b0, t_ed + b0, Ar, r, ZA);
-            }
-            if (par_any & 0x80000000u) bad[c] = 1;
-        }
-        group_sync(g, TPG);
-        bool done = false;
-        if (busy) {
-            done = (a.early_exit && bad[c] == 0) || t >= a.max_iter;
-            if (done) {
-                uint8_t *Bo = a.bits + cw * N;
-                float *Ao = a.app_out ? a.app_out + cw * N : nullptr;
-                for (int j = 0; j < nb; j++) {
-                    const float v = A[j * Z + r];
-                    Bo[j * Z + r] = v < 0.0f ? 1 : 0;
-                    if (Ao) Ao[j * Z + r] = kBase2<MsgT> ? v * kSLn2 : v;
+                uint32_t par[V];
+                lspa_parity<V>(a.deg[l], tab + a.first[l], sm, p, par);
+                bool rest = false;
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    const bool u = __any_sync(0xffffffffu, (par[v] & kSign) != 0);
+                    if (busy[v] && u) seen[v] = true;
+                    rest |= !seen[v];
                 }
-                if (r == 0) {
-                    a.iters[cw] = t;
-                    const unsigned long long k = atomicAdd(a.next, 1ull);
-                    fresh[c] = k < (unsigned long long)a.n_cw ? (int64_t)k : -1;
+                if (!__any_sync(0xffffffffu, rest)) break;
+            }
+            if ((tid & 31) == 0) {
+#pragma unroll
+                for (int v = 0; v < V; v++)
+                    if (seen[v]) book[v].bad[ph] = 1;
+            }
+            gsync();
+        }
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            done[v] = busy[v] && ((a.early_exit && book[v].bad[ph] == 0) || t[v] >= a.max_iter);
+            anydone |= done[v];
+        }
+        if (a.early_exit && lead) {
+            // the other flag was last read in the iteration before
+#pragma unroll
+            for (int v = 0; v < V; v++) book[v].bad[ph ^ 1] = 0;
+        }
+        if (__any_sync(0xffffffffu, anydone)) {
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                if (done[v] && own) {
+                    uint8_t *Bo = a.bits + cw[v] * N + r;
+                    float *Ao = a.app_out ? a.app_out + cw[v] * N + r : nullptr;
+                    for (int j = 0; j < nb; j++) {
+                        const float x = A[j * Z * V + v];
+                        Bo[j * Z] = x < 0.0f ? 1 : 0;
+                        if (Ao) Ao[j * Z] = kBase2<MsgT> ? x * kSLn2 : x;
+                    }
+                    if (lead) {
+                        a.iters[cw[v]] = t[v];
+                        grab(v);
+                    }
                 }
             }
-        }
-        group_sync(g, TPG);
-        if (busy) {
-            if (r == 0) bad[c] = 0;
-            if (done) {
-                cw = fresh[c];
-                t = 0;
-                if (cw >= 0) refill(cw);
+            gsync();
+            any = false;
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                if (done[v]) {
+                    cw[v] = book[v].cw;
+                    t[v] = 0;
+                    if (cw[v] >= 0 && own) refill(v, cw[v]);
+                }
+                any |= cw[v] >= 0;
             }
+            any = __any_sync(0xffffffffu, any);
+            gsync();
         }
-        if (!group_any(cw >= 0)) break;
     }
 }
 
@@ -393,105 +485,121 @@ static size_t lspa_slot_bytes(const CodeDev &h, int msg)
            (size_t)((h.E + 7) & ~7) * (msg == LDPC_MSG_F16 ? sizeof(__half) : sizeof(float));
 }
 
-static int lspa_threads_for(int dc_max, int msg)
-{
-    const int d = dc_max <= 8 ? 8 : dc_max <= 16 ? 16 : dc_max <= 24 ? 24 : 32;
-    if (msg == LDPC_MSG_F16)
-        return d == 8 ? lspa_threads_max<8, __half>() : d == 16 ? lspa_threads_max<16, __half>()
-                                                               : lspa_threads_max<32, __half>();
-    return d <= 16 ? lspa_threads_max<16, float>() : lspa_threads_max<32, float>();
-}
-
 static size_t lspa_smem(const CodeDev &h, int msg, int C)
 {
-    return slots_smem_head(lspa_tables_ints(h.nnz, h.mb)) + (size_t)C * lspa_slot_bytes(h, msg);
+    return slots_smem_head(4 * h.nnz + h.mb + 1) + (size_t)C * lspa_slot_bytes(h, msg);
 }
 
-// Slots per CTA and their grouping: the most slots that fit the instance's threads, 15 named
-// barriers and shared memory, with the fewest slots per group among the arrangements that
-// reach that count.
-struct LspaShape {
-    int C, K, TPG;
-};
-static LspaShape lspa_shape(const CodeDev &h, int msg, int64_t cap = SLOTS_MAX)
+static size_t lspa_limit()
 {
-    LspaShape best = {0, 1, 32};
-    if (h.dc_max > 32 || h.N >= 65536) return best;
     int dev = 0, lim = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&lim, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const size_t limit = lim > 0 ? (size_t)lim : 227 * 1024;
-    int cmax = SLOTS_MAX;
-    while (cmax > 0 && lspa_smem(h, msg, cmax) > limit) cmax--;
-    if (cap >= 1 && cap < cmax) cmax = (int)cap;  // a small batch spreads over the SMs
-    const int tmax = lspa_threads_for(h.dc_max, msg);
-    for (int K = 1; K <= cmax && K <= LDPC_LSPA_KMAX; K++) {
-        const int tpg = ((K * h.Z + 31) / 32) * 32;
-        int G = tmax / tpg;
-        if (tpg > 32 && G > 15) G = 15;
-        int C = G * K;
-        if (C > cmax) C = cmax;
-        if (C > best.C) best = {C, K, tpg};
-    }
-    return best;
+    return lim > 0 ? (size_t)lim : 227 * 1024;
 }
 
-int layered_spa_slots_per_cta(const CodeDev &h, int msg) { return lspa_shape(h, msg).C; }
-
-template <int DMAX, typename MsgT>
-static cudaError_t launch_lspa(const CodeDev &h, const CodeDev *d, const LayeredSpaArgs &a, int msg, cudaStream_t s)
+// Whether the decoder serves a code: one slot in shared memory (beside tables of the size it
+// once needed, so that the line stays where it is) and its rows in a CTA's threads.
+int layered_spa_slots_per_cta(const CodeDev &h, int msg)
 {
-    const size_t sm = lspa_smem(h, msg, a.C);
-    cudaError_t e = ensure_smem<k_layered_spa<DMAX, MsgT>>(sm);
+    if (h.dc_max > 32 || h.N >= 65536) return 0;
+    const int tmax = msg == LDPC_MSG_F16 ? (h.dc_max <= 8 ? 1024 : h.dc_max <= 16 ? 768 : 512)
+                                         : (h.dc_max <= 16 ? 672 : 512);
+    return ((h.Z + 31) / 32) * 32 <= tmax && lspa_smem(h, msg, 1) <= lspa_limit() ? 1 : 0;
+}
+
+// Strides congruent to Z modulo the 32 banks, so that rows of neighbouring slots do not collide.
+static int lspa_stride(int n, int Z) { return n + ((Z % 32) - (n % 32) + 32) % 32; }
+
+// Thread slots of V codewords per CTA, at most cap.
+static int lspa_fit(const CodeDev &h, int msg, int V, int cap)
+{
+    const int wt = ((h.Z + 31) / 32) * 32, dmax = h.dc_max <= 8 ? 8 : 32;
+    int G = lspa_threads(dmax, V, msg == LDPC_MSG_F16) / wt;
+    if (G > cap) G = cap;
+    if (G * V > SLOTS_MAX) G = SLOTS_MAX / V;
+    if (wt > 32 && G > 15) G = 15;  // named barriers
+    const size_t slot = (size_t)V * (4 * (size_t)lspa_stride(h.N, h.Z) +
+                                     (msg == LDPC_MSG_F16 ? 2 : 4) * (size_t)lspa_stride(h.E, h.Z));
+    while (G > 0 && (size_t)G * V * sizeof(LspaBook) + (size_t)h.nnz * 16 + 64 + G * slot > lspa_limit()) G--;
+    return G;
+}
+
+template <int DMAX, int V, typename MsgT, bool HC>
+static cudaError_t launch_lspa(const CodeDev *d, const LayeredSpaArgs &a, size_t smem, int64_t ctas, cudaStream_t s)
+{
+    cudaError_t e = ensure_smem<k_layered_spa<DMAX, V, MsgT, HC>>(smem);
     if (e != cudaSuccess) return e;
-    int dev = 0, nsm = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int64_t ctas = nsm;
-    const int64_t need = (a.n_cw + a.C - 1) / a.C;
-    if (need < ctas) ctas = need;
     LaunchScope ls(F_LAYERED_SPA, s);
-    const int groups = (a.C + a.K - 1) / a.K;
-    k_layered_spa<DMAX, MsgT><<<(unsigned)ctas, groups * a.TPG, sm, s>>>(d, a);
+    k_layered_spa<DMAX, V, MsgT, HC><<<(unsigned)ctas, a.G * a.TPG, smem, s>>>(d, a);
     return cudaGetLastError();
 }
 
-template <typename MsgT>
-static cudaError_t launch_lspa_d(const CodeDev &h, const CodeDev *d, const LayeredSpaArgs &a, int msg, cudaStream_t s)
+template <typename MsgT, bool HC>
+static cudaError_t launch_lspa_d(const CodeDev &h, const CodeDev *d, const LayeredSpaArgs &a, size_t smem,
+                                 int64_t ctas, cudaStream_t s)
 {
-    if (h.dc_max <= 8) return launch_lspa<8, MsgT>(h, d, a, msg, s);
-    if (h.dc_max <= 16) return launch_lspa<16, MsgT>(h, d, a, msg, s);
-    if (h.dc_max <= 24) return launch_lspa<24, MsgT>(h, d, a, msg, s);
-    return launch_lspa<32, MsgT>(h, d, a, msg, s);
+    return h.dc_max <= 8 ? launch_lspa<8, 1, MsgT, HC>(d, a, smem, ctas, s)
+                         : launch_lspa<32, 1, MsgT, HC>(d, a, smem, ctas, s);
 }
 
 cudaError_t layered_spa_decode(const CodeDev &h, const CodeDev *d, const ldpc_decode_params &p, const float *llr,
                                int64_t n_cw, uint8_t *bits, int32_t *iters, float *app_out, void *counter,
                                cudaStream_t s)
 {
-    LayeredSpaArgs a;
-    a.llr = llr;
-    a.n_cw = n_cw;
+    const bool f16 = p.msg == LDPC_MSG_F16;
     int dev = 0, nsm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const LspaShape sh = lspa_shape(h, p.msg, (n_cw + nsm - 1) / nsm);
-    a.C = sh.C;
-    if (a.C < 1) return cudaErrorInvalidValue;
-    a.K = sh.K;
-    a.TPG = sh.TPG;
-    a.strideA = (h.N + 3) & ~3;
-    a.strideR = (h.E + 7) & ~7;
-    a.max_iter = p.max_iter;
-    a.early_exit = p.early_exit;
-    a.X = p.phi_clamp;
+    const int64_t per_sm = (n_cw + nsm - 1) / nsm;  // a small batch spreads over the SMs
+    const int cap1 = (int)(per_sm < SLOTS_MAX ? per_sm : SLOTS_MAX), cap2 = (cap1 + 1) / 2;
+    const int g1 = lspa_fit(h, p.msg, 1, cap1), g2 = lspa_fit(h, p.msg, 2, cap2);
+    // two codewords per thread where that holds more codewords per CTA than the threads allow one
+    // to a thread: FP16 messages, rows of degree <= 8.  (8192 codewords on GB300, one against two:
+    // N = 1944 rate 1/2 FP16 507 / 467 us, 10 slots against 6 pairs; FP32 486 / 597, 7 against 3;
+    // rate 5/6 FP16 489 / 545: there single slots of more warps win.)
+    const int V = f16 && h.dc_max <= 8 && per_sm > g1 && 2 * g2 > g1 ? 2 : 1;
+    LayeredSpaArgs a;
+    a.llr = llr;
+    a.n_cw = n_cw;
     a.bits = bits;
     a.iters = iters;
     a.app_out = app_out;
     a.next = static_cast<unsigned long long *>(counter);
+    a.N = h.N;
+    a.Z = h.Z;
+    a.mb = h.mb;
+    a.nb = h.nb;
+    a.nnz = h.nnz;
+    a.G = V == 2 ? g2 : g1;
+    if (a.G < 1) return cudaErrorInvalidValue;
+    a.TPG = ((h.Z + 31) / 32) * 32;
+    const int SA = 4 * V, SR = (f16 ? 2 : 4) * V;
+    a.tab0 = (a.G * V * (int)sizeof(LspaBook) + 15) & ~15;
+    a.slots0 = a.tab0 + 16 * h.nnz;
+    a.strA = SA * lspa_stride(h.N, h.Z);
+    a.strR = SR * lspa_stride(h.E, h.Z);
+    a.offR = (a.G * a.strA + 15) & ~15;
+    const size_t smem = (size_t)a.slots0 + a.offR + (size_t)a.G * a.strR;
+    a.max_iter = p.max_iter;
+    a.early_exit = p.early_exit;
+    a.X = p.phi_clamp;
+    for (int l = 0; l < h.mb; l++) {
+        a.first[l] = (uint16_t)h.rowptr[l];
+        a.deg[l] = (uint8_t)(h.rowptr[l + 1] - h.rowptr[l]);
+    }
+    const int64_t need = (n_cw + a.G * V - 1) / (a.G * V), ctas = need < nsm ? need : nsm;
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
-    return p.msg == LDPC_MSG_F16 ? launch_lspa_d<__half>(h, d, a, p.msg, s) : launch_lspa_d<float>(h, d, a, p.msg, s);
+    const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
+    if (V == 2)
+        return hc ? launch_lspa<8, 2, __half, true>(d, a, smem, ctas, s)
+                  : launch_lspa<8, 2, __half, false>(d, a, smem, ctas, s);
+    if (f16)
+        return hc ? launch_lspa_d<__half, true>(h, d, a, smem, ctas, s)
+                  : launch_lspa_d<__half, false>(h, d, a, smem, ctas, s);
+    return hc ? launch_lspa_d<float, true>(h, d, a, smem, ctas, s)
+              : launch_lspa_d<float, false>(h, d, a, smem, ctas, s);
 }
 
 }  // namespace ldpc

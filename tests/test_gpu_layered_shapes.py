@@ -1,0 +1,41 @@
+"""Layered sum-product decoder at the edges of its forms: every check-row degree class, slots of Z
+around the warp size, one codeword per thread and (FP16 messages, rows up to degree 8, large
+batches) two."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from paper_1812_06545_gb300 import ldpc
+from tests.gpu_helpers import FP32_TOL, assert_binary16_close, binary16_band, rel_err
+from tests.test_gpu_flood_shapes import CODES, base_of, decode
+
+pytestmark = pytest.mark.gpu
+
+# (two codewords per thread need more codewords per SM than single slots fit: Z = 81, N = 1944)
+ALL = dict(CODES, z81=(base_of([4, 4, 5, 5, 6, 6, 7, 7, 8, 8, 8, 3], 24, 81, 6), 81))
+
+
+@pytest.mark.parametrize("form", ["layered_f32", "layered_f16"])
+@pytest.mark.parametrize("name", list(ALL))
+def test_against_oracle_and_across_forms(cuda_dev, name, form):
+    B, Z = ALL[name]
+    code, oc = ldpc.Code(B, Z), O.QCCode(B, Z)
+    n_small, n_big = 40, 152 * 24 + 5
+    rng = np.random.default_rng(8)
+    L = (2.5 + 2.2 * rng.standard_normal((n_big, code.N))).astype(np.float32)  # noisy all-zero codewords
+    L[::7, ::5] = 0.0
+    for T in (1, 2):
+        app, bits, iters = decode(code, form, L[:n_small].copy(), cuda_dev, max_iter=T, early_exit=0)
+        if form == "layered_f32":
+            ref, _, _ = oc.spa_layered(L[:n_small], T, early_exit=False)
+            assert rel_err(app, ref).max() <= FP32_TOL, (name, T)
+        elif T == 1:
+            ref, band = binary16_band(oc, True, L[:400], 1, 8)
+            app, _, _ = decode(code, form, L[:400].copy(), cuda_dev, max_iter=T, early_exit=0)
+            assert_binary16_close(app, ref, band, strict=False, what=name)
+        assert np.array_equal(bits, (app[:n_small] < 0)) and (iters == T).all()
+    # each codeword's arithmetic is its own: the same, bit for bit, in a large batch with refills
+    small = decode(code, form, L[:n_small].copy(), cuda_dev, max_iter=9)
+    big = decode(code, form, L, cuda_dev, max_iter=9)
+    for a, b in zip(small, big):
+        assert np.array_equal(a, b[:n_small]), name
