@@ -7,8 +7,8 @@
 // fused multiply-add) act on two such values at once and round only when the exact result
 // is not representable.  So a thread carries the same check row of two codewords in the two
 // halves of each 32-bit register and runs every step of the check once for both:
-//   Q_k   = sat(APP_n - R_k, msg_sat)                      add, add, min, max
-//   min1, min2 over |Q_k| (duplicates counted)             and, 3 x min/max per edge
+//   Q_k   = sat(APP_n - R_k, msg_sat)                      sub, min, max
+//   min1, min2 over |Q_k| (duplicates counted)             3 x min/max per edge
 //   S     = XOR of the sign bits of Q_k                    xor of the whole words
 //   mag_k = alpha * (|Q_k| == min1 ? min2 : min1)          compare mask, select
 //   R_k   = mag_k with sign S xor sign(Q_k)                xor of the sign bits
@@ -19,17 +19,30 @@
 // 2^-(alpha_shift + 1): the fractions of alpha m are multiples of 2^-alpha_shift, so alpha m -
 // delta lies strictly within 1/2 of floor(alpha m), and adding 1536 (binary16 spacing 1 in
 // [1024, 2048)) rounds it there; the host admits only parameters for which alpha m - delta is
-// itself exact (layered_pairs_exact).  Zero is never negative: APP starts at +0 (the
-// quantiser's -0 becomes +0), and a sum of two opposite values that cancel is +0, so the sign
-// bit of APP is the hard decision and that of Q is [Q < 0].
+// itself exact (layered_pairs_exact).
 //
-// Storage (shared memory, one CTA per SM, persistent, the slot and barrier-group arrangement
-// of k_layered_slots with a thread slot holding two codewords): APP as half2 [slot][N], and R
-// as two bytes per edge, each R + 128; R is widened to binary16 by placing the byte under the
-// exponent of 1024 (1024 + R + 128, one byte permute) and narrowed again by adding 1152 and
-// taking the low byte of each half.  Messages are in check-row order, edge (b, r) at b*Z + r.
-// Each lane of a thread slot holds its own codeword: it converges, writes its outputs and is
-// refilled from the work counter independently of the other lane.
+// Storage (shared memory, one CTA per SM, persistent): APP and R as one byte per codeword, each
+// the value + 128, the two codewords of a variable or edge in one 16-bit word.  A byte placed under the
+// exponent of 1024 (one byte permute for two) is the binary16 number 1024 + 128 + value: the
+// biases of APP and R cancel in APP - R, and Q + (R + 1152) is the new APP in the same form, so
+// one permute of the low bytes stores both values.  Bit 7 of a byte is set when the value is >= 0:
+// the hard decision, and XORing the words of a check gives both codewords' parities at once.
+// Messages are in check-row order, edge (b, r) at b*Z + r.  Messages are not cleared when a lane
+// takes a codeword: its bytes read as 128 through a mask in its first iteration.
+//
+// Thread r of a thread slot's warps owns check row r of every layer; the thread slot's own
+// barrier separates layers; each lane (codeword) of a thread slot converges, writes its outputs
+// and is refilled from the work counter independently.  After each iteration the syndrome is
+// taken layer by layer until every lane has shown the warp an unsatisfied check.
+//
+// What bounds it (GB300): instruction issue (74 %).  65536 codewords of the N = 1944 rate-5/6
+// code, 4.0 dB: 1858 -> 1429 us per launch, 66 -> 51 warp instructions per edge of two codewords;
+// 4193 codewords of the N = 4000 code, 10 iterations: 421 -> 325 us.  What went: APP as half2
+// (bytes now, whose bias cancels in APP - R), the degree test at every edge (blocks of four, and
+// exact bodies up to degree 8), divergent control around stores and layers, the descriptor, select and
+// add per operand (the offset table: 1667 -> 1429 us), clearing the messages of a new codeword.
+// Four codewords per thread (32-bit words) took 41 instructions per edge of two, but left 15
+// warps instead of 24: 1644 us.
 #include <cuda_fp16.h>
 #include <string.h>
 
@@ -38,20 +51,15 @@
 
 namespace ldpc {
 
-#ifndef LDPC_PAIRS_KMAX
-#define LDPC_PAIRS_KMAX 1  // most thread slots in one barrier group (one: every slot runs on its own)
-#endif
-#ifndef LDPC_PAIRS_REFILL_NOINLINE
-#define LDPC_PAIRS_REFILL_NOINLINE 0  // 1: refill / output as out-of-line functions
-#endif
-#if LDPC_PAIRS_REFILL_NOINLINE
-#define LDPC_PAIRS_COLD __device__ __noinline__
-#else
-#define LDPC_PAIRS_COLD __device__ __forceinline__
-#endif
-#ifndef LDPC_PAIRS_REFILL_CHUNK
-#define LDPC_PAIRS_REFILL_CHUNK 4  // channel values a thread requests at once when a lane takes a codeword
-#endif
+constexpr int kPairRefillChunk = 4;  // channel values a thread requests at once when a lane takes a codeword
+
+// Bookkeeping of one lane (codeword) of a thread slot in shared memory.
+struct PairBook {
+    int64_t cw;      // its next codeword (request-local, -1: none)
+    int32_t req;     // and the request
+    int32_t cur;     // the request of the codeword it decodes
+    int32_t bad[2];  // unsatisfied check seen, by iteration parity
+};
 
 // One launch decodes every codeword of up to MULTI_MAX_REQS requests of one code: the
 // codewords are the items of one work sequence (request i's codewords are items item0 ..
@@ -61,13 +69,18 @@ struct LayeredPairArgs {
     float scale;
     int n_req;
     int64_t n_items;
-    int C2, K, TPG;        // thread slots (two codewords each), thread slots per group, threads per group
-    int strideA, strideR;  // APP stride (half2 elements) and R stride (byte pairs) per thread slot
+    // sizes and layer lists from here, not from the code's device tables: known to be warp-uniform
+    int N, Z, mb, nb, nnz;
+    int G, TPG;            // thread slots per CTA, threads of one (whole warps)
+    int tab0, slots0;      // tables and first slot, bytes from the start of shared memory
+    int strA, strR, offR;  // bytes from one thread slot's posteriors / messages to the next one's; first messages
     int max_iter, early_exit, msg_sat, app_sat;
-    // binary16 pairs: +-msg_sat, +-app_sat, alpha = alpha_num / 2^alpha_shift and -delta =
+    // binary16 pairs: +-msg_sat, +-app_sat + 1152, alpha = alpha_num / 2^alpha_shift and -delta =
     // 2^-(alpha_shift + 1) - 1/2, in both halves
     uint32_t sat, nsat, appmax, appmin, alpha, ndelta;
     unsigned long long *next;
+    uint8_t deg[MB_MAX];    // degree of each layer
+    uint16_t first[MB_MAX]; // its first block
     ReqDev reqs[MULTI_MAX_REQS];
 };
 
@@ -79,143 +92,172 @@ constexpr uint32_t kH1536 = 0x66006600u;    // 1536
 constexpr uint32_t kHm1536 = 0xE600E600u;   // -1536
 constexpr uint32_t kHInf = 0x7C007C00u;     // +infinity
 constexpr uint32_t kSign2 = 0x80008000u;
-constexpr uint32_t kMag2 = 0x7FFF7FFFu;
+constexpr uint32_t kZero2 = 0x8080u;        // the value 0 in both bytes
 
-// R of both codewords of an edge: two biased bytes -> 1024 + (R + 128) in each half
-__device__ __forceinline__ __half2 widen_r(uint32_t two_bytes) { return u2h(__byte_perm(two_bytes, 0x64646464u, 0x5140)); }
-// R (binary16 pair) -> the two biased bytes (low byte of R + 1152 in each half)
-__device__ __forceinline__ uint32_t narrow_r(__half2 r) { return __byte_perm(h2u(__hadd2(r, u2h(kH1152))), 0u, 0x0020); }
+// the two bytes of a word -> 1024 + byte in each half; and back: the low bytes of the halves
+__device__ __forceinline__ __half2 widen(uint32_t w) { return u2h(__byte_perm(w, 0x64646464u, 0x5140)); }
+__device__ __forceinline__ uint16_t narrow(__half2 x) { return (uint16_t)__byte_perm(h2u(x), 0u, 0x0020); }
 
-// The APP byte offset of edge k of a layer for row r of a thread slot, in one of two forms:
-// from the offset table (one 16-bit load: the table holds the offset of every (block, row)), or
-// from the layer's edge descriptors (an 8-byte load shared by all rows: .x = offset of block
-// column position s, .y = Z - s; row r reaches position r + s, less Z when r >= Z - s).
-template <bool TABLE>
-struct EdgeAddr;
-template <>
-struct EdgeAddr<true> {
-    const uint16_t *orow;  // row r's entry of the layer's first block; edge k is Z entries further
-    int Z;
-    __device__ __forceinline__ int operator()(int k) const { return orow[k * Z]; }
-};
-template <>
-struct EdgeAddr<false> {
-    const int2 *ed;  // the layer's first block's descriptor
-    int rA, r, ZA;   // byte offset of position r, the row, and 4 Z
-    __device__ __forceinline__ int operator()(int k) const
-    {
-        const int2 d = ed[k];
-        return rA + d.x - (r >= d.y ? ZA : 0);
+// Shared-memory stores under a predicate: an `if` around them compiles to a divergent region of its
+// own (three control instructions per edge).
+__device__ __forceinline__ void store_if(bool on, uint32_t addr, uint16_t x)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.s32 p, %2, 0;\n\t@p st.shared.u16 [%0], %1;\n\t}" ::"r"(addr), "h"(x),
+                 "r"((int)on)
+                 : "memory");
+}
+// Edges of a check: EXACT, all D; else edges 4b .. 4b + 3 as one straight-line block and the last
+// dc mod 4 one by one: few (warp-uniform) tests of the degree, and a block's loads overlap.
+// f(k, slot): edge k, whose state lives in register slot `slot` (a constant).
+template <int D, bool EXACT, typename F>
+__device__ __forceinline__ void for_edges(int dc, F f)
+{
+    if constexpr (EXACT) {
+#pragma unroll
+        for (int k = 0; k < D; k++) f(k, k);
+    } else {
+        const int nb4 = dc >> 2;
+#pragma unroll
+        for (int b = 0; b < D / 4; b++) {
+            if (b >= nb4) break;
+#pragma unroll
+            for (int i = 0; i < 4; i++) f(4 * b + i, 4 * b + i);
+        }
+        const int k0 = nb4 << 2, rem = dc & 3;
+        if (rem > 0) f(k0, D);
+        if (rem > 1) f(k0 + 1, D + 1);
+        if (rem > 2) f(k0 + 2, D + 2);
     }
+}
+
+// The posterior offsets of a layer's edges for the thread's row, in one of two forms.  TABLE: a
+// 16-bit entry per (block, row), shared by all thread slots: one load, whose address and
+// result take warp-uniform offsets (k blocks further; the slot).  Else from the edge descriptors
+// (.x = offset of position s, .y = Z - s): row r reaches position r + s, less Z when r >= Z - s.
+template <bool TABLE>
+struct PairAt;
+template <>
+struct PairAt<true> {
+    const char *sm;
+    uint32_t t0;    // the thread's entry of the layer's first block (bytes)
+    uint32_t tz;    // bytes of a block's entries
+    uint32_t slot;  // the slot's posteriors
+    __device__ __forceinline__ uint32_t operator()(int k) const
+    {
+        return slot + *reinterpret_cast<const uint16_t *>(sm + (t0 + (uint32_t)k * tz));
+    }
+    __device__ __forceinline__ void again() { asm volatile("" : "+r"(t0)); }
+};
+template <>
+struct PairAt<false> {
+    const char *sm;
+    uint32_t eo;      // the layer's first descriptor
+    uint32_t a0, a1;  // the thread's posterior of block column 0, plain and less one block
+    int r;
+    __device__ __forceinline__ uint32_t operator()(int k) const
+    {
+        const int2 e = *reinterpret_cast<const int2 *>(sm + (eo + 8u * (uint32_t)k));
+        return (r >= e.y ? a1 : a0) + (uint32_t)e.x;
+    }
+    __device__ __forceinline__ void again() { asm volatile("" : "+r"(eo), "+r"(a0), "+r"(a1)); }
 };
 
-#ifndef LDPC_PAIRS_FENCE
-#define LDPC_PAIRS_FENCE 0  // edges between compiler fences in the unrolled edge loops (0: none)
-#endif
-// A compiler-only fence every LDPC_PAIRS_FENCE edges: loads are not hoisted across it, which
-// bounds how many edges' values the unrolled loops keep live at once.
-__device__ __forceinline__ void edge_fence(int k)
-{
-    if constexpr (LDPC_PAIRS_FENCE > 0)
-        if (k % LDPC_PAIRS_FENCE == LDPC_PAIRS_FENCE - 1) asm volatile("" ::: "memory");
-}
-
-#ifndef LDPC_PAIRS_BREAK
-#define LDPC_PAIRS_BREAK 1  // leave the unrolled edge loops every this many edges once past dc (0: never)
-#endif
-// Whether an unrolled edge loop is past the row's degree at edge k: every LDPC_PAIRS_BREAK
-// edges a warp-uniform test (every row of a layer has the same degree) leaves the loop, so
-// the edges of a wide body past dc cost no predicated instructions.  Measured on 65536
-// codewords of the N = 1944 rate-5/6 code (rows of degree 18-21 in the degree-24 body): a
-// test at every edge 2.15 -> 1.87 ms per decode, every 4 edges 1.92, every 8 edges 2.09,
-// bit-identical; it also frees the registers of the skipped edges (80 -> 71, no spill).
-__device__ __forceinline__ bool edges_done(int k, int dc)
-{
-    if constexpr (LDPC_PAIRS_BREAK > 0) return k > 0 && k % LDPC_PAIRS_BREAK == 0 && k >= dc;
-    return false;
-}
-
-// One check row of a layer for the two codewords of a thread slot (edges past dc skipped under
-// a uniform guard).  ea: the edges' APP offsets, Ab: APP base of the slot, Rrow: the byte pairs
-// of the layer's first edge of row r (edge k is Z pairs further).  The second pass forms each
-// APP offset again rather than holding it.
-template <int D, bool SATAPP, bool TABLE>
-__device__ __forceinline__ void pair_check(int dc, const EdgeAddr<TABLE> &ea, char *Ab, uint16_t *Rrow, int Z,
+// One check row of a layer for the two codewords of a thread slot.  at: the edges' posteriors; rr:
+// offset of the first edge's message; zb: bytes of a block of messages; keep: mask of the lanes
+// whose messages are valid; own: whether the thread stores.
+template <int D, bool SATAPP, bool EXACT, typename AT>
+__device__ __forceinline__ void pair_check(int dc, AT at, char *sm, bool own, uint32_t rr, uint32_t zb, uint32_t keep,
                                            const LayeredPairArgs &k_)
 {
-    uint32_t q[D];
+    uint32_t q[EXACT ? D : D + 3];
     __half2 mn1 = u2h(kHInf), mn2 = u2h(kHInf);
     uint32_t S = 0;
-#pragma unroll
-    for (int k = 0; k < D; k++) {
-        if (edges_done(k, dc)) break;
-        if (k < dc) {
-            const __half2 app = *reinterpret_cast<const __half2 *>(Ab + ea(k));
-            const __half2 rb = widen_r(Rrow[k * Z]);
-            __half2 qq = __hadd2(__hsub2(app, rb), u2h(kH1152));
-            qq = __hmax2(__hmin2(qq, u2h(k_.sat)), u2h(k_.nsat));
-            const uint32_t qb = h2u(qq);
-            const __half2 mag = u2h(qb & kMag2);
-            mn2 = __hmin2(mn2, __hmax2(mn1, mag));
-            mn1 = __hmin2(mn1, mag);
-            S ^= qb;
-            q[k] = qb;
-        }
-        edge_fence(k);
-    }
-    // alpha * min as floor(alpha m): round(alpha m - delta) at binary16 spacing 1 (+-1536)
+    for_edges<D, EXACT>(dc, [&](int k, int slot) {
+        const uint32_t aw = *reinterpret_cast<const uint16_t *>(sm + at(k));
+        uint32_t rw = *reinterpret_cast<const uint16_t *>(sm + (rr + (uint32_t)k * zb));
+        rw = (rw & keep) | (kZero2 & ~keep);
+        __half2 qq = __hsub2(widen(aw), widen(rw));
+        qq = __hmax2(__hmin2(qq, u2h(k_.sat)), u2h(k_.nsat));
+        const __half2 mag = __habs2(qq);
+        mn2 = __hmin2(mn2, __hmax2(mn1, mag));
+        mn1 = __hmin2(mn1, mag);
+        S ^= h2u(qq);
+        q[slot] = h2u(qq);
+    });
+    // alpha * min1, min2 as floor(alpha m), carrying the sign of the whole check
     const __half2 m1 = __hadd2(__hadd2(__hfma2(mn1, u2h(k_.alpha), u2h(k_.ndelta)), u2h(kH1536)), u2h(kHm1536));
     const __half2 m2 = __hadd2(__hadd2(__hfma2(mn2, u2h(k_.alpha), u2h(k_.ndelta)), u2h(kH1536)), u2h(kHm1536));
     const uint32_t Sm = S & kSign2;
-    const uint32_t A1 = h2u(m1) ^ Sm, A2 = h2u(m2) ^ Sm;  // magnitudes carrying the sign of the whole check
-#pragma unroll
-    for (int k = 0; k < D; k++) {
-        if (edges_done(k, dc)) break;
-        if (k < dc) {
-            const uint32_t qb = q[k];
-            const uint32_t eq = __heq2_mask(u2h(qb & kMag2), mn1);
-            const uint32_t rn = ((eq & A2) | (~eq & A1)) ^ (qb & kSign2);
-            __half2 an = __hadd2(u2h(qb), u2h(rn));
-            if constexpr (SATAPP) an = __hmax2(__hmin2(an, u2h(k_.appmax)), u2h(k_.appmin));
-            Rrow[k * Z] = (uint16_t)narrow_r(u2h(rn));
-            *reinterpret_cast<__half2 *>(Ab + ea(k)) = an;
-        }
-        edge_fence(k);
+    const uint32_t A1 = h2u(m1) ^ Sm, A2 = h2u(m2) ^ Sm;
+    // (the second pass forms the offsets again: held across the passes they spill)
+    if constexpr (!EXACT) {
+        at.again();
+        asm volatile("" : "+r"(rr));
+    }
+    const uint32_t sb = (uint32_t)__cvta_generic_to_shared(sm);
+    for_edges<D, EXACT>(dc, [&](int k, int slot) {
+        const uint32_t qb = q[slot];
+        const uint32_t eq = __heq2_mask(__habs2(u2h(qb)), mn1);
+        const uint32_t m = ((eq & A2) | (~eq & A1)) ^ (qb & kSign2);
+        const __half2 t = __hadd2(u2h(m), u2h(kH1152));  // R + 1152 (and -0 becomes 1152)
+        __half2 a = __hadd2(u2h(qb), t);
+        if constexpr (SATAPP) a = __hmax2(__hmin2(a, u2h(k_.appmax)), u2h(k_.appmin));
+        store_if(own, sb + (rr + (uint32_t)k * zb), narrow(t));
+        store_if(own, sb + at(k), narrow(a));
+    });
+}
+
+// One layer (the degree is warp-uniform): exact bodies up to degree 8.
+template <int D, int DMAX, bool SATAPP, typename AT>
+__device__ __forceinline__ void pair_layer(int dc, const AT &at, char *sm, bool own, uint32_t rr, uint32_t zb,
+                                           uint32_t keep, const LayeredPairArgs &k_)
+{
+    if constexpr (D <= 8) {
+        if (dc == D)
+            pair_check<D, SATAPP, true>(dc, at, sm, own, rr, zb, keep, k_);
+        else
+            pair_layer<D + 1, DMAX, SATAPP>(dc, at, sm, own, rr, zb, keep, k_);
+    } else if constexpr (DMAX > 8) {
+        pair_check<DMAX, SATAPP, false>(dc, at, sm, own, rr, zb, keep, k_);
     }
 }
 
-// Parity word (XOR of the APP words: sign bits 15 and 31 are the two codewords') of check row r
-// of one block row, edges past dc skipped under a uniform guard.
-template <int D, bool TABLE>
-__device__ __forceinline__ uint32_t pair_parity(int dc, const EdgeAddr<TABLE> &ea, const char *Ab)
+// XOR of the posterior words of check row r of one layer: bit 7 of each byte is the parity of the
+// codeword's decisions [APP >= 0].
+template <typename AT>
+__device__ __forceinline__ uint32_t pair_parity(int dc, const AT &at, const char *sm)
 {
-    uint32_t par = 0;
-#pragma unroll
-    for (int k = 0; k < D; k++) {
-        if (edges_done(k, dc)) break;
-        if (k < dc) par ^= *reinterpret_cast<const uint32_t *>(Ab + ea(k));
-        edge_fence(k);
+    auto word = [&](uint32_t o) -> uint32_t { return *reinterpret_cast<const uint16_t *>(sm + o); };
+    uint32_t par = (dc & 1) ? kZero2 : 0u;  // of [APP < 0] then
+    int k = 0;
+#pragma unroll 1
+    for (; k + 4 <= dc; k += 4) {
+        const uint32_t x0 = at(k), x1 = at(k + 1), x2 = at(k + 2), x3 = at(k + 3);
+        par ^= word(x0) ^ word(x1);
+        par ^= word(x2) ^ word(x3);
     }
+#pragma unroll 1
+    for (; k < dc; k++) par ^= word(at(k));
     return par;
 }
 
 __device__ __forceinline__ int sat_q(int x, int s) { return max(-s, min(s, x)); }
 
-// Load codeword k of request rq into lane v of a thread slot, this thread's row r: APP =
-// quantised LLRs (+0 for zero) at positions j*Z + r, R = 0 (biased byte 128) for every block;
-// the channel values of a chunk are all requested before any is used.
-LDPC_PAIRS_COLD void lpair_refill(const LayeredPairArgs &a, const CodeDev *__restrict__ cd, __half *Ah,
-                                          uint16_t *Rc, int v, int rq, int k, int r, int N, int Z, int nb, int nnz)
+// Load codeword k of request rq into a lane (A: its byte of position r of block column 0; two bytes
+// to a variable): APP = quantised LLRs; the channel values of a chunk are all requested before any is used.
+__device__ __forceinline__ void lpair_refill(const LayeredPairArgs &a, const CodeDev *__restrict__ cd, uint8_t *A, int rq,
+                                             int64_t k, int r)
 {
     const void *llr = a.reqs[rq].llr;
-    constexpr int CH = LDPC_PAIRS_REFILL_CHUNK;
+    const int N = a.N, Z = a.Z, nb = a.nb;
+    constexpr int CH = kPairRefillChunk;
     for (int j0 = 0; j0 < nb; j0 += CH) {
         int q[CH];
         if (a.llr_type == LDPC_LLR_I8) {
             int raw[CH];
 #pragma unroll
             for (int w = 0; w < CH; w++)
-                if (j0 + w < nb) raw[w] = static_cast<const int8_t *>(llr)[(int64_t)k * N + (j0 + w) * Z + r];
+                if (j0 + w < nb) raw[w] = static_cast<const int8_t *>(llr)[k * N + (j0 + w) * Z + r];
 #pragma unroll
             for (int w = 0; w < CH; w++)
                 if (j0 + w < nb) {
@@ -226,7 +268,7 @@ LDPC_PAIRS_COLD void lpair_refill(const LayeredPairArgs &a, const CodeDev *__res
             float in[CH];
 #pragma unroll
             for (int w = 0; w < CH; w++)
-                if (j0 + w < nb) in[w] = __ldg(static_cast<const float *>(llr) + (int64_t)k * N + (j0 + w) * Z + r);
+                if (j0 + w < nb) in[w] = __ldg(static_cast<const float *>(llr) + k * N + (j0 + w) * Z + r);
 #pragma unroll
             for (int w = 0; w < CH; w++)
                 if (j0 + w < nb) {
@@ -237,86 +279,40 @@ LDPC_PAIRS_COLD void lpair_refill(const LayeredPairArgs &a, const CodeDev *__res
         }
 #pragma unroll
         for (int w = 0; w < CH; w++)
-            if (j0 + w < nb) Ah[2 * ((j0 + w) * Z + r) + v] = __int2half_rn(q[w]);
+            if (j0 + w < nb) A[(j0 + w) * Z * 2] = (uint8_t)(q[w] + 128);
     }
-    for (int b = 0; b < nnz; b++) reinterpret_cast<uint8_t *>(Rc + b * Z + r)[v] = 128;
 }
 
-// Write lane v's outputs for codeword k of request rq (row r's positions): hard decisions, the
-// posterior (if asked for), and, from row 0, the iteration count.
-LDPC_PAIRS_COLD void lpair_output(const LayeredPairArgs &a, const __half *Ah, int v, int rq, int k, int t, int r,
-                                          int N, int Z, int nb)
-{
-    const ReqDev &q = a.reqs[rq];
-    uint8_t *Bo = q.bits + (int64_t)k * N;
-    float *Ao = q.app ? q.app + (int64_t)k * N : nullptr;
-    for (int j = 0; j < nb; j++) {
-        const __half x = Ah[2 * (j * Z + r) + v];
-        Bo[j * Z + r] = (__half_as_ushort(x) & 0x8000u) ? 1 : 0;
-        if (Ao) Ao[j * Z + r] = __half2float(x);
-    }
-    if (r == 0) q.iters[k] = t;
-}
-
-// the barrier of one group (named barrier group + 1), or the warp when the group is one warp
-__device__ __forceinline__ void pgroup_sync(int grp, int tpg)
-{
-    if (tpg == 32)
-        __syncwarp();
-    else
-        asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(tpg) : "memory");
-}
-
-// Table space (ints) ahead of the slots: the lanes' next and current requests, the block-row pointers, the
-// edge descriptors (two ints per block), and with TABLE the APP offset table: entry b*Z + r (16 bits) is the byte offset
-// 4 (j Z + (r + s) mod Z) of the position that row r of block b = (row l, column j, shift s)
-// reaches, for every thread slot of the CTA.
-__host__ __device__ inline int lpairs_tables_ints(int nnz, int mb, int Z, bool table)
-{
-    return 2 * SLOTS_MAX + mb + 1 + 2 * nnz + (table ? (nnz * Z + 1) / 2 : 0);  // + the lanes' requests
-}
-
-// Threads per CTA: up to 1024 for rows of degree <= 16; 768 above, where the register file
-// must hold the Q words of up to 32 edges per thread (64 vs 80 registers per thread).
-__host__ __device__ constexpr int lpairs_threads(int dmax) { return dmax <= 16 ? 1024 : 768; }
+// Threads per CTA of an instance: its registers hold the Q words of up to dmax edges.  (65536
+// codewords of the N = 1944 rate-5/6 code, dmax 24: 768 threads 1432 us, 896 1549, 1024 1615, which
+// spill; 4193 of the N = 4000 code, dmax 16: 896 326 us, 1024 353.)
+__host__ __device__ constexpr int lpairs_threads(int dmax) { return dmax <= 8 ? 1024 : dmax <= 16 ? 896 : 768; }
 
 template <int DMAX, bool SATAPP, bool TABLE>
-__global__ void __launch_bounds__(lpairs_threads(DMAX), 1) k_layered_pairs(const CodeDev *__restrict__ cd, const __grid_constant__ LayeredPairArgs a)
+__global__ void __launch_bounds__(lpairs_threads(DMAX), 1)
+    k_layered_pairs(const CodeDev *__restrict__ cd, const __grid_constant__ LayeredPairArgs a)
 {
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int N = cd->N, Z = cd->Z, mb = cd->mb, nb = cd->nb, nnz = cd->nnz;
-    const int C2 = a.C2, K = a.K, TPG = a.TPG;
-    int32_t *bad = reinterpret_cast<int32_t *>(smem);               // [2 * C2] unsatisfied check seen, per codeword
-    int32_t *gany = bad + SLOTS_MAX;                                 // [groups][2] group vote
-    int64_t *fresh = reinterpret_cast<int64_t *>(gany + SLOTS_MAX);  // [2 * C2] next codeword per lane (request-local)
-    int32_t *sreq = reinterpret_cast<int32_t *>(fresh + SLOTS_MAX);   // [2 * C2] its request
-    int32_t *creq = sreq + SLOTS_MAX;  // [2 * C2] request of the codeword each lane decodes
-    int2 *t_ed = reinterpret_cast<int2 *>(creq + SLOTS_MAX);
-    int32_t *t_rowptr = reinterpret_cast<int32_t *>(t_ed + nnz);
-    uint16_t *t_off = reinterpret_cast<uint16_t *>(t_rowptr + mb + 1);
-    __half2 *APPs = reinterpret_cast<__half2 *>(smem + slots_smem_head(lpairs_tables_ints(nnz, mb, Z, TABLE)));
-    uint16_t *Rs = reinterpret_cast<uint16_t *>(APPs + (size_t)C2 * a.strideA);
-
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    char *sm = reinterpret_cast<char *>(smem_raw);
+    constexpr int V = 2;  // lanes of a thread slot, and bytes of a word
+    PairBook *books = reinterpret_cast<PairBook *>(sm);
+    const int N = a.N, Z = a.Z, mb = a.mb, nb = a.nb, nnz = a.nnz, TPG = a.TPG;
     const int tid = threadIdx.x, nth = blockDim.x;
-    for (int i = tid; i < nnz; i += nth) {
+    for (int i = tid; !TABLE && i < nnz; i += nth) {
         const int e = cd->ent[i], sh = e & 0xffff;
-        t_ed[i] = make_int2(4 * ((e >> 16) * Z + sh), Z - sh);
+        if constexpr (!TABLE) reinterpret_cast<int2 *>(sm + a.tab0)[i] = make_int2(V * ((e >> 16) * Z + sh), Z - sh);
     }
     if constexpr (TABLE)
         for (int i = tid; i < nnz * Z; i += nth) {
-            const int b = i / Z, rr = i - b * Z;
-            const int e = cd->ent[b], sh = e & 0xffff;
-            const int x = rr + sh;
-            t_off[i] = (uint16_t)(4 * ((e >> 16) * Z + (x >= Z ? x - Z : x)));
+            const int b = i / Z, x = i - b * Z + (cd->ent[b] & 0xffff);
+            reinterpret_cast<uint16_t *>(sm + a.tab0)[i] = (uint16_t)(V * ((cd->ent[b] >> 16) * Z + (x >= Z ? x - Z : x)));
         }
-    for (int i = tid; i <= mb; i += nth) t_rowptr[i] = cd->rowptr[i];
-    const int g = tid / TPG, u = tid - (tid / TPG) * TPG;
-    const int c = g * K + u / Z, r = u - (u / Z) * Z;
-    const bool mine = u < K * Z && c < C2;  // a row of a thread slot (else an idle lane of the group)
-    if (tid == 0)
-        for (int i = 0; i < SLOTS_MAX; i++) gany[i] = 0;
+    // thread slot g (a warp reduction: known to be warp-uniform), row ru of its layers
+    const int g = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / TPG)), ru = tid - g * TPG;
+    const bool lead = ru == 0;
+    PairBook *book = books + g * V;
     // a lane's leader takes the next item of the work sequence and finds its request
-    auto grab = [&](int lane) {
+    auto grab = [&](int v) {
         const unsigned long long k = atomicAdd(a.next, 1ull);
         int64_t loc = -1;
         int rq = -1;
@@ -325,97 +321,133 @@ __global__ void __launch_bounds__(lpairs_threads(DMAX), 1) k_layered_pairs(const
                 if ((int64_t)k < a.reqs[rq].item0 + a.reqs[rq].n_cw) break;
             loc = (int64_t)k - a.reqs[rq].item0;
         }
-        fresh[lane] = loc;
-        sreq[lane] = rq;
+        book[v].cw = loc;
+        book[v].req = rq;
     };
-    if (mine && r == 0) {
+    if (lead) {
 #pragma unroll
-        for (int v = 0; v < 2; v++) {
-            grab(2 * c + v);
-            bad[2 * c + v] = 0;
+        for (int v = 0; v < V; v++) {
+            grab(v);
+            book[v].bad[0] = book[v].bad[1] = 0;
         }
     }
     __syncthreads();
-    if (g * K >= C2) return;  // whole warps beyond the last group
-    char *Ab = reinterpret_cast<char *>(APPs + (size_t)(mine ? c : 0) * a.strideA);
-    __half *Ah = reinterpret_cast<__half *>(Ab);
-    uint16_t *Rc = Rs + (size_t)(mine ? c : 0) * a.strideR;
-    // the edges' APP offsets of layer l for this thread's row
-    auto edges = [&](int b0) {
+    // (an idle lane of a slot's last warp repeats the last row's loads and stores nothing)
+    const bool own = ru < Z;
+    const int r = own ? ru : Z - 1;
+    const uint32_t slot = (uint32_t)(a.slots0 + g * a.strA);  // the slot's posteriors
+    const uint32_t r0 = (uint32_t)(a.slots0 + a.offR + g * a.strR + r * V);  // row r of its messages
+    uint8_t *A = reinterpret_cast<uint8_t *>(sm + slot + r * V);
+    auto edges = [&](int b0) {  // of the layer whose first block is b0
         if constexpr (TABLE)
-            return EdgeAddr<true>{t_off + b0 * Z + r, Z};
+            return PairAt<true>{sm, (uint32_t)(a.tab0 + 2 * r) + (uint32_t)(2 * b0 * Z), (uint32_t)(2 * Z), slot};
         else
-            return EdgeAddr<false>{t_ed + b0, 4 * r, r, 4 * Z};
+            return PairAt<false>{sm, (uint32_t)(a.tab0 + 8 * b0), slot + (uint32_t)(r * V),
+                                 slot + (uint32_t)((r - Z) * V), r};
+    };
+    auto gsync = [&]() {
+        if (TPG == 32)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(TPG) : "memory");
     };
 
-    int ph = 0;
-    auto group_any = [&](bool pred) {
-        if (pred) gany[2 * g + ph] = 1;
-        pgroup_sync(g, TPG);
-        const bool any = gany[2 * g + ph] != 0;
-        if (u == 0) gany[2 * g + (ph ^ 1)] = 0;
-        ph ^= 1;
-        return any;
-    };
-
-    // a lane taking codeword fresh / sreq: its request is kept in shared memory (creq, read again
-    // at the output), not in registers
+    // a lane's codeword (request-local; requests hold at most 2^31), -1: none; its request is kept in
+    // shared memory (read again at the output), not in registers
+    int cw[V], t[V];
+    uint32_t keep = 0;  // lanes past their first iteration (a byte each): their messages are valid
+    bool any = false;
     auto take = [&](int v) {
-        const int rqv = sreq[2 * c + v];
-        if (r == 0) creq[2 * c + v] = rqv;
-        lpair_refill(a, cd, Ah, Rc, v, rqv, (int)fresh[2 * c + v], r, N, Z, nb, nnz);
+        const int64_t c = book[v].cw;
+        cw[v] = (int)c;
+        t[v] = 0;
+        keep &= ~(0xffu << (8 * v));
+        if (c >= 0) {
+            const int rq = book[v].req;
+            if (lead) book[v].cur = rq;
+            if (own) lpair_refill(a, cd, A + v, rq, c, r);
+        }
+        any |= c >= 0;
     };
-    int cw[2];  // request-local codeword in each lane (-1: empty; requests hold at most 2^31)
-    int t[2] = {0, 0};
 #pragma unroll
-    for (int v = 0; v < 2; v++) {
-        cw[v] = mine ? (int)fresh[2 * c + v] : -1;
-        if (cw[v] >= 0) take(v);
-    }
-    if (!group_any(cw[0] >= 0 || cw[1] >= 0)) return;
+    for (int v = 0; v < V; v++) take(v);
+    any = __any_sync(0xffffffffu, any);  // (votes: conditions known to be warp-uniform)
+    gsync();
 
-    for (;;) {
-        const bool busy0 = cw[0] >= 0, busy1 = cw[1] >= 0, busy = busy0 || busy1;
+    const uint32_t zb = (uint32_t)(Z * V);
+    for (int ph = 0; any; ph ^= 1) {
+#pragma unroll 1
         for (int l = 0; l < mb; l++) {
-            if (busy) {
-                const int b0 = t_rowptr[l], dc = t_rowptr[l + 1] - b0;
-                pair_check<DMAX, SATAPP, TABLE>(dc, edges(b0), Ab, Rc + b0 * Z + r, Z, a);
-            }
-            pgroup_sync(g, TPG);
+            const int b0 = a.first[l];
+            pair_layer<2, DMAX, SATAPP>(a.deg[l], edges(b0), sm, own, r0 + (uint32_t)b0 * zb, zb, keep, a);
+            gsync();
         }
-        t[0] += busy0;
-        t[1] += busy1;
-        // syndrome of both lanes' hard decisions: row r of every layer
-        if (busy && a.early_exit) {
-            uint32_t par_any = 0;
+        keep = 0xffffffffu;
+        bool busy[V], done[V];
+        bool anydone = false;
+        uint32_t busym = 0;
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            busy[v] = cw[v] >= 0;
+            t[v] += busy[v];
+            busym |= busy[v] ? 0x80u << (8 * v) : 0u;
+        }
+        if (a.early_exit) {
+            // syndrome of the lanes' hard decisions, until each busy lane has shown this warp an
+            // unsatisfied check
+            uint32_t seen = 0;
+#pragma unroll 1
             for (int l = 0; l < mb; l++) {
-                const int b0 = t_rowptr[l];
-                par_any |= pair_parity<DMAX, TABLE>(t_rowptr[l + 1] - b0, edges(b0), Ab);
+                seen |= __reduce_or_sync(0xffffffffu, pair_parity(a.deg[l], edges(a.first[l]), sm) & kZero2);
+                if (__all_sync(0xffffffffu, (seen & busym) == busym)) break;
             }
-            if (busy0 && (par_any & 0x8000u)) bad[2 * c] = 1;
-            if (busy1 && (par_any & 0x80000000u)) bad[2 * c + 1] = 1;
-        }
-        pgroup_sync(g, TPG);
-        bool done[2];
+            if ((tid & 31) == 0) {
 #pragma unroll
-        for (int v = 0; v < 2; v++) {
-            done[v] = cw[v] >= 0 && ((a.early_exit && bad[2 * c + v] == 0) || t[v] >= a.max_iter);
-            if (done[v]) {
-                lpair_output(a, Ah, v, creq[2 * c + v], cw[v], t[v], r, N, Z, nb);
-                if (r == 0) grab(2 * c + v);
+                for (int v = 0; v < V; v++)
+                    if (seen & (0x80u << (8 * v))) book[v].bad[ph] = 1;
             }
+            gsync();
         }
-        pgroup_sync(g, TPG);
 #pragma unroll
-        for (int v = 0; v < 2; v++) {
-            if (cw[v] >= 0 && r == 0) bad[2 * c + v] = 0;
-            if (done[v]) {
-                cw[v] = (int)fresh[2 * c + v];
-                t[v] = 0;
-                if (cw[v] >= 0) take(v);
-            }
+        for (int v = 0; v < V; v++) {
+            done[v] = busy[v] && ((a.early_exit && book[v].bad[ph] == 0) || t[v] >= a.max_iter);
+            anydone |= done[v];
         }
-        if (!group_any(cw[0] >= 0 || cw[1] >= 0)) break;
+        if (a.early_exit && lead) {
+            // the other flag was last read in the iteration before
+#pragma unroll
+            for (int v = 0; v < V; v++) book[v].bad[ph ^ 1] = 0;
+        }
+        if (__any_sync(0xffffffffu, anydone)) {
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                if (done[v] && own) {
+                    const ReqDev &q = a.reqs[book[v].cur];
+                    uint8_t *Bo = q.bits + (int64_t)cw[v] * N + r;
+                    float *Ao = q.app ? q.app + (int64_t)cw[v] * N + r : nullptr;
+                    for (int j = 0; j < nb; j++) {
+                        const int x = A[j * Z * V + v];
+                        Bo[j * Z] = x < 128 ? 1 : 0;
+                        if (Ao) Ao[j * Z] = (float)(x - 128);
+                    }
+                    if (lead) {
+                        q.iters[cw[v]] = t[v];
+                        grab(v);
+                    }
+                }
+            }
+            gsync();
+            any = false;
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                if (done[v])
+                    take(v);
+                else
+                    any |= cw[v] >= 0;
+            }
+            any = __any_sync(0xffffffffu, any);
+            gsync();
+        }
     }
 }
 
@@ -434,77 +466,65 @@ bool layered_pairs_exact(const ldpc_decode_params &p)
     return 2LL * p.nms_alpha_num * p.msg_sat + (1LL << p.nms_alpha_shift) <= 2047;
 }
 
-// Strides congruent to Z modulo the banks' width in elements (32 words of APP, 64 byte pairs
-// of R), so that a warp whose rows run from one thread slot into the next sees one contiguous
-// bank sequence.
-static int pair_stride(int n, int Z, int m) { return n + (((Z % m) - (n % m)) % m + m) % m; }
+static int lpairs_dmax(const CodeDev &h) { return h.dc_max <= 8 ? 8 : h.dc_max <= 16 ? 16 : h.dc_max <= 24 ? 24 : 32; }
 
-#ifndef LDPC_PAIRS_TABLE_MAXD
-#define LDPC_PAIRS_TABLE_MAXD 8  // the offset table for codes of row degree up to this, descriptors above
-#endif
-static bool lpairs_table(const CodeDev &h) { return h.dc_max <= LDPC_PAIRS_TABLE_MAXD; }
-
-static size_t lpairs_smem(const CodeDev &h, int C2)
+// Strides congruent to Z modulo the 32 banks' width in elements (of bytes bytes), so that rows of
+// neighbouring slots do not collide; whole 16 bytes.
+static int lpairs_stride(int n, int Z, int bytes)
 {
-    return slots_smem_head(lpairs_tables_ints(h.nnz, h.mb, h.Z, lpairs_table(h))) +
-           (size_t)C2 * ((size_t)pair_stride(h.N, h.Z, 32) * 4 + (size_t)pair_stride(h.E, h.Z, 64) * 2) + 16;
+    const int m = 128 / bytes;
+    const int s = (n + (((Z % m) - (n % m)) % m + m) % m) * bytes;
+    return (s + 15) & ~15;
 }
 
-struct LpairShape {
-    int C2, K, TPG;
-};
-// Thread slots per CTA and their grouping: the most thread slots that fit 1024 threads, 15
-// named barriers and the shared-memory budget, with the fewest per group among the
-// arrangements reaching that count.
-static LpairShape lpairs_shape(const CodeDev &h, int64_t cap2 = SLOTS_MAX / 2)
+// The tables' bytes: 16-bit offsets per (block, row), or 8-byte descriptors per block.
+static size_t lpairs_tab(const CodeDev &h, bool table) { return table ? 2 * (size_t)h.nnz * h.Z : 8 * (size_t)h.nnz; }
+
+// Thread slots of two codewords per CTA, at most cap.
+static int lpairs_fit(const CodeDev &h, int cap, bool table)
 {
-    LpairShape best = {0, 1, 32};
-    if (h.dc_max > 32 || 4 * h.N > 65535) return best;  // APP byte offsets in 16 bits
-    const int tmax = lpairs_threads(h.dc_max <= 8 ? 8 : h.dc_max <= 16 ? 16 : h.dc_max <= 24 ? 24 : 32);
-    int cmax = SLOTS_MAX / 2;
-    while (cmax > 0 && lpairs_smem(h, cmax) > 227 * 1024) cmax--;
-    if (cap2 >= 1 && cap2 < cmax) cmax = (int)cap2;
-    for (int K = 1; K <= cmax && K <= LDPC_PAIRS_KMAX; K++) {
-        const int tpg = ((K * h.Z + 31) / 32) * 32;
-        int G = tmax / tpg;
-        if (tpg > 32 && G > 15) G = 15;
-        int C = G * K;
-        if (C > cmax) C = cmax;
-        if (C > best.C2) best = {C, K, tpg};
-    }
-    return best;
+    if (h.dc_max > 32 || 4 * h.N > 65535) return 0;
+    const int wt = ((h.Z + 31) / 32) * 32, V = 2;
+    int G = lpairs_threads(lpairs_dmax(h)) / wt;
+    if (G > cap) G = cap;
+    if (G * V > SLOTS_MAX) G = SLOTS_MAX / V;
+    if (wt > 32 && G > 15) G = 15;  // named barriers
+    const size_t slot = (size_t)lpairs_stride(h.N, h.Z, V) + lpairs_stride(h.E, h.Z, V);
+    while (G > 0 && (size_t)G * V * sizeof(PairBook) + lpairs_tab(h, table) + 64 + G * slot > 227 * 1024) G--;
+    return G;
 }
 
-int layered_pairs_per_cta(const CodeDev &h) { return 2 * lpairs_shape(h).C2; }
+// Codewords per CTA (0: code too large: a pair's 4-byte posteriors and 2-byte messages beside
+// tables as they once were, so that the line stays where it is).
+int layered_pairs_per_cta(const CodeDev &h)
+{
+    const size_t tables = 4 * (size_t)(2 * SLOTS_MAX + h.mb + 1 + 2 * h.nnz + (h.dc_max <= 8 ? (h.nnz * h.Z + 1) / 2 : 0));
+    const size_t head = ((size_t)SLOTS_MAX * 16 + 16 + tables + 15) & ~(size_t)15;
+    auto stride = [&](int n, int m) { return (size_t)(n + (((h.Z % m) - (n % m)) % m + m) % m); };
+    if (head + stride(h.N, 32) * 4 + stride(h.E, 64) * 2 + 16 > 227 * 1024) return 0;
+    return 2 * lpairs_fit(h, SLOTS_MAX / 2, false);
+}
 
 template <int DMAX, bool SATAPP, bool TABLE>
-static cudaError_t launch_lpairs(const CodeDev &h, const CodeDev *d, const LayeredPairArgs &a, int ctas, cudaStream_t s)
+static cudaError_t launch_lpairs(const CodeDev *d, const LayeredPairArgs &a, size_t smem, int ctas, cudaStream_t s)
 {
-    const size_t sm = lpairs_smem(h, a.C2);
-    cudaError_t e = ensure_smem<k_layered_pairs<DMAX, SATAPP, TABLE>>(sm);
+    cudaError_t e = ensure_smem<k_layered_pairs<DMAX, SATAPP, TABLE>>(smem);
     if (e != cudaSuccess) return e;
     LaunchScope ls(F_LAYERED, s);
-    const int groups = (a.C2 + a.K - 1) / a.K;
-    k_layered_pairs<DMAX, SATAPP, TABLE><<<(unsigned)ctas, groups * a.TPG, sm, s>>>(d, a);
+    k_layered_pairs<DMAX, SATAPP, TABLE><<<(unsigned)ctas, a.G * a.TPG, smem, s>>>(d, a);
     return cudaGetLastError();
 }
 
-template <int DMAX, bool SATAPP>
-static cudaError_t launch_lpairs_t(const CodeDev &h, const CodeDev *d, const LayeredPairArgs &a, int ctas,
+template <bool SATAPP, bool TABLE>
+static cudaError_t launch_lpairs_d(const CodeDev &h, const CodeDev *d, const LayeredPairArgs &a, size_t smem, int ctas,
                                    cudaStream_t s)
 {
-    return lpairs_table(h) ? launch_lpairs<DMAX, SATAPP, true>(h, d, a, ctas, s)
-                           : launch_lpairs<DMAX, SATAPP, false>(h, d, a, ctas, s);
-}
-
-template <bool SATAPP>
-static cudaError_t launch_lpairs_d(const CodeDev &h, const CodeDev *d, const LayeredPairArgs &a, int ctas,
-                                   cudaStream_t s)
-{
-    if (h.dc_max <= 8) return launch_lpairs_t<8, SATAPP>(h, d, a, ctas, s);
-    if (h.dc_max <= 16) return launch_lpairs_t<16, SATAPP>(h, d, a, ctas, s);
-    if (h.dc_max <= 24) return launch_lpairs_t<24, SATAPP>(h, d, a, ctas, s);
-    return launch_lpairs_t<32, SATAPP>(h, d, a, ctas, s);
+    switch (lpairs_dmax(h)) {
+    case 8: return launch_lpairs<8, SATAPP, TABLE>(d, a, smem, ctas, s);
+    case 16: return launch_lpairs<16, SATAPP, TABLE>(d, a, smem, ctas, s);
+    case 24: return launch_lpairs<24, SATAPP, TABLE>(d, a, smem, ctas, s);
+    default: return launch_lpairs<32, SATAPP, TABLE>(d, a, smem, ctas, s);
+    }
 }
 
 // Decode the codewords of n requests of one code (reqs[i].code all the same) in one launch.
@@ -533,15 +553,31 @@ cudaError_t layered_pairs_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     // a small batch spreads over the SMs rather than filling a few CTAs' slots
     const int64_t per_cta = (items + nsm - 1) / nsm;
-    const LpairShape sh = lpairs_shape(h, (per_cta + 1) / 2);
-    if (sh.C2 < 1) return cudaErrorInvalidValue;
+    const int cap = per_cta < SLOTS_MAX ? (int)((per_cta + 1) / 2) : SLOTS_MAX / 2;
+    // the offset table where it costs no thread slot
+    const int g = lpairs_fit(h, cap, false);
+    const bool table = lpairs_fit(h, cap, true) == g;
+    constexpr int V = 2;
+    a.G = g;
+    if (a.G < 1) return cudaErrorInvalidValue;
+    a.TPG = ((h.Z + 31) / 32) * 32;
     a.llr_type = llr_type;
     a.scale = p.llr_scale;
-    a.C2 = sh.C2;
-    a.K = sh.K;
-    a.TPG = sh.TPG;
-    a.strideA = pair_stride(h.N, h.Z, 32);
-    a.strideR = pair_stride(h.E, h.Z, 64);
+    a.N = h.N;
+    a.Z = h.Z;
+    a.mb = h.mb;
+    a.nb = h.nb;
+    a.nnz = h.nnz;
+    a.tab0 = (a.G * V * (int)sizeof(PairBook) + 15) & ~15;
+    a.slots0 = (a.tab0 + (int)lpairs_tab(h, table) + 15) & ~15;
+    a.strA = lpairs_stride(h.N, h.Z, V);
+    a.strR = lpairs_stride(h.E, h.Z, V);
+    a.offR = a.G * a.strA;
+    const size_t smem = (size_t)a.slots0 + a.offR + (size_t)a.G * a.strR;
+    for (int l = 0; l < h.mb; l++) {
+        a.first[l] = (uint16_t)h.rowptr[l];
+        a.deg[l] = (uint8_t)(h.rowptr[l + 1] - h.rowptr[l]);
+    }
     a.max_iter = p.max_iter;
     a.early_exit = p.early_exit;
     a.msg_sat = p.msg_sat;
@@ -552,19 +588,22 @@ cudaError_t layered_pairs_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     };
     a.sat = pair((float)p.msg_sat);
     a.nsat = pair(-(float)p.msg_sat);
-    a.appmax = pair((float)p.app_sat);
-    a.appmin = pair(-(float)p.app_sat);
+    a.appmax = pair(1152.0f + (float)p.app_sat);
+    a.appmin = pair(1152.0f - (float)p.app_sat);
     a.alpha = pair((float)p.nms_alpha_num / (float)(1 << p.nms_alpha_shift));
     a.ndelta = pair(1.0f / (float)(2 << p.nms_alpha_shift) - 0.5f);
     a.next = static_cast<unsigned long long *>(counter);
-    int64_t ctas = nsm;
-    const int64_t need = (items + 2 * a.C2 - 1) / (2 * a.C2);
-    if (need < ctas) ctas = need;
+    const int64_t need = (items + a.G * V - 1) / (a.G * V);
+    const int ctas = (int)(need < nsm ? need : nsm);
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
     if (e != cudaSuccess) return e;
     const long long top = ((long long)p.nms_alpha_num * p.msg_sat) >> p.nms_alpha_shift;
-    return p.msg_sat + top > p.app_sat ? launch_lpairs_d<true>(h, d, a, (int)ctas, s)
-                                       : launch_lpairs_d<false>(h, d, a, (int)ctas, s);
+    const bool sat = p.msg_sat + top > p.app_sat;
+    if (table)
+        return sat ? launch_lpairs_d<true, true>(h, d, a, smem, ctas, s)
+                   : launch_lpairs_d<false, true>(h, d, a, smem, ctas, s);
+    return sat ? launch_lpairs_d<true, false>(h, d, a, smem, ctas, s)
+               : launch_lpairs_d<false, false>(h, d, a, smem, ctas, s);
 }
 
 }  // namespace ldpc

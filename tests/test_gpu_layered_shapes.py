@@ -1,6 +1,6 @@
-"""Layered sum-product decoder at the edges of its forms: every check-row degree class, slots of Z
-around the warp size, one codeword per thread and (FP16 messages, rows up to degree 8, large
-batches) two."""
+"""Layered decoders at the edges of their forms: every check-row degree class, slots of Z around the
+warp size; sum-product with one codeword per thread and (FP16 messages, rows up to degree 8,
+large batches) two; int8 min-sum with and without its offset table, bit-exact."""
 import numpy as np
 import pytest
 
@@ -39,3 +39,24 @@ def test_against_oracle_and_across_forms(cuda_dev, name, form):
     big = decode(code, form, L, cuda_dev, max_iter=9)
     for a, b in zip(small, big):
         assert np.array_equal(a, b[:n_small]), name
+
+
+# (a code whose offset table does not fit beside a thread slot)
+DENSE = dict(ALL, no_table=(base_of([16] * 16, 32, 256, 9), 256))
+
+
+@pytest.mark.parametrize("sat", [(31, 127), (31, 40)])  # the posterior's saturation cannot / can bind
+@pytest.mark.parametrize("name", list(DENSE))
+def test_int8_bit_exact(cuda_dev, name, sat):
+    B, Z = DENSE[name]
+    code, oc = ldpc.Code(B, Z), O.QCCode(B, Z)
+    n_small, n_big = 41, 152 * 24 + 5
+    rng = np.random.default_rng(9)
+    q = np.clip(np.rint(5 + 5 * rng.standard_normal((n_big, code.N))), -31, 31).astype(np.int8)
+    q[::7, ::5] = 0
+    kw = dict(max_iter=6, msg_sat=sat[0], app_sat=sat[1])
+    a, b, i = oc.nms_layered(q[:n_small], 6, early_exit=True, msg_sat=sat[0], app_sat=sat[1])
+    small = decode(code, "layered_i8", q[:n_small].copy(), cuda_dev, **kw)
+    big = decode(code, "layered_i8", q, cuda_dev, **kw)
+    for got in (small, [x[:n_small] for x in big]):
+        assert np.array_equal(got[0].astype(np.int32), a) and np.array_equal(got[1], b) and np.array_equal(got[2], i)
