@@ -127,7 +127,8 @@ ldpc_status ldpc_workspace_size(const ldpc_code *code, const ldpc_decode_params 
  *   app_dev    device, [n_cw][N] fp32 posterior LLRs after the last iteration, or NULL
  *              (integer forms write their integer APP converted exactly to fp32).
  *   workspace  device scratch of >= ldpc_workspace_size() bytes, 256-byte aligned, or NULL
- *              to let the library allocate and free it stream-ordered on `stream`.
+ *              to let the library allocate and free it stream-ordered on `stream` (the
+ *              on-chip decoders take nothing for batches of up to one codeword per SM).
  * n_cw == 0 returns LDPC_OK with nothing launched. */
 ldpc_status ldpc_decode_batch(const ldpc_code *code, const ldpc_decode_params *p,
                               const void *llr_dev, int32_t llr_type, int64_t n_cw,

@@ -315,8 +315,12 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
     a.X = p.phi_clamp;
     int ctas = nsm;
     if (min_ctas < ctas) ctas = (int)min_ctas;
-    cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * ng, s);
-    if (e != cudaSuccess) return e;
+    if (ng == 1 && items_of[0] <= (int64_t)ctas * a.groups[0].G * V) a.next = nullptr;  // no refills: no counter
+    else if (!counters) return cudaErrorInvalidValue;
+    if (a.next) {
+        const cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * ng, s);
+        if (e != cudaSuccess) return e;
+    }
     const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
     if (p.msg == LDPC_MSG_F16)
         return hc ? flood_slots_launch<__half, true>(dmax, V, a, smem, threads, ctas, s)

@@ -52,7 +52,7 @@ struct FloodReq {
 //   32-bit words (from t_row): per block row in ascending degree the index of its first edge
 //     descriptor << 8 | its degree; per block column in ascending degree its number
 struct FloodArgs {
-    unsigned long long *next;  // [n_groups] work counters, zero at launch
+    unsigned long long *next;  // [n_groups] work counters, zero at launch; null: one group, all codewords resident
     int n_groups;
     int max_iter, early_exit;
     float X;

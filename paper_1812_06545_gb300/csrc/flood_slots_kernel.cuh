@@ -152,9 +152,12 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
         FloodBook *book = books + (member ? g : 0) * V;
         const int32_t *rows = reinterpret_cast<const int32_t *>(tab + gd.t_row);
 
-        // a slot's leader takes the group's next codeword and finds its request
-        auto grab = [&](int v) {
-            const unsigned long long k = atomicAdd(a.next + grp, 1ull);
+        // a slot's leader takes the group's next codeword and finds its request; without a work
+        // counter every codeword has a slot from the start
+        auto grab = [&](int v, bool first) {
+            const unsigned long long k = a.next  ? atomicAdd(a.next + grp, 1ull)
+                                         : first ? blockIdx.x + (unsigned long long)gridDim.x * (g * V + v)
+                                                 : ~0ull;
             int64_t loc = -1;
             int rq = -1;
             if (k < (unsigned long long)gd.n_items) {
@@ -169,7 +172,7 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
         if (lead) {
 #pragma unroll
             for (int v = 0; v < V; v++) {
-                grab(v);
+                grab(v, true);
                 book[v].bad[0] = book[v].bad[1] = 0;
             }
         }
@@ -295,7 +298,7 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
                     }
                     if (lead) {
                         q.iters[cw[v]] = t[v];
-                        grab(v);
+                        grab(v, false);
                     }
                 }
             }

@@ -311,9 +311,12 @@ __global__ void __launch_bounds__(lpairs_threads(DMAX), 1)
     const int g = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / TPG)), ru = tid - g * TPG;
     const bool lead = ru == 0;
     PairBook *book = books + g * V;
-    // a lane's leader takes the next item of the work sequence and finds its request
-    auto grab = [&](int v) {
-        const unsigned long long k = atomicAdd(a.next, 1ull);
+    // a lane's leader takes the next item of the work sequence and finds its request; without a
+    // work counter every item has a lane from the start
+    auto grab = [&](int v, bool first) {
+        const unsigned long long k = a.next  ? atomicAdd(a.next, 1ull)
+                                     : first ? blockIdx.x + (unsigned long long)gridDim.x * (g * V + v)
+                                             : ~0ull;
         int64_t loc = -1;
         int rq = -1;
         if (k < (unsigned long long)a.n_items) {
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(lpairs_threads(DMAX), 1)
     if (lead) {
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            grab(v);
+            grab(v, true);
             book[v].bad[0] = book[v].bad[1] = 0;
         }
     }
@@ -432,7 +435,7 @@ __global__ void __launch_bounds__(lpairs_threads(DMAX), 1)
                     }
                     if (lead) {
                         q.iters[cw[v]] = t[v];
-                        grab(v);
+                        grab(v, false);
                     }
                 }
             }
@@ -595,8 +598,12 @@ cudaError_t layered_pairs_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     a.next = static_cast<unsigned long long *>(counter);
     const int64_t need = (items + a.G * V - 1) / (a.G * V);
     const int ctas = (int)(need < nsm ? need : nsm);
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    if (items <= (int64_t)ctas * a.G * V) a.next = nullptr;  // no refills: no counter
+    else if (!counter) return cudaErrorInvalidValue;
+    if (a.next) {
+        const cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+    }
     const long long top = ((long long)p.nms_alpha_num * p.msg_sat) >> p.nms_alpha_shift;
     const bool sat = p.msg_sat + top > p.app_sat;
     if (table)

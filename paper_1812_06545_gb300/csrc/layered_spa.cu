@@ -334,14 +334,17 @@ __global__ void __launch_bounds__(lspa_threads(DMAX, V, sizeof(MsgT) == 2), 1)
     const int g = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / TPG)), ru = tid - g * TPG;
     const bool own = ru < Z, lead = ru == 0;  // (idle lanes of the last warp repeat row Z - 1 and store nothing)
     LspaBook *book = books + g * V;
-    auto grab = [&](int v) {
-        const unsigned long long k = atomicAdd(a.next, 1ull);
+    // the next codeword; without a work counter every codeword has a slot from the start
+    auto grab = [&](int v, bool first) {
+        const unsigned long long k = a.next  ? atomicAdd(a.next, 1ull)
+                                     : first ? blockIdx.x + (unsigned long long)gridDim.x * (g * V + v)
+                                             : ~0ull;
         book[v].cw = k < (unsigned long long)a.n_cw ? (int64_t)k : -1;
     };
     if (lead) {
 #pragma unroll
         for (int v = 0; v < V; v++) {
-            grab(v);
+            grab(v, true);
             book[v].bad[0] = book[v].bad[1] = 0;
         }
     }
@@ -458,7 +461,7 @@ __global__ void __launch_bounds__(lspa_threads(DMAX, V, sizeof(MsgT) == 2), 1)
                     }
                     if (lead) {
                         a.iters[cw[v]] = t[v];
-                        grab(v);
+                        grab(v, false);
                     }
                 }
             }
@@ -589,8 +592,12 @@ cudaError_t layered_spa_decode(const CodeDev &h, const CodeDev *d, const ldpc_de
         a.deg[l] = (uint8_t)(h.rowptr[l + 1] - h.rowptr[l]);
     }
     const int64_t need = (n_cw + a.G * V - 1) / (a.G * V), ctas = need < nsm ? need : nsm;
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+    if (n_cw <= ctas * a.G * V) a.next = nullptr;  // no refills: no counter
+    else if (!counter) return cudaErrorInvalidValue;
+    if (a.next) {
+        const cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return e;
+    }
     const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
     if (V == 2)
         return hc ? launch_lspa<8, 2, __half, true>(d, a, smem, ctas, s)

@@ -127,6 +127,71 @@ cudaError_t device_status_word(int dev, unsigned int **out)
     return cudaSuccess;
 }
 
+// Scratch of calls that bring no workspace.  The on-chip decoders need SLOTS_WS_BYTES of work
+// counters.  The device's default pool gives its memory back to the system at every
+// synchronisation, so a call that was waited for mapped it anew each time: one frame of the
+// N = 648 code, launched and waited for, took 238 us, of which 220 were the allocation.  A pool
+// of the library's own that keeps the one chunk it reserves (32 MiB, the driver's granularity;
+// a threshold of 2 MiB changed nothing) takes that to 55 us.  It lives with the codes of its
+// device and is destroyed with the last of them.
+namespace {
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[64];
+int g_pool_users[64];
+constexpr uint64_t kPoolKeep = 32u << 20;  // bytes the pool keeps across synchronisations
+}  // namespace
+
+// Take a share in the device's scratch pool (null if the device has none: the default pool serves).
+static cudaMemPool_t pool_acquire(int dev)
+{
+    if (dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pool[dev]) {
+        cudaMemPoolProps pr;
+        memset(&pr, 0, sizeof pr);
+        pr.allocType = cudaMemAllocationTypePinned;
+        pr.handleTypes = cudaMemHandleTypeNone;
+        pr.location.type = cudaMemLocationTypeDevice;
+        pr.location.id = dev;
+        uint64_t keep = kPoolKeep;
+        if (cudaMemPoolCreate(&g_pool[dev], &pr) != cudaSuccess ||
+            cudaMemPoolSetAttribute(g_pool[dev], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            if (g_pool[dev]) cudaMemPoolDestroy(g_pool[dev]);
+            g_pool[dev] = nullptr;
+            cudaGetLastError();
+            return nullptr;
+        }
+    }
+    g_pool_users[dev]++;
+    return g_pool[dev];
+}
+
+static void pool_release(int dev, cudaMemPool_t pool)
+{
+    if (!pool) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (--g_pool_users[dev] == 0) {
+        cudaMemPoolDestroy(g_pool[dev]);  // (memory still in use is released when its stream is done with it)
+        g_pool[dev] = nullptr;
+    }
+}
+
+// Allocate scratch on the stream: the work counters from the code's pool, everything else, and
+// everything in a stream capture (whose allocations become graph nodes), as the runtime does.
+static cudaError_t scratch_alloc(const ldpc_code *c, void **ws, size_t bytes, cudaStream_t s)
+{
+    if (c->pool && bytes <= SLOTS_WS_BYTES) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        int dev = -1;
+        if (cudaStreamIsCapturing(s, &st) == cudaSuccess && st == cudaStreamCaptureStatusNone &&
+            cudaGetDevice(&dev) == cudaSuccess && dev == c->device &&
+            cudaMallocFromPoolAsync(ws, bytes, c->pool, s) == cudaSuccess)
+            return cudaSuccess;
+        cudaGetLastError();
+    }
+    return cudaMallocAsync(ws, bytes, s);
+}
+
 // Swap the status word for zero in stream order (kernels of other streams may set bits at
 // any time; an exchange loses none of them).
 __global__ void k_take_status(unsigned int *w) { w[1] = atomicExch(w, 0u); }
@@ -169,6 +234,7 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
     if (!c) return fail(LDPC_ENOMEM, "host allocation failed");
     memset(&c->host, 0, sizeof c->host);
     c->dev = nullptr;
+    c->pool = nullptr;
     c->tuned_flood[0] = c->tuned_flood[1] = SCHED_UNTUNED;
     c->tuned_layered = SCHED_UNTUNED;
     CodeDev &h = c->host;
@@ -244,6 +310,9 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
         delete c;
         return cuda_fail(e, "device code tables");
     }
+    c->sms = 0;
+    if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
+    c->pool = ldpc::pool_acquire(c->device);
     *out = c;
     return LDPC_OK;
 }
@@ -252,6 +321,7 @@ void ldpc_code_destroy(ldpc_code *c)
 {
     if (!c) return;
     if (c->dev) cudaFree(c->dev);
+    ldpc::pool_release(c->device, c->pool);
     delete c;
 }
 
@@ -372,6 +442,16 @@ static bool use_layered_spa(const ldpc_decode_params *p)
     return p->sched == LDPC_SCHED_LAYERED && p->algo == LDPC_ALGO_SPA;
 }
 
+// Whether a decode of n_cw codewords runs without scratch: no more of them than SMs, so that
+// every one has a slot from the start and the on-chip decoders need no work counter.  Without
+// the allocation, the counter's clearing and the free, one frame of the N = 648 code takes 18 us
+// back to back (24 with them, from the pool) and 36 waited for (55).  Beyond that many the
+// decoders choose how many slots an SM gets, so that the counter's memory is there for them.
+static bool no_scratch(const ldpc_code *c, const ldpc_decode_params *p, int64_t n_cw)
+{
+    return n_cw <= c->sms && (use_layered_spa(p) || (use_layered_slots(c, p) && use_layered_pairs(c, p)) || use_slots(c, p));
+}
+
 static size_t ws_bytes(const ldpc_code *c, const ldpc_decode_params *p, int64_t n_cw)
 {
     if (n_cw == 0) return 0;
@@ -414,8 +494,8 @@ ldpc_status ldpc_decode_batch(const ldpc_code *c, const ldpc_decode_params *p, c
         if (workspace_bytes < need)
             return fail(LDPC_ENOMEM, "workspace of %zu bytes < %zu needed", workspace_bytes, need);
         if (reinterpret_cast<uintptr_t>(ws) & 255) return fail(LDPC_EINVAL, "workspace must be 256-byte aligned");
-    } else {
-        e = cudaMallocAsync(&ws, need, s);
+    } else if (!no_scratch(c, p, n_cw)) {
+        e = ldpc::scratch_alloc(c, &ws, need, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(LDPC_ENOMEM, "workspace allocation of %zu bytes failed: %s", need, cudaGetErrorString(e));
@@ -486,7 +566,7 @@ ldpc_status ldpc_decode_multi(const ldpc_request *reqs, int32_t n_req, const ldp
             return fail(LDPC_ENOMEM, "workspace of %zu bytes < %zu needed", workspace_bytes, ldpc::SLOTS_WS_BYTES);
         if (reinterpret_cast<uintptr_t>(ws) & 255) return fail(LDPC_EINVAL, "workspace must be 256-byte aligned");
     } else {
-        e = cudaMallocAsync(&ws, ldpc::SLOTS_WS_BYTES, s);
+        e = ldpc::scratch_alloc(reqs[0].code, &ws, ldpc::SLOTS_WS_BYTES, s);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return fail(LDPC_ENOMEM, "workspace allocation failed: %s", cudaGetErrorString(e));

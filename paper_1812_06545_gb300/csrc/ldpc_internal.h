@@ -147,6 +147,8 @@ struct ldpc_code {
     ldpc::CodeDev host;
     ldpc::CodeDev *dev;
     int device;
+    int sms;             // SMs of the device
+    cudaMemPool_t pool;  // the device's scratch pool (shared with its other codes), or null
     int4 *ftab;          // flooding slot decoder's tables: [2 * (F16) + V - 1][n_ftab] (flood_slots.h)
     int n_ftab;
     int tuned_flood[2];  // per message type (F32, F16)

@@ -3,6 +3,7 @@ warp size; sum-product with one codeword per thread and (FP16 messages, rows up 
 large batches) two; int8 min-sum with and without its offset table, bit-exact."""
 import numpy as np
 import pytest
+import torch
 
 from oracle import oracle as O
 from paper_1812_06545_gb300 import ldpc
@@ -60,3 +61,17 @@ def test_int8_bit_exact(cuda_dev, name, sat):
     big = decode(code, "layered_i8", q, cuda_dev, **kw)
     for got in (small, [x[:n_small] for x in big]):
         assert np.array_equal(got[0].astype(np.int32), a) and np.array_equal(got[1], b) and np.array_equal(got[2], i)
+
+
+@pytest.mark.parametrize("form", ["flood_f32", "flood_f16", "layered_f32", "layered_f16", "layered_i8"])
+def test_batches_around_the_number_of_sms(cuda_dev, form):
+    """Up to one codeword per SM needs no scratch, up to one per slot no work counter: at each edge
+    every codeword is decoded once, as in a larger batch."""
+    sms = torch.cuda.get_device_properties(cuda_dev).multi_processor_count
+    code = ldpc.Code(*CODES["to12"])
+    rng = np.random.default_rng(10)
+    L = (2.5 + 2.2 * rng.standard_normal((40 * sms, code.N))).astype(np.float32)
+    big = decode(code, form, L, cuda_dev, max_iter=7)
+    for n in (1, 2, sms - 1, sms, sms + 1, 2 * sms + 1, 3 * sms):
+        for a, b in zip(decode(code, form, L[:n].copy(), cuda_dev, max_iter=7), big):
+            assert np.array_equal(a, b[:n]), (form, n)
