@@ -1,15 +1,16 @@
 // The flooding check-node update of one check row, for one or two codewords per thread
-// (flooding slot decoder, two-SM cluster decoder).
+// (flooding slot decoder) or of two check rows of one codeword (two-SM cluster decoder).
 #pragma once
 
 #include "slot_common.cuh"
 
 namespace ldpc {
 
-// ------------------------------------------------------------------ V codewords per thread
+// ------------------------------------------------------------------ V rows per thread
 //
-// A value of a thread is a float (one codeword) or a float2 (two codewords, whose multiplies
-// and adds issue as packed pairs; each half is rounded exactly as the scalar operation).
+// A value of a thread is a float (one codeword) or a float2 (two codewords, or two check rows
+// of one block row, whose multiplies and adds issue as packed pairs; each half is rounded
+// exactly as the scalar operation).
 template <int V>
 struct Vec;
 template <>
@@ -84,10 +85,18 @@ struct OwnMem {
     char *sm;
     __device__ __forceinline__ VT<V> app(uint32_t o) const { return Sm<float, V>::ld(sm + o); }
     __device__ __forceinline__ VT<V> msg(uint32_t o) const { return Sm<MsgT, V>::ld(sm + o); }
-    __device__ __forceinline__ void put(uint32_t o, VT<V> x) const { Sm<MsgT, V>::st(sm + o, x); }
+    template <typename PL>
+    __device__ __forceinline__ void put(const PL &p, uint32_t o, VT<V> x) const
+    {
+        if (p.own) Sm<MsgT, V>::st(sm + o, x);
+    }
     // a message's word as the place of a float (FP32 messages)
     __device__ __forceinline__ VT<V> word(uint32_t o) const { return Sm<float, V>::ld(sm + o); }
-    __device__ __forceinline__ void put_word(uint32_t o, VT<V> x) const { Sm<float, V>::st(sm + o, x); }
+    template <typename PL>
+    __device__ __forceinline__ void put_word(const PL &p, uint32_t o, VT<V> x) const
+    {
+        if (p.own) Sm<float, V>::st(sm + o, x);
+    }
 };
 
 // ------------------------------------------------------------------ the check rule
@@ -131,6 +140,7 @@ __device__ __forceinline__ float2 neg_mag(float2 al, float2 be)
 // and less one block (for the edges whose row wraps), and its row.
 template <int V>
 struct Place {
+    using Ref = uint32_t;  // an operand's offset
     uint32_t a0, a1, r0, r1;
     int r;
     bool own;  // an idle lane of a slot's last warp repeats the last row's loads and stores nothing
@@ -138,7 +148,7 @@ struct Place {
 
 // The edge's operand offsets.  With one element size for APP and messages the two regions of
 // a slot are at a fixed distance (already in the descriptor's .y), so one select serves both.
-template <int V, typename MsgT>
+template <typename MsgT, int V>
 __device__ __forceinline__ void edge_at(const int4 &e, const Place<V> &p, uint32_t &ao, uint32_t &ro)
 {
     const bool w = p.r >= e.z;
@@ -151,22 +161,23 @@ __device__ __forceinline__ void edge_at(const int4 &e, const Place<V> &p, uint32
 }
 
 // Rows up to degree 8: every edge's state in registers.
-template <int D, int V, typename MsgT, bool B2, bool HC, typename MEM>
-__device__ __forceinline__ void check_narrow(const int4 *__restrict__ ed, const MEM mem, const Place<V> &p, float Xb,
+template <int D, int V, typename MsgT, bool B2, bool HC, typename MEM, typename PL>
+__device__ __forceinline__ void check_narrow(const int4 *__restrict__ ed, const MEM mem, const PL &p, float Xb,
                                              float Pb, uint32_t (&pbad)[V])
 {
     constexpr uint32_t kSign = 0x80000000u;
     using T = VT<V>;
     const T one = vset(T(), 1.0f), zero = vset(T(), 0.0f);
     T d[D];
-    uint32_t ro[D], par[V];
+    typename PL::Ref ro[D];
+    uint32_t par[V];
     uint32_t sg[V];  // the signs of Q: edge k's in bit D - 1 - k (a word per codeword, not one per edge)
 #pragma unroll
     for (int v = 0; v < V; v++) sg[v] = par[v] = 0;
 #pragma unroll
     for (int k = 0; k < D; k++) {
-        uint32_t ao;
-        edge_at<V, MsgT>(ed[k], p, ao, ro[k]);
+        typename PL::Ref ao;
+        edge_at<MsgT>(ed[k], p, ao, ro[k]);
         T ap = mem.app(ao);
         const T n = mem.msg(ro[k]);
         T q = B2 ? vfma(ap, vset(T(), kSLog2e), n) : vadd(ap, n);
@@ -203,7 +214,7 @@ __device__ __forceinline__ void check_narrow(const int4 *__restrict__ ed, const 
         }
         T n = neg_mag<B2>(al, be);
         each(n, [&](float &x, int v) { x = __uint_as_float(__float_as_uint(x) & ~((sg[v] << (32 - D + k)) & kSign)); });
-        if (p.own) mem.put(ro[k], n);
+        mem.put(p, ro[k], n);
         if (k == 0) {
             pb = d[0];
         } else if (k < D - 1) {
@@ -269,8 +280,8 @@ struct Const {
 };
 
 // Degree 9..12: the factors held in registers between the passes.
-template <int V, typename MsgT, bool B2, bool HC, typename MEM>
-__device__ __forceinline__ void check_12(int dc, const int4 *__restrict__ ed, const MEM mem, const Place<V> &p,
+template <int V, typename MsgT, bool B2, bool HC, typename MEM, typename PL>
+__device__ __forceinline__ void check_12(int dc, const int4 *__restrict__ ed, const MEM mem, const PL &p,
                                          float Xb, float Pb, uint32_t (&pbad)[V])
 {
     using T = VT<V>;
@@ -282,8 +293,8 @@ __device__ __forceinline__ void check_12(int dc, const int4 *__restrict__ ed, co
     for (int k = 0; k < 12; k++) {
         d[k] = vset(T(), 0.0f);
         if (k < 9 || k < dc) {
-            uint32_t ao, ro;
-            edge_at<V, MsgT>(ed[k], p, ao, ro);
+            typename PL::Ref ao, ro;
+            edge_at<MsgT>(ed[k], p, ao, ro);
             T ap = mem.app(ao);
             const T n = mem.msg(ro);
             T q = B2 ? vfma(ap, vset(T(), kSLog2e), n) : vadd(ap, n);
@@ -316,9 +327,9 @@ __device__ __forceinline__ void check_12(int dc, const int4 *__restrict__ ed, co
 #pragma unroll
         for (int v = 0; v < V; v++) s8[v] = sg[v] << (8 * g);
         auto put = [&](int i, T x) {
-            uint32_t ao, ro;
-            edge_at<V, MsgT>(ed[8 * g + i], p, ao, ro);
-            if (p.own) mem.put(ro, x);
+            typename PL::Ref ao, ro;
+            edge_at<MsgT>(ed[8 * g + i], p, ao, ro);
+            mem.put(p, ro, x);
         };
         if (g == 0)
             group_out<true, B2, V>(8, e, ga[1], gb[1], s8, put);
@@ -334,8 +345,8 @@ __device__ __forceinline__ void check_12(int dc, const int4 *__restrict__ ed, co
 // mixed-code launch overflow the instruction cache (its share of stalls was 1.6 per issue).
 // One codeword per thread, the form of small batches, unrolls G groups, whose loads then
 // overlap.
-template <int G, int V, typename MsgT, bool B2, bool HC, typename MEM>
-__device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, const MEM mem, const Place<V> &p,
+template <int G, int V, typename MsgT, bool B2, bool HC, typename MEM, typename PL>
+__device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, const MEM mem, const PL &p,
                                            float Xb, float Pb, uint32_t (&pbad)[V])
 {
     constexpr bool HOLD = G == 2, INPLACE = !HOLD && sizeof(MsgT) == sizeof(float);
@@ -356,9 +367,9 @@ __device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, 
 #pragma unroll
         for (int k = 0; k < 8 * GM; k++) held[k] = zero;
     }
-    auto q_of = [&](int k, uint32_t &ro, bool first) -> T {
-        uint32_t ao;
-        edge_at<V, MsgT>(ed[k], p, ao, ro);
+    auto q_of = [&](int k, typename PL::Ref &ro, bool first) -> T {
+        typename PL::Ref ao;
+        edge_at<MsgT>(ed[k], p, ao, ro);
         T ap = mem.app(ao);
         const T n = mem.msg(ro);
         if (first) each(ap, [&](float x, int v) { par[v] ^= __float_as_uint(x); });
@@ -370,12 +381,12 @@ __device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, 
 #pragma unroll
         for (int i = 0; i < 8; i++) {
             if (!FULL && k0 + i >= dc) break;
-            uint32_t ro;
+            typename PL::Ref ro;
             T q = q_of(k0 + i, ro, true);
             each(q, [&](float x, int v) { sg[v] = __funnelshift_l(__float_as_uint(x), sg[v], 1); });
             const T d = form_d<B2, HC>(q, Xb, Pb);
             if constexpr (HOLD) held[k0 + i] = d;
-            if (INPLACE && p.own) mem.put_word(ro, d);
+            if constexpr (INPLACE) mem.put_word(p, ro, d);
             if (i == 0) {
                 b = d;
             } else {
@@ -402,18 +413,18 @@ __device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, 
             pb = vfma(b1, ga[h], vmul(a1, gb[h]));
         }
         T d[8];
-        uint32_t ro[8];
+        typename PL::Ref ro[8];
 #pragma unroll
         for (int i = 0; i < 8; i++) {
             d[i] = zero;
-            ro[i] = 0;
+            ro[i] = typename PL::Ref();
         }
 #pragma unroll
         for (int i = 0; i < 8; i++) {
             if (!FULL && k0 + i >= dc) break;
             if constexpr (INPLACE || HOLD) {
-                uint32_t ao;
-                edge_at<V, MsgT>(ed[k0 + i], p, ao, ro[i]);
+                typename PL::Ref ao;
+                edge_at<MsgT>(ed[k0 + i], p, ao, ro[i]);
                 if constexpr (HOLD)
                     d[i] = held[k0 + i];
                 else
@@ -423,7 +434,7 @@ __device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, 
             }
         }
         group_out<FULL, B2, V>(dc - k0, d, pa, pb, sg, [&](int i, T x) {
-            if (p.own) mem.put(ro[i], x);
+            mem.put(p, ro[i], x);
         });
 #pragma unroll
         for (int v = 0; v < V; v++) sg[v] <<= 8;

@@ -19,12 +19,18 @@
 // block, edge (b, r) of the owned block b at (b - first owned block) * Z + (r + s) mod Z;
 // posteriors at (place of column j) * Z + c.
 //
-// Threads: W row groups of whole warps; thread r of row group w owns row r of every W-th owned
-// block row and position r of every W-th owned column, both in ascending degree, so that a
-// warp runs one straight-line body at a time (flood_check.cuh).  The table entries hold
-// complete shared::cluster addresses (own CTA or the other), so an operand in either CTA costs one add.
-// Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB: 6727 -> 5378 us per launch,
-// 71 -> 55 warp instructions per edge update (bound by instruction issue, 65 %).
+// Check-node threads: W row groups of whole warps; thread r of a row group owns rows r and
+// r + ceil(Z / 2) of the block rows that fall to its group in ascending degree, so that a warp runs
+// one straight-line body at a time (flood_check.cuh) with two rows' arithmetic packed and one read
+// of each edge descriptor.  One CTA has several times more rows than threads, so that pairing them
+// costs no parallelism.  Variable-node threads: W4 groups; a thread owns four consecutive positions
+// of every W4-th column, one access per block (where Z is a multiple of 4; else its two rows'
+// positions).  The table entries hold complete shared::cluster addresses (own CTA or the other),
+// so an operand in either CTA costs one add.
+// Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB, per launch, and warp
+// instructions per edge update (both phases): one row and one position per thread 5378 us, 57; two
+// rows 5087 us, 49; and four positions 4706 us, 43.  Bound by instruction issue (56 %) and the waits
+// at the two cluster barriers of a round (18 % of a warp's time).
 #include <string.h>
 
 #include "flood_check.cuh"
@@ -44,7 +50,10 @@ struct ClusterArgs {
     int n_req;
     // from here (neither loaded nor divided in the kernel) these are known to be warp-uniform: the
     // code's sizes, and W row groups of WT threads
-    int Z, N, W, WT;
+    int Z, H, N, W, WT;
+    // the variable-node phase in quads: W4 groups of WT4 threads, wt4 = the warps' worth of quads
+    // of a column (W4 = 0: Z is no multiple of 4)
+    int W4, WT4, wt4, wide_L;
     int64_t n_items;
     unsigned long long *next;
     int row_split[CLUSTER_CTAS + 1];  // block rows [row_split[q], row_split[q+1]) belong to CTA q
@@ -85,6 +94,20 @@ __device__ __forceinline__ float cl_ld(const __half *, uint32_t addr)
     asm volatile("ld.shared::cluster.u16 %0, [%1];" : "=h"(v) : "r"(addr));
     return __half2float(__ushort_as_half(v));
 }
+// four consecutive messages (aligned)
+__device__ __forceinline__ void cl_ld4(const float *, uint32_t addr, float2 (&m)[2])
+{
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(m[0].x), "=f"(m[0].y), "=f"(m[1].x), "=f"(m[1].y)
+                 : "r"(addr));
+}
+__device__ __forceinline__ void cl_ld4(const __half *, uint32_t addr, float2 (&m)[2])
+{
+    uint32_t u, v;
+    asm volatile("ld.shared::cluster.v2.b32 {%0, %1}, [%2];" : "=r"(u), "=r"(v) : "r"(addr));
+    m[0] = __half22float2(*reinterpret_cast<const __half2 *>(&u));
+    m[1] = __half22float2(*reinterpret_cast<const __half2 *>(&v));
+}
 __device__ __forceinline__ void cl_st(uint32_t addr, int x)
 {
     asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(x) : "memory");
@@ -104,15 +127,56 @@ __host__ __device__ inline int cl_owner(const int *split, int x)
     return q;
 }
 
-// A check's operands: the posterior at a shared::cluster address, the message in the own CTA.
+// A thread's place: two rows r and s = r + H of its block row (H = ceil(Z / 2)), plain and less
+// one block.  An idle lane of a group's last warp repeats the last rows, and row Z (odd Z) is row
+// Z - 1 once more; neither stores anything.
+struct PairPlace {
+    struct Ref {  // the two rows' operands
+        uint32_t x, y;
+    };
+    int r, rw, s, sw;
+    bool own, own2;
+};
+template <typename MsgT>
+__device__ __forceinline__ void edge_at(const int4 &e, const PairPlace &p, PairPlace::Ref &ao, PairPlace::Ref &ro)
+{
+    const int t = p.r >= e.z ? p.rw : p.r, u = p.s >= e.z ? p.sw : p.s;
+    ao = {(uint32_t)(e.x + 4 * t), (uint32_t)(e.x + 4 * u)};
+    ro = {(uint32_t)(e.y + (int)sizeof(MsgT) * t), (uint32_t)(e.y + (int)sizeof(MsgT) * u)};
+}
+
+// Two checks' operands: the posteriors at shared::cluster addresses, the messages in the own CTA.
 template <typename MsgT>
 struct ClusterMem {
+    using Ref = PairPlace::Ref;
     char *sm;
-    __device__ __forceinline__ float app(uint32_t o) const { return cl_ld((const float *)nullptr, o); }
-    __device__ __forceinline__ float msg(uint32_t o) const { return Sm<MsgT, 1>::ld(sm + o); }
-    __device__ __forceinline__ void put(uint32_t o, float x) const { Sm<MsgT, 1>::st(sm + o, x); }
-    __device__ __forceinline__ float word(uint32_t o) const { return Sm<float, 1>::ld(sm + o); }
-    __device__ __forceinline__ void put_word(uint32_t o, float x) const { Sm<float, 1>::st(sm + o, x); }
+    __device__ __forceinline__ float2 app(Ref o) const
+    {
+        return make_float2(cl_ld((const float *)nullptr, o.x), cl_ld((const float *)nullptr, o.y));
+    }
+    __device__ __forceinline__ float2 msg(Ref o) const
+    {
+        return make_float2(Sm<MsgT, 1>::ld(sm + o.x), Sm<MsgT, 1>::ld(sm + o.y));
+    }
+    __device__ __forceinline__ void put(const PairPlace &p, Ref o, float2 x) const
+    {
+        if constexpr (sizeof(MsgT) == 2) {
+            const __half2 h = __floats2half2_rn(x.x, x.y);
+            if (p.own) *reinterpret_cast<__half *>(sm + o.x) = __low2half(h);
+            if (p.own2) *reinterpret_cast<__half *>(sm + o.y) = __high2half(h);
+        } else {
+            put_word(p, o, x);
+        }
+    }
+    __device__ __forceinline__ float2 word(Ref o) const
+    {
+        return make_float2(Sm<float, 1>::ld(sm + o.x), Sm<float, 1>::ld(sm + o.y));
+    }
+    __device__ __forceinline__ void put_word(const PairPlace &p, Ref o, float2 x) const
+    {
+        if (p.own) Sm<float, 1>::st(sm + o.x, x.x);
+        if (p.own2) Sm<float, 1>::st(sm + o.y, x.y);
+    }
 };
 
 // Row r of every W-th owned block row from list position i, in ascending degree (see rows_of of
@@ -120,7 +184,7 @@ struct ClusterMem {
 template <int CLS, int DMAX, typename MsgT, bool HC>
 __device__ __forceinline__ void cl_rows(const uint8_t *rend, const int4 *__restrict__ tab,
                                         const int32_t *__restrict__ rows, const ClusterMem<MsgT> mem,
-                                        const Place<1> &p, float Xb, float Pb, uint32_t (&pbad)[1], int i, int step,
+                                        const PairPlace &p, float Xb, float Pb, uint32_t (&pbad)[2], int i, int step,
                                         int W2)
 {
     constexpr int D = cl_class_degree(CLS);
@@ -129,64 +193,119 @@ __device__ __forceinline__ void cl_rows(const uint8_t *rend, const int4 *__restr
         for (; i < end; i += step, step = W2 - step) {
             const int hd = rows[i];
             if constexpr (D <= 8)
-                check_narrow<D, 1, MsgT, false, HC>(tab + (hd >> 8), mem, p, Xb, Pb, pbad);
+                check_narrow<D, 2, MsgT, false, HC>(tab + (hd >> 8), mem, p, Xb, Pb, pbad);
             else if constexpr (D == 12)
-                check_12<1, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
+                check_12<2, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
             else
-                check_wide<D / 8, 1, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
+                check_wide<0, 2, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
         }
         if constexpr (CLS + 1 < CL_CLASSES)
             cl_rows<CLS + 1, DMAX, MsgT, HC>(rend, tab, rows, mem, p, Xb, Pb, pbad, i, step, W2);
     }
 }
 
-// Position r of every W-th owned column from list position i, in ascending degree: APP = L + the
-// column's messages in block-row order.  Lr: channel values at position r of block column 0;
-// rb: the thread's byte offset in a block of messages; A: its place in the posteriors.
-constexpr int kClChunk = 4;  // columns whose channel values a thread requests at once
-template <int DV, typename MsgT>
+// The positions of a column that a thread of the variable-node phase owns, and their values in
+// packed pairs.  rb: byte offsets in a block of messages; L: channel values of block column 0;
+// A: posteriors of place 0.
+//   VarPair  positions r and s = r + H, the thread's rows of the check-node phase
+//   VarQuad  four consecutive positions, whose messages and posteriors are one access each
+//            (Z a multiple of 4)
+template <typename MsgT>
+struct VarPair {
+    static constexpr int NV = 1;
+    const float *L, *L2;
+    uint32_t rb, rb2;
+    float *A, *A2;
+    bool own, own2;
+    __device__ __forceinline__ void channel(int o, float2 (&x)[1]) const { x[0] = make_float2(__ldg(L + o), __ldg(L2 + o)); }
+    __device__ __forceinline__ void add(float2 (&s)[1], int addr) const
+    {
+        const float2 m = make_float2(cl_ld((const MsgT *)nullptr, rb + (uint32_t)addr),
+                                     cl_ld((const MsgT *)nullptr, rb2 + (uint32_t)addr));
+        s[0] = __ffma2_rn(m, make_float2(-1.0f, -1.0f), s[0]);
+    }
+    __device__ __forceinline__ void put(int a, const float2 (&s)[1]) const
+    {
+        if (own) A[a] = s[0].x + 0.0f;  // -0 -> +0: the sign bit is the decision
+        if (own2) A2[a] = s[0].y + 0.0f;
+    }
+};
+template <typename MsgT>
+struct VarQuad {
+    static constexpr int NV = 2;
+    const float *L;
+    uint32_t rb;
+    float *A;
+    bool own, wide;  // wide: the channel values are 16-byte aligned
+    __device__ __forceinline__ void channel(int o, float2 (&x)[2]) const
+    {
+        float4 v;
+        if (wide)
+            v = __ldg(reinterpret_cast<const float4 *>(L + o));
+        else
+            v = make_float4(__ldg(L + o), __ldg(L + o + 1), __ldg(L + o + 2), __ldg(L + o + 3));
+        x[0] = make_float2(v.x, v.y);
+        x[1] = make_float2(v.z, v.w);
+    }
+    __device__ __forceinline__ void add(float2 (&s)[2], int addr) const
+    {
+        float2 m[2];
+        cl_ld4((const MsgT *)nullptr, rb + (uint32_t)addr, m);
+#pragma unroll
+        for (int i = 0; i < 2; i++) s[i] = __ffma2_rn(m[i], make_float2(-1.0f, -1.0f), s[i]);
+    }
+    __device__ __forceinline__ void put(int a, const float2 (&s)[2]) const
+    {
+        const float2 z = make_float2(0.0f, 0.0f), u = __fadd2_rn(s[0], z), v = __fadd2_rn(s[1], z);
+        if (own) *reinterpret_cast<float4 *>(A + a) = make_float4(u.x, u.y, v.x, v.y);
+    }
+};
+
+// A thread's positions of every W-th owned column from list position i, in ascending degree:
+// APP = L + the column's messages in block-row order.
+constexpr int kClChunk = 2;  // columns whose channel values a thread requests at once
+template <int DV, typename VAR>
 __device__ __forceinline__ void cl_cols(const uint8_t *cend, const int4 *__restrict__ ctab,
-                                        const int4 *__restrict__ tab, const int32_t *__restrict__ cols,
-                                        const float *__restrict__ Lr, uint32_t rb, float *A, int Z, bool own, int i,
-                                        int W)
+                                        const int4 *__restrict__ tab, const int32_t *__restrict__ cols, const VAR p,
+                                        int Z, int i, int W)
 {
     const int end = cend[DV - 1];
-    auto add = [&](float s, int addr) { return s - cl_ld((const MsgT *)nullptr, rb + (uint32_t)addr); };
     for (; i < end;) {
-        float lv[kClChunk];
+        float2 s[kClChunk][VAR::NV];
         int jc[kClChunk];
 #pragma unroll
         for (int c = 0; c < kClChunk; c++) {
-            lv[c] = 0.0f;
+#pragma unroll
+            for (int v = 0; v < VAR::NV; v++) s[c][v] = make_float2(0.0f, 0.0f);
             jc[c] = 0;
             if (c == 0 || i + c * W < end) {
                 jc[c] = cols[i + c * W];
-                lv[c] = __ldg(Lr + (jc[c] & 255) * Z);
+                p.channel((jc[c] & 255) * Z, s[c]);
             }
         }
 #pragma unroll
         for (int c = 0; c < kClChunk; c++) {
             if (c == 0 || i < end) {
                 const int4 o = ctab[i];
-                float s = add(lv[c], o.x);
-                if constexpr (DV > 1) s = add(s, o.y);
-                if constexpr (DV > 2) s = add(s, o.z);
-                if constexpr (DV == 4) s = add(s, o.w);
+                p.add(s[c], o.x);
+                if constexpr (DV > 1) p.add(s[c], o.y);
+                if constexpr (DV > 2) p.add(s[c], o.z);
+                if constexpr (DV == 4) p.add(s[c], o.w);
                 if constexpr (DV == 5) {
                     const int4 *m = tab + (o.w >> 8);
                     for (int k = o.w & 255; k > 0; k -= 4, m++) {
-                        s = add(s, m->x);
-                        if (k > 1) s = add(s, m->y);
-                        if (k > 2) s = add(s, m->z);
-                        if (k > 3) s = add(s, m->w);
+                        p.add(s[c], m->x);
+                        if (k > 1) p.add(s[c], m->y);
+                        if (k > 2) p.add(s[c], m->z);
+                        if (k > 3) p.add(s[c], m->w);
                     }
                 }
-                if (own) A[(jc[c] >> 8) * Z] = s + 0.0f;  // -0 -> +0: the sign bit is the decision
+                p.put((jc[c] >> 8) * Z, s[c]);
                 i += W;
             }
         }
     }
-    if constexpr (DV < 5) cl_cols<DV + 1, MsgT>(cend, ctab, tab, cols, Lr, rb, A, Z, own, i, W);
+    if constexpr (DV < 5) cl_cols<DV + 1>(cend, ctab, tab, cols, p, Z, i, W);
 }
 
 // Shared memory ahead of the posterior array (flags, codeword, tables; see the kernel).
@@ -208,7 +327,7 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
     extern __shared__ __align__(16) unsigned char smem[];
     const int q = (int)(blockIdx.x % CLUSTER_CTAS);  // the rank in the cluster (one-dimensional grid)
     const int tid = threadIdx.x, nth = blockDim.x;
-    const int Z = a.Z, N = a.N;
+    const int Z = a.Z, H = a.H, N = a.N;
     const float Xb = a.X * kSLog2e, Pb = s_phi_b2(a.X);  // the clamp [phi(X), X] in base-2 units
 
     // bookkeeping: [0] bad flags (2, alternating by round; a check of either CTA sets both
@@ -257,10 +376,13 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
     const uint32_t flag_0 = cl_map(flags, 0), flag_1 = cl_map(flags, 1);
     // row groups of WT threads; when a row needs more threads than the CTA has, one group whose
     // threads take positions ru, ru + nth, ...
-    const int wt = (Z + 31) & ~31, W = a.W, WT = a.WT;
+    const int wt = (H + 31) & ~31, W = a.W, WT = a.WT;
     const int w0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT));  // (a warp reduction: known to be uniform)
     const int ru = tid - w0 * WT;
     const bool works = w0 < W;
+    // the variable-node phase's groups (VarQuad); threads past the last group find no column
+    const int WT4 = a.WT4, w4t = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT4));
+    const int ru4 = tid - w4t * WT4, w4 = w4t < a.W4 ? w4t : NB_MAX;
     const uint32_t cw0 = cl_map(cwp, 0);
     cl_sync();  // tables built in every CTA before any remote access
 
@@ -302,18 +424,18 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             uint32_t bad = 0;
             if (works)
                 for (int rr = 0; rr < wt; rr += WT) {
-                    Place<1> p;
+                    PairPlace p;
                     const int r = rr + ru;
-                    p.own = r < Z;
-                    p.r = p.own ? r : Z - 1;
-                    p.a0 = 4u * (uint32_t)p.r;
-                    p.a1 = p.a0 - 4u * (uint32_t)Z;
-                    p.r0 = (uint32_t)SR * (uint32_t)p.r;
-                    p.r1 = p.r0 - (uint32_t)SR * (uint32_t)Z;
-                    uint32_t pbad[1] = {0};
+                    p.own = r < H;
+                    p.r = p.own ? r : H - 1;
+                    p.own2 = p.own && p.r + H < Z;
+                    p.s = p.r + H < Z ? p.r + H : Z - 1;
+                    p.rw = p.r - Z;
+                    p.sw = p.s - Z;
+                    uint32_t pbad[2] = {0, 0};
                     cl_rows<0, DMAX, MsgT, HC>(a.rend[q], tab, rows, ClusterMem<MsgT>{reinterpret_cast<char *>(smem)},
                                                p, Xb, Pb, pbad, w0, 2 * (W - w0) - 1, 2 * W);
-                    if (p.own) bad |= pbad[0];
+                    bad |= pbad[0] | pbad[1];
                 }
             if (__any_sync(0xffffffffu, (bad & kSign) != 0) && (tid & 31) == 0) {
                 cl_st(flag_0 + 4 * (tr & 1), 1);
@@ -324,12 +446,21 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             const bool conv = tr >= 1 && a.early_exit && flags[tr & 1] == 0;
             if (!__any_sync(0xffffffffu, conv)) {
                 // ---------------- variable-node phase over the owned variables
-                if (works)
-                    for (int rr = 0; rr < wt; rr += WT) {
-                        const int r = rr + ru, rc = r < Z ? r : Z - 1;
-                        cl_cols<1, MsgT>(a.cend[q], ctab, tab, cols, L + rc, (uint32_t)(SR * rc), app + rc, Z, r < Z,
-                                         w0, W);
+                if (a.W4 > 0) {
+                    const bool wide = a.wide_L;
+                    for (int qq = 0; qq < a.wt4; qq += a.WT4) {
+                        const int x = qq + ru4, xc = 4 * x < Z ? 4 * x : Z - 4;
+                        const VarQuad<MsgT> v{L + xc, (uint32_t)(SR * xc), app + xc, 4 * x < Z, wide};
+                        cl_cols<1>(a.cend[q], ctab, tab, cols, v, Z, w4, a.W4);
                     }
+                } else if (works) {
+                    for (int rr = 0; rr < wt; rr += WT) {
+                        const int r = rr + ru, rc = r < H ? r : H - 1, sc = rc + H < Z ? rc + H : Z - 1;
+                        const VarPair<MsgT> v{L + rc,   L + sc,   (uint32_t)(SR * rc), (uint32_t)(SR * sc),
+                                              app + rc, app + sc, r < H,               r < H && rc + H < Z};
+                        cl_cols<1>(a.cend[q], ctab, tab, cols, v, Z, w0, W);
+                    }
+                }
                 t++;
             }
             done = __any_sync(0xffffffffu, conv || t >= a.max_iter);
@@ -498,9 +629,15 @@ static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, con
         __atomic_store_n(&cached[dev], clusters, __ATOMIC_RELAXED);
     }
     if ((int64_t)clusters > n_cw) clusters = (int)n_cw;
-    const int wt = (a.Z + 31) & ~31, nth = cl_threads<DMAX>();
+    const int wt = (a.H + 31) & ~31, nth = cl_threads<DMAX>();
     a.W = wt <= nth ? nth / wt : 1;
     a.WT = wt <= nth ? wt : nth;
+    a.wt4 = (a.Z / 4 + 31) & ~31;
+    a.WT4 = a.Z % 4 ? 32 : a.wt4 <= nth ? a.wt4 : nth;
+    a.W4 = a.Z % 4 ? 0 : nth / a.WT4;
+    a.wide_L = a.N % 4 == 0;
+    for (int i = 0; i < a.n_req; i++)
+        if (reinterpret_cast<uintptr_t>(a.reqs[i].llr) & 15) a.wide_L = 0;
     LaunchScope ls(F_SLOTS, s);
     k_flood_cluster<DMAX, MsgT, HC><<<(unsigned)(clusters * CLUSTER_CTAS), cl_threads<DMAX>(), smem, s>>>(d, a);
     return cudaGetLastError();
@@ -538,6 +675,7 @@ cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     if (items == 0) return cudaSuccess;
     a.n_items = items;
     a.Z = h.Z;
+    a.H = (h.Z + 1) / 2;
     a.N = h.N;
     a.next = static_cast<unsigned long long *>(counter);
     a.max_iter = p.max_iter;

@@ -66,3 +66,31 @@ def test_against_oracle_and_across_forms(cuda_dev, name, form):
     big = decode(code, form, L, cuda_dev, max_iter=9)
     for a, b in zip(small, big):
         assert np.array_equal(a, b[:n_small]), name
+
+
+@pytest.mark.parametrize("form", ["cluster_f32", "cluster_f16"])
+@pytest.mark.parametrize("name", list(CODES))
+def test_cluster_against_oracle(cuda_dev, name, form):
+    """Two rows per thread (odd Z: a last row without a partner), columns in quads where Z is a
+    multiple of 4 (channel values on a 16-byte boundary or not)."""
+    B, Z = CODES[name]
+    code, oc = ldpc.Code(B, Z), O.QCCode(B, Z)
+    n = 200  # more codewords than clusters
+    rng = np.random.default_rng(11)
+    L = (2.5 + 2.2 * rng.standard_normal((n, code.N))).astype(np.float32)
+    L[::7, ::5] = 0.0
+    for T in (1, 2):
+        app, bits, iters = decode(code, form, L, cuda_dev, max_iter=T, early_exit=0)
+        if form == "cluster_f32":
+            ref, _, _ = oc.spa_flood(L, T, early_exit=False)
+            assert rel_err(app, ref).max() <= FP32_TOL, (name, T)
+        elif T == 1:
+            ref, band = binary16_band(oc, False, L, 1, 4)
+            assert_binary16_close(app, ref, band, strict=True, what=name)
+        assert np.array_equal(bits, app < 0) and (iters == T).all()
+    odd = torch.empty(L.size + 1, device=cuda_dev)[1:].view(n, code.N)
+    odd.copy_(torch.from_numpy(L))
+    a = ldpc.decode(code, ldpc.params_for(form, max_iter=9), odd, app=True)
+    b = ldpc.decode(code, ldpc.params_for(form, max_iter=9), torch.from_numpy(L).to(cuda_dev), app=True)
+    for x, y in zip(a, b):
+        assert torch.equal(x, y), name
