@@ -195,7 +195,7 @@ void flood_build_table(CodeDev &h, int msg, int V, int4 *tab)
                 auto off = [&](int i) { return i < dv ? SR * (h.colent[i0 + i] >> 16) * h.Z : 0; };
                 const int take = dv > 4 ? 3 : 4;
                 col[nc] = make_int4(off(0), off(1), off(2), dv > 4 ? (nx << 8) | (dv - 3) : off(3));
-                cols[nc++] = j;
+                cols[nc++] = j * h.Z;
                 for (int i = take; i < dv; i += 4) tab[nx++] = make_int4(off(i), off(i + 1), off(i + 2), off(i + 3));
             }
         h.cend[c - 1] = (uint8_t)nc;

@@ -50,7 +50,7 @@ struct FloodReq {
 //     their number).  Messages are stored at the variable's position inside the block, so the
 //     variable-node phase needs no wrap
 //   32-bit words (from t_row): per block row in ascending degree the index of its first edge
-//     descriptor << 8 | its degree; per block column in ascending degree its number
+//     descriptor << 8 | its degree; per block column in ascending degree its first variable
 struct FloodArgs {
     unsigned long long *next;  // [n_groups] work counters, zero at launch; null: one group, all codewords resident
     int n_groups;
