@@ -39,7 +39,8 @@ _CSRC = os.path.join(ROOT, "paper_1812_06545_gb300", "csrc")
 # the files each profiled kernel is compiled from: a stored ncu traffic figure is used only
 # while their combined hash is unchanged
 CN_SOURCES = ("flood_kernels.cu", "ldpc_internal.h")
-SLOTS_SOURCES = ("flood_slots.cu", "flood_slots_kernel.cuh", "flood_slots.h", "slot_common.cuh", "ldpc_internal.h")
+SLOTS_SOURCES = ("flood_slots.cu", "flood_slots_kernel.cuh", "flood_slots.h", "flood_check.cuh", "slot_common.cuh",
+                 "ldpc_internal.h")
 
 
 def strip_comments(src: str) -> str:

@@ -21,10 +21,10 @@
 //   barrier
 //   decision           a codeword with >= 1 iteration done and no unsatisfied check has
 //                      converged: its APP (from that iteration) is final
+//   output             converged codewords write bits / APP / iteration count; one thread per
+//                      slot takes the next codeword index from the global work counter
 //   variable-node phase the others: APP = L + sum of the new R (block-row order,
-//                      deterministic); a codeword reaching max_iter is final
-//   output             final codewords write bits / APP / iteration count; one thread per slot
-//                      takes the next codeword index from the global work counter
+//                      deterministic); a codeword reaching max_iter is final and written out
 //   barrier
 //   refill             (only after an output) APP = L, R = 0 of the new codeword; barrier
 // Codewords therefore leave as soon as they converge and slots are refilled at once: early
@@ -43,6 +43,7 @@
 //   two per thread and barrier groups of three slots                        790 us FP16
 //   two per thread, two row groups, one slot per barrier       964            679
 //   + degree-ordered loops, uniform control, signs in a word   906            645
+//   + output ahead of the variable-node phase                  887            629
 // FP32: 18 warps of 3 thread slots (57 warp instructions per edge of two codewords, was 2 x 40);
 // FP16: 24 warps of 4 (six slots of one row group each, 18 warps, took 718).
 #include <string.h>
