@@ -24,13 +24,15 @@
 // one straight-line body at a time (flood_check.cuh) with two rows' arithmetic packed and one read
 // of each edge descriptor.  One CTA has several times more rows than threads, so that pairing them
 // costs no parallelism.  Variable-node threads: W4 groups; a thread owns four consecutive positions
-// of every W4-th column, one access per block (where Z is a multiple of 4; else its two rows'
-// positions).  The table entries hold complete shared::cluster addresses (own CTA or the other),
+// of its group's columns, one access per block (where Z is a multiple of 4; else its two rows'
+// positions).  Rows and columns are dealt to the groups by weight on the host, because a phase ends
+// at a cluster barrier.  The table entries hold complete shared::cluster addresses (own CTA or the other),
 // so an operand in either CTA costs one add.
 // Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB, per launch, and warp
 // instructions per edge update (both phases): one row and one position per thread 5378 us, 57; two
-// rows 5087 us, 49; and four positions 4706 us, 43.  Bound by instruction issue (56 %) and the waits
-// at the two cluster barriers of a round (18 % of a warp's time).
+// rows 5087 us, 49; and four positions 4706 us, 43; dealt by weight (not back and forth) 4609 us.
+// Bound by instruction issue (58 %) and the waits at the two cluster barriers of a round (15 % of a
+// warp's time).
 #include <string.h>
 
 #include "flood_check.cuh"
@@ -43,6 +45,8 @@ __host__ __device__ constexpr int cl_class_degree(int c)
 {
     return c < 7 ? c + 2 : c == 7 ? 12 : c == 8 ? 16 : c == 9 ? 24 : 32;
 }
+
+constexpr int CL_GROUPS = 24;  // groups of whole warps a CTA can have
 
 // One launch decodes every codeword of up to MULTI_MAX_REQS requests of one code: the codewords
 // are the items of one work sequence (request i's are items item0 .. item0 + n_cw - 1).
@@ -60,10 +64,12 @@ struct ClusterArgs {
     int ncols[CLUSTER_CTAS];          // block columns CTA q holds the posteriors of
     int col_owner[NB_MAX];            // owner of block column j
     int col_slot[NB_MAX];             // its place among the owner's columns
-    // CTA q's rows and columns in ascending degree, the ends of their degree classes, the
-    // rows' first edge descriptors, and the elements of its table
+    // CTA q's rows and columns group by group (a group's share in ascending degree), where each
+    // group's share starts and the ends of its degree classes, the rows' first edge
+    // descriptors, and the elements of the CTA's table
     uint8_t row_list[CLUSTER_CTAS][MB_MAX], col_list[CLUSTER_CTAS][NB_MAX];
-    uint8_t rend[CLUSTER_CTAS][CL_CLASSES], cend[CLUSTER_CTAS][5];
+    uint8_t rstart[CLUSTER_CTAS][CL_GROUPS], cstart[CLUSTER_CTAS][CL_GROUPS];
+    uint8_t rend[CLUSTER_CTAS][CL_GROUPS][CL_CLASSES], cend[CLUSTER_CTAS][CL_GROUPS][5];
     uint16_t row_e0[CLUSTER_CTAS][MB_MAX], col_x0[CLUSTER_CTAS][NB_MAX];
     int n_edge[CLUSTER_CTAS], n_tab[CLUSTER_CTAS];
     int off_app, off_r;  // posteriors and messages, bytes from the start of shared memory
@@ -179,18 +185,17 @@ struct ClusterMem {
     }
 };
 
-// Row r of every W-th owned block row from list position i, in ascending degree (see rows_of of
-// the slot decoder).
+// The thread's two rows of its group's block rows from list position i, in ascending degree (see
+// rows_of of the slot decoder).
 template <int CLS, int DMAX, typename MsgT, bool HC>
 __device__ __forceinline__ void cl_rows(const uint8_t *rend, const int4 *__restrict__ tab,
                                         const int32_t *__restrict__ rows, const ClusterMem<MsgT> mem,
-                                        const PairPlace &p, float Xb, float Pb, uint32_t (&pbad)[2], int i, int step,
-                                        int W2)
+                                        const PairPlace &p, float Xb, float Pb, uint32_t (&pbad)[2], int i)
 {
     constexpr int D = cl_class_degree(CLS);
     if constexpr (D <= DMAX) {
         const int end = rend[CLS];
-        for (; i < end; i += step, step = W2 - step) {
+        for (; i < end; i++) {
             const int hd = rows[i];
             if constexpr (D <= 8)
                 check_narrow<D, 2, MsgT, false, HC>(tab + (hd >> 8), mem, p, Xb, Pb, pbad);
@@ -200,7 +205,7 @@ __device__ __forceinline__ void cl_rows(const uint8_t *rend, const int4 *__restr
                 check_wide<0, 2, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
         }
         if constexpr (CLS + 1 < CL_CLASSES)
-            cl_rows<CLS + 1, DMAX, MsgT, HC>(rend, tab, rows, mem, p, Xb, Pb, pbad, i, step, W2);
+            cl_rows<CLS + 1, DMAX, MsgT, HC>(rend, tab, rows, mem, p, Xb, Pb, pbad, i);
     }
 }
 
@@ -261,13 +266,13 @@ struct VarQuad {
     }
 };
 
-// A thread's positions of every W-th owned column from list position i, in ascending degree:
+// A thread's positions of its group's columns from list position i, in ascending degree:
 // APP = L + the column's messages in block-row order.
 constexpr int kClChunk = 2;  // columns whose channel values a thread requests at once
 template <int DV, typename VAR>
 __device__ __forceinline__ void cl_cols(const uint8_t *cend, const int4 *__restrict__ ctab,
                                         const int4 *__restrict__ tab, const int32_t *__restrict__ cols, const VAR p,
-                                        int Z, int i, int W)
+                                        int Z, int i)
 {
     const int end = cend[DV - 1];
     for (; i < end;) {
@@ -278,8 +283,8 @@ __device__ __forceinline__ void cl_cols(const uint8_t *cend, const int4 *__restr
 #pragma unroll
             for (int v = 0; v < VAR::NV; v++) s[c][v] = make_float2(0.0f, 0.0f);
             jc[c] = 0;
-            if (c == 0 || i + c * W < end) {
-                jc[c] = cols[i + c * W];
+            if (c == 0 || i + c < end) {
+                jc[c] = cols[i + c];
                 p.channel((jc[c] & 255) * Z, s[c]);
             }
         }
@@ -301,11 +306,11 @@ __device__ __forceinline__ void cl_cols(const uint8_t *cend, const int4 *__restr
                     }
                 }
                 p.put((jc[c] >> 8) * Z, s[c]);
-                i += W;
+                i++;
             }
         }
     }
-    if constexpr (DV < 5) cl_cols<DV + 1>(cend, ctab, tab, cols, p, Z, i, W);
+    if constexpr (DV < 5) cl_cols<DV + 1>(cend, ctab, tab, cols, p, Z, i);
 }
 
 // Shared memory ahead of the posterior array (flags, codeword, tables; see the kernel).
@@ -380,9 +385,9 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
     const int w0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT));  // (a warp reduction: known to be uniform)
     const int ru = tid - w0 * WT;
     const bool works = w0 < W;
-    // the variable-node phase's groups (VarQuad); threads past the last group find no column
-    const int WT4 = a.WT4, w4t = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT4));
-    const int ru4 = tid - w4t * WT4, w4 = w4t < a.W4 ? w4t : NB_MAX;
+    // the variable-node phase's groups (VarQuad)
+    const int WT4 = a.WT4, w4 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT4));
+    const int ru4 = tid - w4 * WT4;
     const uint32_t cw0 = cl_map(cwp, 0);
     cl_sync();  // tables built in every CTA before any remote access
 
@@ -433,8 +438,9 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
                     p.rw = p.r - Z;
                     p.sw = p.s - Z;
                     uint32_t pbad[2] = {0, 0};
-                    cl_rows<0, DMAX, MsgT, HC>(a.rend[q], tab, rows, ClusterMem<MsgT>{reinterpret_cast<char *>(smem)},
-                                               p, Xb, Pb, pbad, w0, 2 * (W - w0) - 1, 2 * W);
+                    cl_rows<0, DMAX, MsgT, HC>(a.rend[q][w0], tab, rows,
+                                               ClusterMem<MsgT>{reinterpret_cast<char *>(smem)}, p, Xb, Pb, pbad,
+                                               a.rstart[q][w0]);
                     bad |= pbad[0] | pbad[1];
                 }
             if (__any_sync(0xffffffffu, (bad & kSign) != 0) && (tid & 31) == 0) {
@@ -451,14 +457,14 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
                     for (int qq = 0; qq < a.wt4; qq += a.WT4) {
                         const int x = qq + ru4, xc = 4 * x < Z ? 4 * x : Z - 4;
                         const VarQuad<MsgT> v{L + xc, (uint32_t)(SR * xc), app + xc, 4 * x < Z, wide};
-                        cl_cols<1>(a.cend[q], ctab, tab, cols, v, Z, w4, a.W4);
+                        if (w4 < a.W4) cl_cols<1>(a.cend[q][w4], ctab, tab, cols, v, Z, a.cstart[q][w4]);
                     }
                 } else if (works) {
                     for (int rr = 0; rr < wt; rr += WT) {
                         const int r = rr + ru, rc = r < H ? r : H - 1, sc = rc + H < Z ? rc + H : Z - 1;
                         const VarPair<MsgT> v{L + rc,   L + sc,   (uint32_t)(SR * rc), (uint32_t)(SR * sc),
                                               app + rc, app + sc, r < H,               r < H && rc + H < Z};
-                        cl_cols<1>(a.cend[q], ctab, tab, cols, v, Z, w0, W);
+                        cl_cols<1>(a.cend[q][w0], ctab, tab, cols, v, Z, a.cstart[q][w0]);
                     }
                 }
                 t++;
@@ -546,30 +552,71 @@ static size_t cl_plan(const CodeDev &h, int msg, ClusterArgs &a, size_t limit)
     for (int j = 0; j < h.nb; j++) a.col_slot[j] = a.ncols[a.col_owner[j]]++;
     int nmax = 0;
     for (int q = 0; q < CLUSTER_CTAS; q++) nmax = a.ncols[q] > nmax ? a.ncols[q] : nmax;
-    // the CTAs' lists in ascending degree, and the size of their tables
+    // groups of whole warps: W for two rows per thread, W4 for four positions (Z a multiple of 4;
+    // else the columns go to the row groups too)
+    const int nth = h.dc_max <= 12 ? cl_threads<12>() : cl_threads<32>();
+    a.Z = h.Z;
+    a.H = (h.Z + 1) / 2;
+    const int wt = (a.H + 31) & ~31;
+    a.W = wt <= nth ? nth / wt : 1;
+    a.WT = wt <= nth ? wt : nth;
+    a.wt4 = (a.Z / 4 + 31) & ~31;
+    a.WT4 = a.Z % 4 ? 32 : a.wt4 <= nth ? a.wt4 : nth;
+    a.W4 = a.Z % 4 ? 0 : nth / a.WT4;
+    // the CTAs' lists, and the size of their tables.  A phase ends at a cluster barrier, so its
+    // rows (columns) go to the groups by weight, heaviest first to the least loaded group
     size_t tables = cl_tables_bytes(h.nnz);
     for (int q = 0; q < CLUSTER_CTAS; q++) {
         int ne = 0, nr = 0, nc = 0;
-        for (int c = 0; c < CL_CLASSES; c++) {
-            for (int d = (c ? cl_class_degree(c - 1) : 0) + 1; d <= cl_class_degree(c); d++)
-                for (int l = a.row_split[q]; l < a.row_split[q + 1]; l++)
-                    if (h.rowptr[l + 1] - h.rowptr[l] == d) {
-                        a.row_e0[q][nr] = (uint16_t)ne;
-                        a.row_list[q][nr++] = (uint8_t)l;
-                        ne += d;
-                    }
-            a.rend[q][c] = (uint8_t)nr;
+        uint8_t order[MB_MAX > NB_MAX ? MB_MAX : NB_MAX], group[sizeof order];
+        // the items of degree deg(i) (0: not this CTA's) in ascending degree, each with its group
+        auto deal = [&](int n, auto deg, int dmax, int overhead, int W) {
+            int load[CL_GROUPS] = {}, m = 0;
+            for (int d = 1; d <= dmax; d++)
+                for (int i = 0; i < n; i++)
+                    if (deg(i) == d) order[m++] = (uint8_t)i;
+            for (int k = m - 1; k >= 0; k--) {
+                int w = 0;
+                for (int g = 1; g < W; g++)
+                    if (load[g] < load[w]) w = g;
+                group[k] = (uint8_t)w;
+                load[w] += deg(order[k]) + overhead;
+            }
+            return m;
+        };
+        auto rdeg = [&](int l) {
+            return l >= a.row_split[q] && l < a.row_split[q + 1] ? h.rowptr[l + 1] - h.rowptr[l] : 0;
+        };
+        auto cdeg = [&](int j) { return a.col_owner[j] == q ? h.colptr[j + 1] - h.colptr[j] : 0; };
+        int m = deal(h.mb, rdeg, h.dc_max, 1, a.W);
+        for (int w = 0; w < a.W; w++) {
+            int c = 0;
+            a.rstart[q][w] = (uint8_t)nr;
+            for (int k = 0; k < m; k++) {
+                if (group[k] != w) continue;
+                const int d = rdeg(order[k]);
+                while (d > cl_class_degree(c)) a.rend[q][w][c++] = (uint8_t)nr;
+                a.row_e0[q][nr] = (uint16_t)ne;
+                a.row_list[q][nr++] = order[k];
+                ne += d;
+            }
+            while (c < CL_CLASSES) a.rend[q][w][c++] = (uint8_t)nr;
         }
         int nx = ne + a.ncols[q];
-        for (int c = 1; c <= 5; c++) {
-            for (int d = c; d <= (c < 5 ? c : h.mb); d++)
-                for (int j = 0; j < h.nb; j++)
-                    if (a.col_owner[j] == q && h.colptr[j + 1] - h.colptr[j] == d) {
-                        a.col_x0[q][nc] = (uint16_t)nx;
-                        a.col_list[q][nc++] = (uint8_t)j;
-                        if (d > 4) nx += d / 4;
-                    }
-            a.cend[q][c - 1] = (uint8_t)nc;
+        const int Wv = a.W4 ? a.W4 : a.W;
+        m = deal(h.nb, cdeg, h.mb, 3, Wv);
+        for (int w = 0; w < Wv; w++) {
+            int c = 1;
+            a.cstart[q][w] = (uint8_t)nc;
+            for (int k = 0; k < m; k++) {
+                if (group[k] != w) continue;
+                const int d = cdeg(order[k]);
+                while (c < 5 && d > c) a.cend[q][w][c++ - 1] = (uint8_t)nc;
+                a.col_x0[q][nc] = (uint16_t)nx;
+                a.col_list[q][nc++] = order[k];
+                if (d > 4) nx += d / 4;
+            }
+            while (c <= 5) a.cend[q][w][c++ - 1] = (uint8_t)nc;
         }
         a.n_edge[q] = ne;
         a.n_tab[q] = nx;
@@ -629,12 +676,6 @@ static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, con
         __atomic_store_n(&cached[dev], clusters, __ATOMIC_RELAXED);
     }
     if ((int64_t)clusters > n_cw) clusters = (int)n_cw;
-    const int wt = (a.H + 31) & ~31, nth = cl_threads<DMAX>();
-    a.W = wt <= nth ? nth / wt : 1;
-    a.WT = wt <= nth ? wt : nth;
-    a.wt4 = (a.Z / 4 + 31) & ~31;
-    a.WT4 = a.Z % 4 ? 32 : a.wt4 <= nth ? a.wt4 : nth;
-    a.W4 = a.Z % 4 ? 0 : nth / a.WT4;
     a.wide_L = a.N % 4 == 0;
     for (int i = 0; i < a.n_req; i++)
         if (reinterpret_cast<uintptr_t>(a.reqs[i].llr) & 15) a.wide_L = 0;
@@ -674,8 +715,6 @@ cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     }
     if (items == 0) return cudaSuccess;
     a.n_items = items;
-    a.Z = h.Z;
-    a.H = (h.Z + 1) / 2;
     a.N = h.N;
     a.next = static_cast<unsigned long long *>(counter);
     a.max_iter = p.max_iter;
