@@ -106,21 +106,25 @@ static SlotLayout slot_layout(const CodeDev &h, int msg, int V, int G)
     return l;
 }
 
-// Shared memory of a launch ahead of its slots: the group hand-over, the slots' bookkeeping
-// and the tables.
-static int tab_offset(int slots) { return (16 + slots * (int)sizeof(FloodBook) + 15) & ~15; }
+// Shared memory ahead of a code's slots: the group hand-over, the code's tables and its slots'
+// bookkeeping.  Each code of a launch is laid out by its own sizes (a CTA that takes up another code lays
+// all of it out anew), so that a code which fits alone fits beside any other.
+static int book_offset(int n_tab) { return FLOOD_TAB0 + n_tab * (int)sizeof(int4); }
+static int slots_offset(int n_tab, int slots)
+{
+    return (book_offset(n_tab) + slots * (int)sizeof(FloodBook) + 15) & ~15;
+}
 
 // Thread slots of a code per CTA and the row groups each is spread over.
 struct SlotShape {
     int G, W, TPG;
 };
 
-// The shape for V codewords per thread, given the table space reserved, with at most `cap`
-// thread slots: the most warps that the instance's threads (dmax: the launch's largest row
+// The shape for V codewords per thread with at most `cap` thread slots: the most warps that the instance's threads (dmax: the launch's largest row
 // degree), the named barriers and shared memory allow, with no more than two row groups
 // unless that leaves fewer than 16 warps: each further row group adds its share of the round's
 // fixed work (N = 1944 rate-1/2 FP32: 3 slots x 2 row groups 906 us, 2 x 4 928 us).
-static SlotShape slot_shape(const CodeDev &h, int msg, int V, int dmax, int n_tab, size_t limit, int cap)
+static SlotShape slot_shape(const CodeDev &h, int msg, int V, int dmax, size_t limit, int cap)
 {
     SlotShape best = {0, 1, 32};
     if (h.dc_max > 32 || h.N >= 65536) return best;
@@ -128,7 +132,8 @@ static SlotShape slot_shape(const CodeDev &h, int msg, int V, int dmax, int n_ta
     int gmax = tmax / wt;
     if (gmax * V > SLOTS_MAX) gmax = SLOTS_MAX / V;
     if (gmax > cap) gmax = cap;
-    while (gmax > 0 && tab_offset(gmax * V) + (size_t)n_tab * sizeof(int4) + slot_layout(h, msg, V, gmax).bytes > limit)
+    const int n_tab = flood_table_size(h);
+    while (gmax > 0 && slots_offset(n_tab, gmax * V) + slot_layout(h, msg, V, gmax).bytes > limit)
         gmax--;
     for (int W = 1; W <= h.mb && W * wt <= tmax; W++) {
         int G = tmax / (W * wt);
@@ -147,7 +152,7 @@ static bool fits_slot(const CodeDev &h, int msg, int V, size_t limit)
     const size_t head = ((size_t)SLOTS_MAX * 16 + 16 + (size_t)4 * (5 * h.nnz + 2 * h.mb + h.nb + 11) + 15) & ~(size_t)15;
     const size_t sa = ((size_t)V * slot_stride(h.N, h.Z) * 4 + 15) & ~(size_t)15;
     return head + sa + (size_t)V * slot_stride(h.E, h.Z) * (msg == LDPC_MSG_F16 ? 2 : 4) <= limit &&
-           slot_shape(h, msg, V, h.dc_max, flood_table_size(h), limit, 1).G > 0;
+           slot_shape(h, msg, V, h.dc_max, limit, 1).G > 0;
 }
 
 int slots_supported(const CodeDev &h, int msg) { return fits_slot(h, msg, 1, 227 * 1024); }
@@ -203,11 +208,12 @@ void flood_build_table(CodeDev &h, int msg, int V, int4 *tab)
     }
 }
 
-// Group the requests by code object, size every group's slots and launch one persistent grid
-// over all of them.
-cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters, cudaStream_t s)
+// Group the requests by code object and size every group's slots for one persistent grid over all of
+// them.
+cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters, size_t limit, int nsm,
+                       FloodPlan &out)
 {
-    FloodArgs a;  // ~7 KB, passed by value as the kernel parameter
+    FloodArgs &a = out.a;  // ~7 KB, passed by value as the kernel parameter
     const ldpc_code *codes[MULTI_MAX_GROUPS];
     int ng = 0;
     for (int i = 0; i < n; i++) {
@@ -219,11 +225,9 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
             codes[ng++] = reqs[i].code;
         }
     }
+    out.ctas = 0;
     if (ng == 0) return cudaSuccess;
-    const size_t limit = max_smem_optin();
-    const int nsm = sm_count();
-    int dmax = 0, n_tab = 0;
-    for (int g = 0; g < ng; g++) n_tab = codes[g]->n_ftab > n_tab ? codes[g]->n_ftab : n_tab;
+    int dmax = 0;
     int64_t items_of[MULTI_MAX_GROUPS] = {};
     for (int g = 0; g < ng; g++) {
         dmax = codes[g]->host.dc_max > dmax ? codes[g]->host.dc_max : dmax;
@@ -237,7 +241,7 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
     auto shapes = [&](int V) {
         for (int g = 0; g < ng; g++) {
             const int64_t per_sm = (items_of[g] + nsm - 1) / nsm, cap = (per_sm + V - 1) / V;
-            shape[g] = slot_shape(codes[g]->host, p.msg, V, dmax, n_tab, limit, cap < SLOTS_MAX ? (int)cap : SLOTS_MAX);
+            shape[g] = slot_shape(codes[g]->host, p.msg, V, dmax, limit, cap < SLOTS_MAX ? (int)cap : SLOTS_MAX);
             if (shape[g].G < 1) return false;
         }
         return true;
@@ -260,10 +264,7 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
     if (V == 2 && !shapes(2)) V = 1;
     if (V == 1 && !shapes(1)) return cudaErrorInvalidValue;
     size_t smem = 0;
-    int threads = 32, nr = 0, slots = 0;
-    for (int g = 0; g < ng; g++) slots = shape[g].G * V > slots ? shape[g].G * V : slots;
-    a.tab0 = tab_offset(slots);
-    a.slots0 = a.tab0 + n_tab * (int)sizeof(int4);
+    int threads = 32, nr = 0;
     double wsum = 0.0, acc = 0.0;
     int64_t min_ctas = 0;
     for (int g = 0; g < ng; g++) wsum += (double)items_of[g] * codes[g]->host.E;
@@ -296,7 +297,9 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
         gd.strA = l.strA;
         gd.strR = l.strR;
         gd.offR = l.offR;
-        smem = a.slots0 + l.bytes > smem ? a.slots0 + l.bytes : smem;
+        gd.book0 = book_offset(codes[g]->n_ftab);
+        gd.slots0 = slots_offset(codes[g]->n_ftab, gd.G * V);
+        smem = gd.slots0 + l.bytes > smem ? gd.slots0 + l.bytes : smem;
         gd.tab = codes[g]->ftab + (size_t)codes[g]->n_ftab * ((p.msg == LDPC_MSG_F16 ? 2 : 0) + V - 1);
         gd.n_tab = codes[g]->n_ftab;
         gd.t_col = h.nnz;
@@ -310,6 +313,7 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
         gd.cumw = g == ng - 1 ? 1.0f : (float)(acc / wsum);
     }
     a.n_groups = ng;
+    a.tab0 = FLOOD_TAB0;
     a.next = static_cast<unsigned long long *>(counters);
     a.max_iter = p.max_iter;
     a.early_exit = p.early_exit;
@@ -318,16 +322,29 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
     if (min_ctas < ctas) ctas = (int)min_ctas;
     if (ng == 1 && items_of[0] <= (int64_t)ctas * a.groups[0].G * V) a.next = nullptr;  // no refills: no counter
     else if (!counters) return cudaErrorInvalidValue;
-    if (a.next) {
-        const cudaError_t e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * ng, s);
+    out.dmax = dmax;
+    out.V = V;
+    out.threads = threads;
+    out.ctas = ctas;
+    out.smem = smem;
+    return cudaSuccess;
+}
+
+cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters, cudaStream_t s)
+{
+    FloodPlan q;
+    cudaError_t e = flood_plan(reqs, n, p, counters, max_smem_optin(), sm_count(), q);
+    if (e != cudaSuccess || q.ctas == 0) return e;
+    if (q.a.next) {
+        e = cudaMemsetAsync(counters, 0, sizeof(unsigned long long) * q.a.n_groups, s);
         if (e != cudaSuccess) return e;
     }
     const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
     if (p.msg == LDPC_MSG_F16)
-        return hc ? flood_slots_launch<__half, true>(dmax, V, a, smem, threads, ctas, s)
-                  : flood_slots_launch<__half, false>(dmax, V, a, smem, threads, ctas, s);
-    return hc ? flood_slots_launch<float, true>(dmax, V, a, smem, threads, ctas, s)
-              : flood_slots_launch<float, false>(dmax, V, a, smem, threads, ctas, s);
+        return hc ? flood_slots_launch<__half, true>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s)
+                  : flood_slots_launch<__half, false>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s);
+    return hc ? flood_slots_launch<float, true>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s)
+              : flood_slots_launch<float, false>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s);
 }
 
 }  // namespace ldpc

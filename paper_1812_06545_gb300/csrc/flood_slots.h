@@ -22,6 +22,7 @@ struct FloodGroup {
     int W, TPG;      // row groups a thread slot is spread over; its threads (W whole-warp groups)
     int strA, strR;  // bytes from one thread slot's posteriors / messages to the next one's
     int offR;        // first thread slot's messages, bytes after the first one's posteriors
+    int book0, slots0;  // its bookkeeping and first slot, bytes from the start of shared memory
     const int4 *tab; // the code's tables on the device (see below), n_tab elements
     int n_tab, t_col, t_row;
     uint8_t rend[FLOOD_CLASSES], cend[5];  // end of each degree class in the row and column lists
@@ -56,7 +57,7 @@ struct FloodArgs {
     int n_groups;
     int max_iter, early_exit;
     float X;
-    int tab0, slots0;  // the tables and the first slot, bytes from the start of shared memory
+    int tab0;  // a code's tables, bytes from the start of shared memory (the same for all: see flood_slots.cu)
     FloodGroup groups[MULTI_MAX_GROUPS];
     FloodReq reqs[MULTI_MAX_REQS];
 };
@@ -70,6 +71,15 @@ struct FloodBook {
     int32_t pad;
 };
 
+// A launch: its parameters and the instance they are for.
+struct FloodPlan {
+    FloodArgs a;
+    int dmax, V, threads, ctas;
+    size_t smem;
+};
+
+constexpr int FLOOD_TAB0 = 16;  // a code's tables, bytes from the start of shared memory
+
 // Named barriers thread slots can have (barrier 0 is the CTA's).
 constexpr int FLOOD_BARRIERS = 15;
 
@@ -78,6 +88,11 @@ __host__ __device__ constexpr int flood_threads_max(int dmax, int V, bool f16)
 {
     return V == 2 && (dmax <= 8 || f16) ? 768 : 640;
 }
+
+// Size a launch for n requests (a.next: the counters, or null where none are needed and none are
+// given); no call to the device.
+cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters, size_t limit, int nsm,
+                       FloodPlan &out);
 
 // Launch the instance for rows of degree <= dmax (8 or 32) and V codewords per thread.
 template <typename MsgT, bool HC>

@@ -116,7 +116,6 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
     extern __shared__ __align__(16) unsigned char smem_raw[];
     char *sm = reinterpret_cast<char *>(smem_raw);
     int32_t *misc = reinterpret_cast<int32_t *>(sm);                // [4] code-group hand-over
-    FloodBook *books = reinterpret_cast<FloodBook *>(sm + 16);      // [slots]
     int4 *tab = reinterpret_cast<int4 *>(sm + a.tab0);              // the code's tables
     using T = VT<V>;
     const int tid = threadIdx.x, nth = blockDim.x;
@@ -145,7 +144,7 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
         const bool mine = member && ru < Z;      // a row of it (else an idle lane of the last warp)
         const int r = ru < Z ? ru : Z - 1;
         const bool lead = mine && ru == 0 && w0 == 0;  // the thread that takes codewords for the slot
-        FloodBook *book = books + (member ? g : 0) * V;
+        FloodBook *book = reinterpret_cast<FloodBook *>(sm + gd.book0) + (member ? g : 0) * V;
         const int32_t *rows = reinterpret_cast<const int32_t *>(tab + gd.t_row);
 
         // a slot's leader takes the group's next codeword and finds its request; without a work
@@ -177,9 +176,9 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
         Place<V> p;
         p.r = r;
         p.own = mine;
-        p.a0 = (uint32_t)(a.slots0 + (member ? g : 0) * gd.strA + r * SA);
+        p.a0 = (uint32_t)(gd.slots0 + (member ? g : 0) * gd.strA + r * SA);
         p.a1 = p.a0 - (uint32_t)(Z * SA);
-        p.r0 = (uint32_t)(a.slots0 + gd.offR + (member ? g : 0) * gd.strR + r * SR);
+        p.r0 = (uint32_t)(gd.slots0 + gd.offR + (member ? g : 0) * gd.strR + r * SR);
         p.r1 = p.r0 - (uint32_t)(Z * SR);
         float *A = reinterpret_cast<float *>(sm + p.a0);   // position r of block column 0
         MsgT *R = reinterpret_cast<MsgT *>(sm + p.r0);     // position r of block 0
