@@ -19,7 +19,8 @@ INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libldpc_gb300.so")
 SOURCES = ["ldpc_api.cu", "flood_kernels.cu", "flood_slots.cu", "flood_slots_f32.cu", "flood_slots_f16.cu",
-           "flood_slots_f32_clamp.cu", "flood_slots_f16_clamp.cu", "flood_cluster.cu", "layered_kernels.cu", "layered_pairs.cu", "layered_spa.cu", "ldpc_static.cu",
+           "flood_slots_f32_clamp.cu", "flood_slots_f16_clamp.cu", "flood_packed_f32.cu", "flood_packed_f16.cu",
+           "flood_packed_f32_clamp.cu", "flood_packed_f16_clamp.cu", "flood_cluster.cu", "layered_kernels.cu", "layered_pairs.cu", "layered_spa.cu", "ldpc_static.cu",
            "ldpc_session.cu", "ldpc_diag.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

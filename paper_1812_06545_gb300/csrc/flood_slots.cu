@@ -12,6 +12,8 @@
 // one straight-line body of exact degree at a time, and control and table indexes are the same
 // for all its lanes.  Only the thread slot's own warps synchronise (a named barrier): the
 // thread slots of a CTA run their rounds independently.
+// Where whole warps would leave many lanes idle (Z below a warp, or just above a multiple of 32), the
+// rows of several thread slots, or of several row groups, lie end to end (flood_packed_kernel.cuh).
 //
 // One round of a thread slot (Sec. II two-phase message passing, Algorithm 1 loop order):
 //   check-node phase   Q = APP - R, R' from the check rule in the product (tanh) domain
@@ -46,7 +48,10 @@
 //   + output ahead of the variable-node phase                  887            629
 // FP32: 18 warps of 3 thread slots (57 warp instructions per edge of two codewords, was 2 x 40);
 // FP16: 24 warps of 4 (six slots of one row group each, 18 warps, took 718).
+#include <math.h>
 #include <string.h>
+
+#include <numeric>
 
 #include "flood_slots.h"
 
@@ -115,31 +120,104 @@ static int slots_offset(int n_tab, int slots)
     return (book_offset(n_tab) + slots * (int)sizeof(FloodBook) + 15) & ~15;
 }
 
-// Thread slots of a code per CTA and the row groups each is spread over.
+// Thread slots of a code per CTA, the row groups each is spread over, and the barrier groups they
+// form: K thread slots of TPG threads together.
 struct SlotShape {
-    int G, W, TPG;
+    int G, W, TPG, K;
 };
 
-// The shape for V codewords per thread with at most `cap` thread slots: the most warps that the instance's threads (dmax: the launch's largest row
-// degree), the named barriers and shared memory allow, with no more than two row groups
-// unless that leaves fewer than 16 warps: each further row group adds its share of the round's
-// fixed work (N = 1944 rate-1/2 FP32: 3 slots x 2 row groups 906 us, 2 x 4 928 us).
+// The most thread slots, up to cap, that shared memory and the bookkeeping allow.
+static int slots_fit(const CodeDev &h, int msg, int V, size_t limit, int cap)
+{
+    if (h.dc_max > 32 || h.N >= 65536) return 0;
+    int G = cap * V > SLOTS_MAX ? SLOTS_MAX / V : cap;
+    while (G > 0 && slots_offset(h.n_ftab, G * V) + slot_layout(h, msg, V, G).bytes > limit) G--;
+    return G;
+}
+
+// The shape of whole-warp rows (k_flood_slots) for V codewords per thread with at most `cap` thread
+// slots: the most warps that the instance's threads (dmax: the launch's largest row degree), the named
+// barriers and shared memory allow, with no more than two row groups unless that leaves fewer than
+// 16 warps: each further row group adds its share of the round's fixed work (N = 1944 rate-1/2 FP32:
+// 3 slots x 2 row groups 906 us, 2 x 4 928 us).
 static SlotShape slot_shape(const CodeDev &h, int msg, int V, int dmax, size_t limit, int cap)
 {
-    SlotShape best = {0, 1, 32};
-    if (h.dc_max > 32 || h.N >= 65536) return best;
+    SlotShape best = {0, 1, 32, 1};
     const int wt = ((h.Z + 31) / 32) * 32, tmax = flood_threads_max(dmax, V, msg == LDPC_MSG_F16);
-    int gmax = tmax / wt;
-    if (gmax * V > SLOTS_MAX) gmax = SLOTS_MAX / V;
-    if (gmax > cap) gmax = cap;
-    const int n_tab = flood_table_size(h);
-    while (gmax > 0 && slots_offset(n_tab, gmax * V) + slot_layout(h, msg, V, gmax).bytes > limit)
-        gmax--;
+    const int gmax = slots_fit(h, msg, V, limit, tmax / wt < cap ? tmax / wt : cap);
     for (int W = 1; W <= h.mb && W * wt <= tmax; W++) {
         int G = tmax / (W * wt);
         if (G > gmax) G = gmax;
         if (W * wt > 32 && G > FLOOD_BARRIERS) G = FLOOD_BARRIERS;
-        if (G * W > best.G * best.W && (W <= 2 || best.G * best.TPG < 512)) best = {G, W, W * wt};
+        if (G * W > best.G * best.W && (W <= 2 || best.G * best.TPG < 512)) best = {G, W, W * wt, 1};
+    }
+    return best;
+}
+
+// What n codewords cost an SM in a shape of V codewords per thread, as warps times check rows:
+//   a round takes ceil(mb / W) block rows of every warp, and as long as 14 more edges for the rest of it;
+//   fewer than 20 warps take as long as 20 (latency);
+//   a few times the resident codewords take whole turns of them;
+//   a row of two codewords takes 1.35 times as long as a row of one (FP16, rows above degree 12, which
+//     spill: 1.55, packed 1.9);
+//   K thread slots in step: 3 % and 2 % each, as some of many codewords end in every round and hold up
+//     the others;
+//   spread row groups: a vote per row, and a warp covers 1 + (32 - gcd) / (K Z) of them on average,
+//     whose rows need different bodies with the share `change` of the degree-ordered list's neighbours.
+// Measured (us, whole warps / packed / spread, 10 iterations): at widths without idle lanes, N = 768 rate 1/2,
+// FP32 675 / 711 / 881, rate 5/6 1000 / 1048 / 1190; 600 codewords of a 12 x 24 code of Z = 3 42 / 27 / 27;
+// 39 of a 46 x 92 code of Z = 9 112 / - / 54; 16588 of a rate-5/6 code of Z = 20, FP16 733 / 600 / 712.
+static double shape_cost(const CodeDev &h, int msg, const SlotShape &s, int V, int64_t n, FloodForm form, double change)
+{
+    const double warps = s.G / s.K * (s.TPG / 32.0), degree = (double)h.nnz / h.mb;
+    double turns = (double)((n + V - 1) / V) / s.G;
+    turns = turns < 8.0 ? ceil(turns) : turns + 0.5;
+    double rows = (h.mb + s.W - 1) / s.W;
+    if (form == FLOOD_SPREAD) {
+        const int block = s.K * h.Z;
+        double span = 1.0 + (32 - std::gcd(block, 32)) / (double)block;
+        if (span > s.W) span = s.W;
+        rows *= 1.0 + 0.25 * (span - 1.0) * change;
+    }
+    double c = (rows + 14.0 / degree) * turns * (warps > 20.0 ? warps : 20.0);
+    if (V == 2) c *= h.dc_max <= 12 || msg != LDPC_MSG_F16 ? 1.35 : form == FLOOD_WHOLE ? 1.55 : 1.9;
+    if (form != FLOOD_WHOLE) c *= (form == FLOOD_SPREAD ? 1.0 + 2.1 / degree : 1.03) + 0.02 * (s.K - 1);
+    return c;
+}
+
+// The share of neighbouring rows of the degree-ordered list that have different bodies.
+static double body_changes(const CodeDev &h)
+{
+    int n = 0;
+    for (int c = 0, end = 0; c < FLOOD_CLASSES; end = h.rend[c++]) n += h.rend[c] > end;
+    return h.mb > 1 ? (n - 1.0) / (h.mb - 1.0) : 0.0;
+}
+
+// The cheapest shape with the rows of K thread slots end to end (k_flood_packed), or with those of the
+// row groups too (spread).
+static SlotShape packed_shape(const CodeDev &h, int msg, int V, int dmax, size_t limit, int cap, int64_t n, FloodForm form)
+{
+    SlotShape best = {0, 1, 32, 1};
+    double cost = 0.0;
+    const int tmax = flood_threads_max(dmax, V, msg == LDPC_MSG_F16);
+    const int gmax = slots_fit(h, msg, V, limit, cap);
+    const bool spread = form == FLOOD_SPREAD;
+    const double change = spread ? body_changes(h) : 0.0;
+    // (of narrow rows, which have many shapes, 1, 2, 3, 4, 6, 8, 12, 16, ...)
+    auto next = [&](int x) { return h.Z >= 16 || x < 4 ? x + 1 : x % 3 ? x / 2 * 3 : x / 3 * 4; };
+    for (int K = spread ? 1 : 2; K <= gmax && K * V <= 32 && K * h.Z <= tmax; K = next(K)) {
+        for (int W = 1; W <= h.mb; W = W == h.mb ? W + 1 : next(W) < h.mb ? next(W) : h.mb) {
+            const int tpg = spread ? (K * W * h.Z + 31) & ~31 : W * ((K * h.Z + 31) & ~31);
+            if (tpg > tmax) break;
+            int groups = tmax / tpg < gmax / K ? tmax / tpg : gmax / K;
+            if (tpg > 32 && groups > FLOOD_BARRIERS) groups = FLOOD_BARRIERS;
+            const SlotShape s = {groups * K, W, tpg, K};
+            const double c = shape_cost(h, msg, s, V, n, form, change);
+            if (best.G == 0 || c < cost * 0.999) {
+                best = s;
+                cost = c;
+            }
+        }
     }
     return best;
 }
@@ -175,7 +253,7 @@ void flood_build_table(CodeDev &h, int msg, int V, int4 *tab)
 {
     const int SA = 4 * V, SR = (msg == LDPC_MSG_F16 ? 2 : 4) * V;
     const int base_r = msg == LDPC_MSG_F16 ? 0 : slot_layout(h, msg, V, 1).offR;
-    int32_t *rows = reinterpret_cast<int32_t *>(tab + flood_table_size(h) - table_words(h)), *cols = rows + h.mb;
+    int32_t *rows = reinterpret_cast<int32_t *>(tab + h.n_ftab - table_words(h)), *cols = rows + h.mb;
     int ne = 0, nr = 0;
     for (int c = 0; c < FLOOD_CLASSES; c++) {
         const int lo = c ? flood_class_degree(c - 1) : 0, hi = flood_class_degree(c);
@@ -238,31 +316,69 @@ cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, 
     // shapes with V codewords per thread; a small batch spreads over the SMs rather than
     // filling a few CTAs' slots
     SlotShape shape[MULTI_MAX_GROUPS];
-    auto shapes = [&](int V) {
+    int64_t per_sm[MULTI_MAX_GROUPS];
+    for (int g = 0; g < ng; g++) per_sm[g] = (items_of[g] + nsm - 1) / nsm;
+    // (in s; returns the launch's estimated cost, 0: some code has no slot)
+    auto shapes = [&](int V, FloodForm form, SlotShape *s) {
+        double cost = 0.0;
         for (int g = 0; g < ng; g++) {
-            const int64_t per_sm = (items_of[g] + nsm - 1) / nsm, cap = (per_sm + V - 1) / V;
-            shape[g] = slot_shape(codes[g]->host, p.msg, V, dmax, limit, cap < SLOTS_MAX ? (int)cap : SLOTS_MAX);
-            if (shape[g].G < 1) return false;
+            const CodeDev &h = codes[g]->host;
+            const int64_t want = (per_sm[g] + V - 1) / V;
+            const int cap = want < SLOTS_MAX ? (int)want : SLOTS_MAX;
+            s[g] = form == FLOOD_WHOLE ? slot_shape(h, p.msg, V, dmax, limit, cap)
+                                       : packed_shape(h, p.msg, V, dmax, limit, cap, per_sm[g], form);
+            if (s[g].G < 1) return 0.0;
+            cost += h.nnz / (double)h.mb *
+                    shape_cost(h, p.msg, s[g], V, per_sm[g], form, body_changes(h));
         }
-        return true;
+        return cost;
     };
+    SlotShape pair[MULTI_MAX_GROUPS];
+    const double one = tuned == SCHED_SLOTS_V2 ? 0.0 : shapes(1, FLOOD_WHOLE, shape);
     int V = tuned == SCHED_SLOTS_V1 ? 1 : 2;
-    if (!tuned && shapes(1)) {
+    double whole = one;
+    if (!tuned && one > 0.0) {
         // one codeword per thread where every code's codewords are all resident at once with two
-        // row groups or more each; with rows above degree 16 (few block rows, long serial rows) also
-        // with one, up to 12 warps.  Per launch on GB300, one against two codewords per thread, 3 / 4
+        // row groups or more each, or one to an SM; with rows above degree 16 (few block rows, long
+        // serial rows) also with one, up to 12 warps.  Per launch on GB300, one against two codewords per thread, 3 / 4
         // / 6 codewords per SM: N = 1944 rate 1/2 FP32 82 / 100, 116 / 100, 140 / 127 us; rate 5/6
         // 126 / 178, 156 / 181, 226 / 211; N = 648 rate 1/2 46 / 66, 55 / 68, 66 / 75 (and 12: 113 / 110).
         bool single = true;
-        for (int g = 0; g < ng && single; g++) {
-            const CodeDev &h = codes[g]->host;
-            const int64_t per_sm = (items_of[g] + nsm - 1) / nsm;
-            single = per_sm <= shape[g].G && (shape[g].W >= 2 || (h.dc_max > 16 && per_sm * shape[g].TPG <= 400));
-        }
+        for (int g = 0; g < ng && single; g++)
+            single = per_sm[g] <= shape[g].G && (shape[g].W >= 2 || per_sm[g] == 1 ||
+                                                 (codes[g]->host.dc_max > 16 && per_sm[g] * shape[g].TPG <= 400));
         if (single) V = 1;
     }
-    if (V == 2 && !shapes(2)) V = 1;
-    if (V == 1 && !shapes(1)) return cudaErrorInvalidValue;
+    if (V == 2) {
+        whole = shapes(2, FLOOD_WHOLE, pair);
+        if (whole == 0.0 || (one > 0.0 && one * 1.2 < whole)) {  // (clearly cheaper: fewer pairs fit than half the codewords)
+            V = 1;
+            whole = tuned == SCHED_SLOTS_V2 ? shapes(1, FLOOD_WHOLE, shape) : one;
+        } else {
+            memcpy(shape, pair, sizeof shape);
+        }
+    }
+    if (whole == 0.0) return cudaErrorInvalidValue;
+    // rows end to end where a quarter of some code's warps would be idle and that is estimated 5 % cheaper
+    out.form = FLOOD_WHOLE;
+    bool idle = false;
+    int64_t most = 0;  // (one codeword to an SM has nothing to be packed with)
+    for (int g = 0; g < ng; g++) {
+        idle |= 4 * codes[g]->host.Z <= 3 * ((codes[g]->host.Z + 31) & ~31);
+        most = per_sm[g] > most ? per_sm[g] : most;
+    }
+    const struct { FloodForm form; int V; } other[3] = {{FLOOD_PACKED, 1}, {FLOOD_PACKED, 2}, {FLOOD_SPREAD, 1}};
+    for (int i = 0; i < 3 && idle; i++) {
+        SlotShape s[MULTI_MAX_GROUPS];
+        if ((tuned && other[i].V != V) || (other[i].form == FLOOD_PACKED && most < 2 * other[i].V)) continue;
+        const double cost = shapes(other[i].V, other[i].form, s);
+        if (cost > 0.0 && cost * (out.form ? 1.0 : 1.05) < whole) {
+            out.form = other[i].form;
+            whole = cost;
+            V = other[i].V;
+            memcpy(shape, s, sizeof shape);
+        }
+    }
     size_t smem = 0;
     int threads = 32, nr = 0;
     double wsum = 0.0, acc = 0.0;
@@ -293,21 +409,22 @@ cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, 
         gd.G = shape[g].G;
         gd.W = shape[g].W;
         gd.TPG = shape[g].TPG;
+        gd.K = shape[g].K;
         const SlotLayout l = slot_layout(h, p.msg, V, gd.G);
         gd.strA = l.strA;
         gd.strR = l.strR;
         gd.offR = l.offR;
-        gd.book0 = book_offset(codes[g]->n_ftab);
-        gd.slots0 = slots_offset(codes[g]->n_ftab, gd.G * V);
+        gd.book0 = book_offset(h.n_ftab);
+        gd.slots0 = slots_offset(h.n_ftab, gd.G * V);
         smem = gd.slots0 + l.bytes > smem ? gd.slots0 + l.bytes : smem;
-        gd.tab = codes[g]->ftab + (size_t)codes[g]->n_ftab * ((p.msg == LDPC_MSG_F16 ? 2 : 0) + V - 1);
-        gd.n_tab = codes[g]->n_ftab;
+        gd.tab = codes[g]->ftab + (size_t)h.n_ftab * ((p.msg == LDPC_MSG_F16 ? 2 : 0) + V - 1);
+        gd.n_tab = h.n_ftab;
         gd.t_col = h.nnz;
-        gd.t_row = codes[g]->n_ftab - table_words(h);
+        gd.t_row = h.n_ftab - table_words(h);
         gd.mb = h.mb;
         memcpy(gd.rend, h.rend, sizeof gd.rend);
         memcpy(gd.cend, h.cend, sizeof gd.cend);
-        threads = gd.G * gd.TPG > threads ? gd.G * gd.TPG : threads;
+        threads = gd.G / gd.K * gd.TPG > threads ? gd.G / gd.K * gd.TPG : threads;
         min_ctas += (items + gd.G * V - 1) / (gd.G * V);
         acc += (double)items * h.E;
         gd.cumw = g == ng - 1 ? 1.0f : (float)(acc / wsum);
@@ -330,6 +447,12 @@ cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, 
     return cudaSuccess;
 }
 
+template <typename MsgT, bool HC>
+static cudaError_t launch(const FloodPlan &q, cudaStream_t s)
+{
+    return q.form == FLOOD_WHOLE ? flood_slots_launch<MsgT, HC>(q, s) : flood_packed_launch<MsgT, HC>(q, s);
+}
+
 cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters, cudaStream_t s)
 {
     FloodPlan q;
@@ -340,11 +463,8 @@ cudaError_t flood_multi_decode(const HostReq *reqs, int n, const ldpc_decode_par
         if (e != cudaSuccess) return e;
     }
     const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
-    if (p.msg == LDPC_MSG_F16)
-        return hc ? flood_slots_launch<__half, true>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s)
-                  : flood_slots_launch<__half, false>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s);
-    return hc ? flood_slots_launch<float, true>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s)
-              : flood_slots_launch<float, false>(q.dmax, q.V, q.a, q.smem, q.threads, q.ctas, s);
+    if (p.msg == LDPC_MSG_F16) return hc ? launch<__half, true>(q, s) : launch<__half, false>(q, s);
+    return hc ? launch<float, true>(q, s) : launch<float, false>(q, s);
 }
 
 }  // namespace ldpc

@@ -19,7 +19,8 @@ struct FloodGroup {
     int req_begin, req_end;
     int N, Z, mb, nb, nnz;
     int G;           // thread slots (V codewords each) per CTA
-    int W, TPG;      // row groups a thread slot is spread over; its threads (W whole-warp groups)
+    int W, TPG;      // row groups a thread slot is spread over; threads of a barrier group
+    int K;           // thread slots of a barrier group (1 unless they lie end to end in a warp)
     int strA, strR;  // bytes from one thread slot's posteriors / messages to the next one's
     int offR;        // first thread slot's messages, bytes after the first one's posteriors
     int book0, slots0;  // its bookkeeping and first slot, bytes from the start of shared memory
@@ -71,10 +72,16 @@ struct FloodBook {
     int32_t pad;
 };
 
-// A launch: its parameters and the instance they are for.
+// How rows lie in a warp: whole warps to a thread slot's rows (flood_slots_kernel.cuh), the rows of K
+// thread slots end to end, or those and the row groups end to end (flood_packed_kernel.cuh).
+enum FloodForm { FLOOD_WHOLE, FLOOD_PACKED, FLOOD_SPREAD };
+
+// A launch: its parameters and the instance they are for (rows of degree <= 8, or up to 32; V codewords
+// per thread).
 struct FloodPlan {
     FloodArgs a;
     int dmax, V, threads, ctas;
+    FloodForm form;
     size_t smem;
 };
 
@@ -94,9 +101,11 @@ __host__ __device__ constexpr int flood_threads_max(int dmax, int V, bool f16)
 cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, void *counters, size_t limit, int nsm,
                        FloodPlan &out);
 
-// Launch the instance for rows of degree <= dmax (8 or 32) and V codewords per thread.
+// Launch a plan.
 template <typename MsgT, bool HC>
-cudaError_t flood_slots_launch(int dmax, int V, const FloodArgs &a, size_t smem, int threads, int ctas,
-                               cudaStream_t s);
+cudaError_t flood_slots_launch(const FloodPlan &q, cudaStream_t s);
+
+template <typename MsgT, bool HC>
+cudaError_t flood_packed_launch(const FloodPlan &q, cudaStream_t s);
 
 }  // namespace ldpc

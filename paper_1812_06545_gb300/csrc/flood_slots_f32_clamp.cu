@@ -2,5 +2,5 @@
 #include "flood_slots_kernel.cuh"
 
 namespace ldpc {
-template cudaError_t flood_slots_launch<float, true>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
+template cudaError_t flood_slots_launch<float, true>(const FloodPlan &, cudaStream_t);
 }  // namespace ldpc

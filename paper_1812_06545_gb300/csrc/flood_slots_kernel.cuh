@@ -343,24 +343,20 @@ __global__ void __launch_bounds__(flood_threads_max(DMAX, V, sizeof(MsgT) == 2),
 }
 
 template <int DMAX, int V, typename MsgT, bool HC>
-static cudaError_t launch_one(const FloodArgs &a, size_t smem, int threads, int ctas, cudaStream_t s)
+static cudaError_t launch_one(const FloodPlan &q, cudaStream_t s)
 {
-    cudaError_t e = ensure_smem<k_flood_slots<DMAX, V, MsgT, HC>>(smem);
+    cudaError_t e = ensure_smem<k_flood_slots<DMAX, V, MsgT, HC>>(q.smem);
     if (e != cudaSuccess) return e;
     LaunchScope ls(F_SLOTS, s);
-    k_flood_slots<DMAX, V, MsgT, HC><<<(unsigned)ctas, threads, smem, s>>>(a);
+    k_flood_slots<DMAX, V, MsgT, HC><<<(unsigned)q.ctas, q.threads, q.smem, s>>>(q.a);
     return cudaGetLastError();
 }
 
 template <typename MsgT, bool HC>
-cudaError_t flood_slots_launch(int dmax, int V, const FloodArgs &a, size_t smem, int threads, int ctas,
-                               cudaStream_t s)
+cudaError_t flood_slots_launch(const FloodPlan &q, cudaStream_t s)
 {
-    if (dmax <= 8)
-        return V == 2 ? launch_one<8, 2, MsgT, HC>(a, smem, threads, ctas, s)
-                      : launch_one<8, 1, MsgT, HC>(a, smem, threads, ctas, s);
-    return V == 2 ? launch_one<32, 2, MsgT, HC>(a, smem, threads, ctas, s)
-                  : launch_one<32, 1, MsgT, HC>(a, smem, threads, ctas, s);
+    if (q.dmax <= 8) return q.V == 2 ? launch_one<8, 2, MsgT, HC>(q, s) : launch_one<8, 1, MsgT, HC>(q, s);
+    return q.V == 2 ? launch_one<32, 2, MsgT, HC>(q, s) : launch_one<32, 1, MsgT, HC>(q, s);
 }
 
 }  // namespace ldpc

@@ -288,19 +288,19 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
     cudaError_t e = cudaGetDevice(&c->device);
     if (e == cudaSuccess) e = ldpc::device_status_word(c->device, &h.status);
     // one allocation: the code's description, then the flooding slot decoder's tables
-    c->n_ftab = h.dc_max <= 32 ? ldpc::flood_table_size(h) : 0;
+    h.n_ftab = h.dc_max <= 32 ? ldpc::flood_table_size(h) : 0;
     const size_t head = (sizeof(CodeDev) + 255) & ~(size_t)255;
     std::vector<char> img;
     try {
-        img.resize(head + (size_t)4 * c->n_ftab * sizeof(int4));
+        img.resize(head + (size_t)4 * h.n_ftab * sizeof(int4));
     } catch (const std::bad_alloc &) {
         delete c;
         return fail(LDPC_ENOMEM, "host allocation failed");
     }
     int4 *tab = reinterpret_cast<int4 *>(img.data() + head);
-    if (c->n_ftab)
+    if (h.n_ftab)
         for (int v = 0; v < 4; v++)
-            ldpc::flood_build_table(h, v < 2 ? LDPC_MSG_F32 : LDPC_MSG_F16, 1 + (v & 1), tab + (size_t)v * c->n_ftab);
+            ldpc::flood_build_table(h, v < 2 ? LDPC_MSG_F32 : LDPC_MSG_F16, 1 + (v & 1), tab + (size_t)v * h.n_ftab);
     memcpy(img.data(), &h, sizeof h);
     if (e == cudaSuccess) e = cudaMalloc(&c->dev, img.size());
     if (e == cudaSuccess) e = cudaMemcpy(c->dev, img.data(), img.size(), cudaMemcpyHostToDevice);

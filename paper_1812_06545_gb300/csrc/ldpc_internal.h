@@ -24,7 +24,7 @@ constexpr int TILE = 128;
 struct CodeDev {
     int32_t mb, nb, Z, nnz;
     int32_t N, M, K, E;
-    int32_t dc_max, dv_max, pad0, pad1;
+    int32_t dc_max, dv_max, n_ftab, pad;  // n_ftab: elements of the flooding slot decoder's tables
     int32_t rowptr[MB_MAX + 1];  // blocks of block row l: [rowptr[l], rowptr[l+1])
     int32_t ent[NNZ_MAX];        // (j << 16) | s for block b
     int32_t colptr[NB_MAX + 1];  // entries of block column j: [colptr[j], colptr[j+1])
@@ -149,8 +149,7 @@ struct ldpc_code {
     int device;
     int sms;             // SMs of the device
     cudaMemPool_t pool;  // the device's scratch pool (shared with its other codes), or null
-    int4 *ftab;          // flooding slot decoder's tables: [2 * (F16) + V - 1][n_ftab] (flood_slots.h)
-    int n_ftab;
+    int4 *ftab;          // flooding slot decoder's tables: [2 * (F16) + V - 1][host.n_ftab] (flood_slots.h)
     int tuned_flood[2];  // per message type (F32, F16)
     int tuned_layered;
 };

@@ -2,8 +2,9 @@
 // codes and launches from standard input, prints what flood_plan made of each launch.
 //   code:   C mb nb Z, then mb * nb shifts (-1: no block)
 //   launch: L f16 n, then n pairs (code, codewords)
-// Output per launch: the status, bytes of shared memory, threads, CTAs, codewords per thread, then
-// per code its thread slots, their row groups and threads, and where its layout ends.
+// Output per launch: whether every code is served alone, the status, bytes of shared memory, threads,
+// CTAs, codewords per thread, the form, then per code its width, thread slots, row
+// groups, threads and thread slots of a barrier group, and where its layout ends.
 #include <stdio.h>
 
 #include <vector>
@@ -12,11 +13,17 @@
 
 namespace ldpc {
 template <typename M, bool H>
-cudaError_t flood_slots_launch(int, int, const FloodArgs &, size_t, int, int, cudaStream_t) { return cudaErrorUnknown; }
-template cudaError_t flood_slots_launch<float, false>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
-template cudaError_t flood_slots_launch<float, true>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
-template cudaError_t flood_slots_launch<__half, false>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
-template cudaError_t flood_slots_launch<__half, true>(int, int, const FloodArgs &, size_t, int, int, cudaStream_t);
+cudaError_t flood_slots_launch(const FloodPlan &, cudaStream_t) { return cudaErrorUnknown; }
+template <typename M, bool H>
+cudaError_t flood_packed_launch(const FloodPlan &, cudaStream_t) { return cudaErrorUnknown; }
+template cudaError_t flood_slots_launch<float, false>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_packed_launch<float, false>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_slots_launch<float, true>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_packed_launch<float, true>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_slots_launch<__half, false>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_packed_launch<__half, false>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_slots_launch<__half, true>(const FloodPlan &, cudaStream_t);
+template cudaError_t flood_packed_launch<__half, true>(const FloodPlan &, cudaStream_t);
 }  // namespace ldpc
 
 using namespace ldpc;
@@ -45,8 +52,8 @@ static ldpc_code *read_code()
     h.colptr[h.nb] = k;
     h.N = h.nb * h.Z;
     h.E = h.nnz * h.Z;
-    c->n_ftab = flood_table_size(h);
-    std::vector<int4> tab(c->n_ftab);
+    h.n_ftab = flood_table_size(h);
+    std::vector<int4> tab(h.n_ftab);
     flood_build_table(h, LDPC_MSG_F32, 1, tab.data());  // (sets the degree classes)
     return c;
 }
@@ -81,13 +88,13 @@ int main()
         static FloodPlan q;
         unsigned long long counters[MULTI_MAX_GROUPS];
         const cudaError_t e = flood_plan(reqs.data(), n, p, counters, limit, 152, q);
-        printf("%d %d %zu %d %d %d", (int)ok, (int)e, q.smem, q.threads, q.ctas, q.V);
+        printf("%d %d %zu %d %d %d %d", (int)ok, (int)e, q.smem, q.threads, q.ctas, q.V, (int)q.form);
         for (int g = 0; e == cudaSuccess && g < q.a.n_groups; g++) {
             const FloodGroup &d = q.a.groups[g];
             const size_t E = (size_t)d.nnz * d.Z;
             const size_t end_a = (size_t)(d.G - 1) * d.strA + 4 * (size_t)q.V * d.N;
             const size_t end_r = d.offR + (size_t)(d.G - 1) * d.strR + (f16 ? 2 : 4) * q.V * E;
-            printf(" %d %d %d %zu", d.G, d.W, d.TPG, d.slots0 + (end_a > end_r ? end_a : end_r));
+            printf(" %d %d %d %d %d %zu", d.Z, d.G, d.W, d.TPG, d.K, d.slots0 + (end_a > end_r ? end_a : end_r));
         }
         printf("\n");
     }

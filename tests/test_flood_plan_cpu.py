@@ -45,14 +45,19 @@ def plan(tmp_path_factory):
 
 
 def check(launch, row):
-    served, status, smem, threads, ctas, V = row[:6]
+    served, status, smem, threads, ctas, V, form = row[:7]
     if not served:
         return False
     assert status == 0, (launch, row)
     assert smem <= LIMIT and threads <= 768 and 1 <= ctas <= 152, (launch, row)
-    for g in range(6, len(row), 4):
-        G, W, TPG, end = row[g:g + 4]
-        assert G >= 1 and G * TPG <= threads and end <= smem, (launch, row)
+    for g in range(7, len(row), 6):
+        Z, G, W, TPG, K, end = row[g:g + 6]
+        assert G >= 1 and G % K == 0 and G // K * TPG <= threads and end <= smem, (launch, row)
+        # K thread slots' rows (form 2: of all row groups) end to end over whole warps, a warp's lane to
+        # each of their codewords
+        lanes = K * Z * (W if form == 2 else 1)
+        assert TPG == (lanes + 31) // 32 * 32 * (1 if form == 2 else W), (launch, row)
+        assert K * V <= 32 and (form or K == 1) and (form != 2 or V == 1), (launch, row)
     return True
 
 
