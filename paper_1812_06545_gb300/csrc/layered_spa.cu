@@ -8,7 +8,8 @@
 // of every block row (layer): the Z checks of a QC layer touch disjoint variables (each block
 // is one circulant), so the row threads update a layer at once, and the thread slot's own
 // barrier (a named barrier, or the warp itself) separates consecutive layers; the thread slots
-// of a CTA run independently.  Messages are in check-row order, edge (b, r) at b*Z + r: the
+// of a CTA run independently (narrow codes: several thread slots to a barrier, see
+// k_layered_spa_packed).  Messages are in check-row order, edge (b, r) at b*Z + r: the
 // layered schedule has no variable-node pass, so a warp reads and writes them contiguously.
 // Per check (the arithmetic of the flooding slot decoder, only the schedule differs):
 //   Q_k   = APP_n - R_k                                   over the check's edges
@@ -32,6 +33,8 @@
 // APP is never -0: the refill adds +0 to the (scaled) channel value and Q + R' is -0 only when both
 // are -0, which cannot happen while APP is not -0 (then Q = APP - R is not -0).  The sign
 // bit therefore is the hard decision [APP < 0] and sgn(0) = +1, as the oracle reads it.
+#include <math.h>
+
 #include "flood_check.cuh"
 
 namespace ldpc {
@@ -60,7 +63,8 @@ struct LayeredSpaArgs {
     unsigned long long *next;
     // sizes and layer lists from here, not from the code's device tables: known to be warp-uniform
     int N, Z, mb, nb, nnz;
-    int G, TPG;        // thread slots per CTA, threads of one (whole warps)
+    int G, TPG;        // thread slots per CTA, threads of a barrier group (whole warps)
+    int K;             // thread slots of a barrier group (1 unless packed)
     int tab0, slots0;  // tables and first slot, bytes from the start of shared memory
     int strA, strR, offR;  // bytes from one thread slot's posteriors / messages to the next one's; first messages
     int max_iter, early_exit;
@@ -482,6 +486,167 @@ __global__ void __launch_bounds__(lspa_threads(DMAX, V, sizeof(MsgT) == 2), 1)
     }
 }
 
+// The same for widths that whole warps fit badly (Z of a few lanes, or just above a multiple of 32): the
+// rows of K thread slots lie end to end over ceil(K Z / 32) warps.  They share a barrier and run their
+// layers in step, so that layers, degrees and tables stay the same for all lanes of a warp and only
+// the slot is a lane's own; each codeword still ends, is written out and refilled by itself.  The state
+// of the group's codewords is kept by every warp, codeword i in lane i (so K V <= 32), and what a warp
+// does next is decided by votes, alike in all warps of the group.  Results are bit-equal.
+template <int DMAX, int V, typename MsgT, bool HC>
+__global__ void __launch_bounds__(lspa_threads(DMAX, V, sizeof(MsgT) == 2), 1)
+    k_layered_spa_packed(const CodeDev *__restrict__ cd, const __grid_constant__ LayeredSpaArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    char *sm = reinterpret_cast<char *>(smem_raw);
+    LspaBook *books = reinterpret_cast<LspaBook *>(sm);
+    int4 *tab = reinterpret_cast<int4 *>(sm + a.tab0);
+    constexpr int SA = (int)sizeof(float) * V, SR = (int)sizeof(MsgT) * V;
+    constexpr uint32_t kSign = 0x80000000u;
+    constexpr unsigned kFull = 0xffffffffu;
+    const int N = a.N, Z = a.Z, mb = a.mb, nb = a.nb, nnz = a.nnz, TPG = a.TPG, K = a.K, KV = K * V;
+    const int tid = threadIdx.x, nth = blockDim.x, lane = tid & 31;
+    const float Xb = a.X * kSLog2e, Pb = s_phi_b2(a.X);  // the clamp [phi(X), X] in base-2 units
+    for (int i = tid; i < nnz; i += nth) {
+        const int e = cd->ent[i], sh = e & 0xffff;
+        tab[i] = make_int4(SA * ((e >> 16) * Z + sh), SR * i * Z, Z - sh, 0);
+    }
+    // barrier group g (a warp reduction: known to be warp-uniform); a lane's thread slot k and row r
+    const int g = (int)__reduce_min_sync(kFull, (unsigned)(tid / TPG)), x = tid - g * TPG;
+    const bool own = x < K * Z;  // (else an idle lane of the group's last warp)
+    const int k = own ? x / Z : 0, r = own ? x - k * Z : 0, slot = g * K + k;
+    const bool lead = own && r == 0;
+    LspaBook *gbook = books + g * KV, *book = gbook + k * V;
+    const unsigned peers = __match_any_sync(kFull, own ? k : -1);  // the warp's lanes of the same thread slot
+    auto grab = [&](int v, bool first) {
+        const unsigned long long n = a.next  ? atomicAdd(a.next, 1ull)
+                                     : first ? blockIdx.x + (unsigned long long)gridDim.x * (slot * V + v)
+                                             : ~0ull;
+        book[v].cw = n < (unsigned long long)a.n_cw ? (int64_t)n : -1;
+    };
+    if (lead) {
+#pragma unroll
+        for (int v = 0; v < V; v++) {
+            grab(v, true);
+            book[v].bad[0] = book[v].bad[1] = 0;
+        }
+    }
+    __syncthreads();
+    Place<V> p;
+    p.own = own;
+    p.r = r;
+    p.a0 = (uint32_t)(a.slots0 + slot * a.strA + r * SA);
+    p.a1 = p.a0 - (uint32_t)(Z * SA);
+    p.r0 = (uint32_t)(a.slots0 + a.offR + slot * a.strR + r * SR);
+    p.r1 = p.r0;
+    float *A = reinterpret_cast<float *>(sm + p.a0);
+    MsgT *R = reinterpret_cast<MsgT *>(sm + p.r0);
+    auto gsync = [&]() {
+        if (TPG == 32)
+            __syncwarp();
+        else
+            asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(TPG) : "memory");
+    };
+    auto refill = [&](int v, int64_t n) {  // as k_layered_spa's
+        const float *L = a.llr + n * N + r;
+        constexpr int CH = 4;
+        for (int j0 = 0; j0 < nb; j0 += CH) {
+            float y[CH];
+#pragma unroll
+            for (int w = 0; w < CH; w++)
+                if (j0 + w < nb) y[w] = __ldg(L + (j0 + w) * Z);
+#pragma unroll
+            for (int w = 0; w < CH; w++)
+                if (j0 + w < nb) {
+                    if (!isfinite(y[w])) atomicOr(cd->status, IN_NONFINITE);
+                    A[(j0 + w) * Z * V + v] = kBase2<MsgT> ? fmaf(y[w], kSLog2e, 0.0f) : y[w] + 0.0f;
+                }
+        }
+        for (int b = 0; b < nnz; b++) R[b * Z * V + v] = MsgT(0.0f);
+    };
+    int64_t cw[V];  // the lane's codewords
+#pragma unroll
+    for (int v = 0; v < V; v++) {
+        cw[v] = book[v].cw;
+        if (cw[v] >= 0 && own) refill(v, cw[v]);
+    }
+    // codeword `lane` of the group: whether there is one, and iterations completed on it
+    bool has = lane < KV && gbook[lane].cw >= 0;
+    int t = 0;
+    unsigned busy = __ballot_sync(kFull, has);
+    auto bit = [&](unsigned m, int v) -> bool { return (m >> (k * V + v)) & 1u; };
+    gsync();
+
+    for (int ph = 0; busy != 0; ph ^= 1) {
+#pragma unroll 1
+        for (int l = 0; l < mb; l++) {
+            layer_check<DMAX, V, MsgT, HC>(a.deg[l], tab + a.first[l], sm, p, Xb, Pb);
+            gsync();
+        }
+        t += has;
+        if (a.early_exit) {
+            // syndrome of the hard decisions, until each codeword with rows in this warp has shown an
+            // unsatisfied check
+            bool seen[V];
+#pragma unroll
+            for (int v = 0; v < V; v++) seen[v] = !own || !bit(busy, v);
+#pragma unroll 1
+            for (int l = 0; l < mb; l++) {
+                uint32_t par[V];
+                lspa_parity<V>(a.deg[l], tab + a.first[l], sm, p, par);
+                bool rest = false;
+#pragma unroll
+                for (int v = 0; v < V; v++) {
+                    seen[v] |= (__ballot_sync(kFull, (par[v] & kSign) != 0) & peers) != 0;
+                    rest |= !seen[v];
+                }
+                if (!__any_sync(kFull, rest)) break;
+            }
+            if (own && lane == __ffs(peers) - 1) {
+#pragma unroll
+                for (int v = 0; v < V; v++)
+                    if (seen[v]) book[v].bad[ph] = 1;
+            }
+            gsync();
+        }
+        const bool end = has && ((a.early_exit && gbook[lane].bad[ph] == 0) || t >= a.max_iter);
+        const unsigned done = __ballot_sync(kFull, end);
+        // the other flag was last read in the iteration before
+        if (a.early_exit && x < KV) gbook[x].bad[ph ^ 1] = 0;
+        if (done != 0) {
+#pragma unroll
+            for (int v = 0; v < V; v++) {
+                const int tv = __shfl_sync(kFull, t, k * V + v);
+                if (own && bit(done, v)) {
+                    uint8_t *Bo = a.bits + cw[v] * N + r;
+                    float *Ao = a.app_out ? a.app_out + cw[v] * N + r : nullptr;
+                    for (int j = 0; j < nb; j++) {
+                        const float y = A[j * Z * V + v];
+                        Bo[j * Z] = y < 0.0f ? 1 : 0;
+                        if (Ao) Ao[j * Z] = kBase2<MsgT> ? y * kSLn2 : y;
+                    }
+                    if (lead) {
+                        a.iters[cw[v]] = tv;
+                        grab(v, false);
+                    }
+                }
+            }
+            gsync();
+            if (end) {
+                has = gbook[lane].cw >= 0;
+                t = 0;
+            }
+            busy = __ballot_sync(kFull, has);
+#pragma unroll
+            for (int v = 0; v < V; v++)
+                if (bit(done, v)) {
+                    cw[v] = book[v].cw;
+                    if (cw[v] >= 0 && own) refill(v, cw[v]);
+                }
+            gsync();
+        }
+    }
+}
+
 static size_t lspa_slot_bytes(const CodeDev &h, int msg)
 {
     return (size_t)((h.N + 3) & ~3) * sizeof(float) +
@@ -514,27 +679,52 @@ int layered_spa_slots_per_cta(const CodeDev &h, int msg)
 // Strides congruent to Z modulo the 32 banks, so that rows of neighbouring slots do not collide.
 static int lspa_stride(int n, int Z) { return n + ((Z % 32) - (n % 32) + 32) % 32; }
 
-// Thread slots of V codewords per CTA, at most cap.
+// Thread slots of V codewords per CTA, at most cap, that the bookkeeping and shared memory allow.
+static int lspa_room(const CodeDev &h, int msg, int V, int cap)
+{
+    int G = cap * V > SLOTS_MAX ? SLOTS_MAX / V : cap;
+    const size_t slot = (size_t)V * (4 * (size_t)lspa_stride(h.N, h.Z) +
+                                     (msg == LDPC_MSG_F16 ? 2 : 4) * (size_t)lspa_stride(h.E, h.Z)), limit = lspa_limit();
+    while (G > 0 && (size_t)G * V * sizeof(LspaBook) + (size_t)h.nnz * 16 + 64 + G * slot > limit) G--;
+    return G;
+}
+
+// Thread slots of whole warps.
 static int lspa_fit(const CodeDev &h, int msg, int V, int cap)
 {
     const int wt = ((h.Z + 31) / 32) * 32, dmax = h.dc_max <= 8 ? 8 : 32;
     int G = lspa_threads(dmax, V, msg == LDPC_MSG_F16) / wt;
     if (G > cap) G = cap;
-    if (G * V > SLOTS_MAX) G = SLOTS_MAX / V;
     if (wt > 32 && G > 15) G = 15;  // named barriers
-    const size_t slot = (size_t)V * (4 * (size_t)lspa_stride(h.N, h.Z) +
-                                     (msg == LDPC_MSG_F16 ? 2 : 4) * (size_t)lspa_stride(h.E, h.Z));
-    while (G > 0 && (size_t)G * V * sizeof(LspaBook) + (size_t)h.nnz * 16 + 64 + G * slot > lspa_limit()) G--;
-    return G;
+    return lspa_room(h, msg, V, G);
+}
+
+// What n codewords cost an SM with G thread slots in groups of K and so many warps, in warps times
+// turns: fewer than 20 warps take as long as 20 (latency), a few times the resident codewords take
+// whole turns of them, a row of two codewords takes 1.6 times as long as a row of one, and K slots in
+// step 5 % and 2 % each, as some of many codewords end in every iteration and hold up the others.
+static double lspa_cost(int64_t n, int G, int K, int V, int warps)
+{
+    double turns = (double)((n + V - 1) / V) / G;
+    turns = turns < 8.0 ? ceil(turns) : turns + 0.5;
+    return turns * (warps > 20 ? warps : 20) * (V == 2 ? 1.6 : 1.0) * (K > 1 ? 1.05 + 0.02 * (K - 1) : 1.0);
 }
 
 template <int DMAX, int V, typename MsgT, bool HC>
 static cudaError_t launch_lspa(const CodeDev *d, const LayeredSpaArgs &a, size_t smem, int64_t ctas, cudaStream_t s)
 {
+    const unsigned threads = a.G / a.K * a.TPG;
+    if (a.K > 1) {
+        cudaError_t e = ensure_smem<k_layered_spa_packed<DMAX, V, MsgT, HC>>(smem);
+        if (e != cudaSuccess) return e;
+        LaunchScope ls(F_LAYERED_SPA, s);
+        k_layered_spa_packed<DMAX, V, MsgT, HC><<<(unsigned)ctas, threads, smem, s>>>(d, a);
+        return cudaGetLastError();
+    }
     cudaError_t e = ensure_smem<k_layered_spa<DMAX, V, MsgT, HC>>(smem);
     if (e != cudaSuccess) return e;
     LaunchScope ls(F_LAYERED_SPA, s);
-    k_layered_spa<DMAX, V, MsgT, HC><<<(unsigned)ctas, a.G * a.TPG, smem, s>>>(d, a);
+    k_layered_spa<DMAX, V, MsgT, HC><<<(unsigned)ctas, threads, smem, s>>>(d, a);
     return cudaGetLastError();
 }
 
@@ -561,8 +751,38 @@ cudaError_t layered_spa_decode(const CodeDev &h, const CodeDev *d, const ldpc_de
     // to a thread: FP16 messages, rows of degree <= 8.  (8192 codewords on GB300, one against two:
     // N = 1944 rate 1/2 FP16 507 / 467 us, 10 slots against 6 pairs; FP32 486 / 597, 7 against 3;
     // rate 5/6 FP16 489 / 545: there single slots of more warps win.)
-    const int V = f16 && h.dc_max <= 8 && per_sm > g1 && 2 * g2 > g1 ? 2 : 1;
+    const bool pairs = f16 && h.dc_max <= 8;
+    int V = pairs && per_sm > g1 && 2 * g2 > g1 ? 2 : 1;
+    const int wt = (h.Z + 31) & ~31;
     LayeredSpaArgs a;
+    a.G = V == 2 ? g2 : g1;
+    a.K = 1;
+    a.TPG = wt;
+    if (a.G < 1) return cudaErrorInvalidValue;
+    // thread slots end to end in a warp where two fifths of the lanes would be idle and that is estimated
+    // 5 % cheaper.  (GB300, 12 x 24 code, us per launch, whole warps / packed: Z = 8 FP32 65536 codewords
+    // 2226 / 910, Z = 16 FP16 41472 1345 / 1071, Z = 33 FP32 20107 1826 / 1454, Z = 36 FP32 18432 1498 /
+    // 1282; with fewer lanes idle whole warps win, as codewords do not wait for one another: Z = 24 FP32
+    // 1003 / 1129, Z = 70 FP32 1202 / 1547.)
+    if (5 * h.Z <= 3 * wt && per_sm > 1) {
+        double cost = lspa_cost(per_sm, a.G, 1, V, a.G * wt / 32) / 1.05;
+        for (int v = 1; v <= (pairs ? 2 : 1); v++) {
+            const int tmax = lspa_threads(h.dc_max <= 8 ? 8 : 32, v, f16), room = lspa_room(h, p.msg, v, v == 2 ? cap2 : cap1);
+            for (int K = 2; K <= room && K * v <= 32 && K * h.Z <= tmax; K++) {
+                const int tpg = (K * h.Z + 31) & ~31;
+                int n = tmax / tpg < room / K ? tmax / tpg : room / K;
+                if (tpg > 32 && n > 15) n = 15;  // named barriers
+                const double c = lspa_cost(per_sm, n * K, K, v, n * tpg / 32);
+                if (c < cost * 0.999) {
+                    cost = c;
+                    V = v;
+                    a.G = n * K;
+                    a.K = K;
+                    a.TPG = tpg;
+                }
+            }
+        }
+    }
     a.llr = llr;
     a.n_cw = n_cw;
     a.bits = bits;
@@ -574,9 +794,6 @@ cudaError_t layered_spa_decode(const CodeDev &h, const CodeDev *d, const ldpc_de
     a.mb = h.mb;
     a.nb = h.nb;
     a.nnz = h.nnz;
-    a.G = V == 2 ? g2 : g1;
-    if (a.G < 1) return cudaErrorInvalidValue;
-    a.TPG = ((h.Z + 31) / 32) * 32;
     const int SA = 4 * V, SR = (f16 ? 2 : 4) * V;
     a.tab0 = (a.G * V * (int)sizeof(LspaBook) + 15) & ~15;
     a.slots0 = a.tab0 + 16 * h.nnz;
