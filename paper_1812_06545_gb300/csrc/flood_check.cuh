@@ -467,4 +467,31 @@ __device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, 
     }
 }
 
+// ------------------------------------------------------------------ rows end to end over warps
+//
+// A warp whose lanes are at rows of different degree takes them in turns of one body each, agreed on by
+// a vote; a lane without a row for that body repeats another's loads and stores nothing.
+
+constexpr unsigned kFullWarp = 0xffffffffu;
+constexpr int kNoRow = 255;  // above any degree
+
+// The body that rows of degree dc share: exact up to 8, then up to 12, 16, 24, 32.
+__device__ __forceinline__ int body_of(int dc) { return dc <= 8 ? dc : dc <= 12 ? 12 : dc <= 16 ? 16 : dc <= 24 ? 24 : dc <= 32 ? 32 : dc; }
+
+// The first body any lane is at (kNoRow: none has a row left); hd: a lane's row << 8 | degree (kNoRow: none),
+// afterwards a row for that body; on: whether it is the lane's own.
+__device__ __forceinline__ int vote_body(int &hd, bool &on)
+{
+    const int mine = body_of(hd & 255);
+    const int body = (int)__reduce_min_sync(kFullWarp, (unsigned)mine);
+    on = mine == body && body != kNoRow;
+    const unsigned m = __ballot_sync(kFullWarp, on);
+    const int hs = __shfl_sync(kFullWarp, hd, m ? __ffs(m) - 1 : 0);
+    if (!on) hd = hs;
+    return body;
+}
+
+__device__ __forceinline__ float pick(bool c, float a, float b) { return c ? a : b; }
+__device__ __forceinline__ float2 pick(bool c, float2 a, float2 b) { return make_float2(c ? a.x : b.x, c ? a.y : b.y); }
+
 }  // namespace ldpc

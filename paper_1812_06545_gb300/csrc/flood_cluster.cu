@@ -26,13 +26,15 @@
 // costs no parallelism.  Variable-node threads: W4 groups; a thread owns four consecutive positions
 // of its group's columns, one access per block (where Z is a multiple of 4; else its two rows'
 // positions).  Rows and columns are dealt to the groups by weight on the host, because a phase ends
-// at a cluster barrier.  The table entries hold complete shared::cluster addresses (own CTA or the other),
+// at a cluster barrier.  Where groups of whole warps would leave too many lanes idle, rows and columns lie
+// end to end over the threads instead (cl_rows_spread).  The table entries hold complete shared::cluster addresses (own CTA or the other),
 // so an operand in either CTA costs one add.
 // Measured on 2048 codewords of the N = 26112 code, FP16, 2.0 dB, per launch, and warp
 // instructions per edge update (both phases): one row and one position per thread 5378 us, 57; two
 // rows 5087 us, 49; and four positions 4706 us, 43; dealt by weight (not back and forth) 4609 us.
 // Bound by instruction issue (58 %) and the waits at the two cluster barriers of a round (15 % of a
 // warp's time).
+#include <math.h>
 #include <string.h>
 
 #include "flood_check.cuh"
@@ -58,6 +60,7 @@ struct ClusterArgs {
     // the variable-node phase in quads: W4 groups of WT4 threads, wt4 = the warps' worth of quads
     // of a column (W4 = 0: Z is no multiple of 4)
     int W4, WT4, wt4, wide_L;
+    int spread;  // rows and columns end to end over the threads instead
     int64_t n_items;
     unsigned long long *next;
     int row_split[CLUSTER_CTAS + 1];  // block rows [row_split[q], row_split[q+1]) belong to CTA q
@@ -313,6 +316,106 @@ __device__ __forceinline__ void cl_cols(const uint8_t *cend, const int4 *__restr
     if constexpr (DV < 5) cl_cols<DV + 1>(cend, ctab, tab, cols, p, Z, i);
 }
 
+// Rows and positions end to end over the CTA's threads (SPREAD), for widths that whole warps fit badly:
+// thread x has rows r and r + H of list row i, where i H + r = x, x + threads, ...; a warp's lanes can
+// be at two or more rows (flood_check.cuh, vote_body).
+template <int DMAX, typename MsgT, bool HC>
+__device__ __forceinline__ void cl_rows_spread(const int4 *__restrict__ tab, const int32_t *__restrict__ rows, int n_rows,
+                                               const ClusterMem<MsgT> mem, int Z, int H, int tid, int nth, float Xb,
+                                               float Pb, uint32_t (&pbad)[2])
+{
+    int i = tid / H, r = tid - i * H;
+    const int di = nth / H, dr = nth - di * H;
+    for (;;) {
+        int hd = i < n_rows ? rows[i] : kNoRow;
+        bool on;
+        const int body = vote_body(hd, on), dc = hd & 255;
+        if (body == kNoRow) break;
+        const int4 *ed = tab + (hd >> 8);
+        PairPlace p;
+        p.own = on;
+        p.own2 = on && r + H < Z;
+        p.r = r;
+        p.s = r + H < Z ? r + H : Z - 1;
+        p.rw = p.r - Z;
+        p.sw = p.s - Z;
+        switch (body) {
+        case 2: check_narrow<2, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        case 3: check_narrow<3, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        case 4: check_narrow<4, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        case 5: check_narrow<5, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        case 6: check_narrow<6, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        case 7: check_narrow<7, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        case 8: check_narrow<8, 2, MsgT, false, HC>(ed, mem, p, Xb, Pb, pbad); break;
+        default:
+            if constexpr (DMAX > 8) {
+                if (body == 12)
+                    check_12<2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
+                else if constexpr (DMAX > 12)
+                    check_wide<0, 2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
+            }
+        }
+        if (on) {
+            i += di;
+            r += dr;
+            if (r >= H) {
+                r -= H;
+                i++;
+            }
+        }
+    }
+}
+
+// The same of the columns, Q positions (pairs or quads) each; at(r): the thread's place at position r.
+template <typename VAR, typename AT>
+__device__ __forceinline__ void cl_cols_spread(const uint8_t *cend, const int4 *__restrict__ ctab,
+                                               const int4 *__restrict__ tab, const int32_t *__restrict__ cols, int n_cols,
+                                               int Z, int Q, int tid, int nth, AT at)
+{
+    int i = tid / Q, r = tid - i * Q;
+    const int di = nth / Q, dr = nth - di * Q;
+    for (; __any_sync(kFullWarp, i < n_cols);) {
+        const bool ok = i < n_cols;
+        const int ic = ok ? i : n_cols - 1, jw = cols[ic];
+        const int dv = 1 + (ic >= cend[0]) + (ic >= cend[1]) + (ic >= cend[2]) + (ic >= cend[3]);  // 5: above 4
+        const int top = (int)__reduce_max_sync(kFullWarp, ok ? (unsigned)dv : 0u);
+        const int4 o = ctab[ic];
+        const VAR p = at(r, ok);
+        float2 s[VAR::NV];
+        p.channel((jw & 255) * Z, s);
+        auto add = [&](bool c, int addr) {  // (a lane without a message there reads its first once more)
+            float2 m[VAR::NV];
+#pragma unroll
+            for (int v = 0; v < VAR::NV; v++) m[v] = s[v];
+            p.add(m, c ? addr : o.x);
+#pragma unroll
+            for (int v = 0; v < VAR::NV; v++) s[v] = pick(c, m[v], s[v]);
+        };
+        p.add(s, o.x);
+        if (top > 1) add(dv > 1, o.y);
+        if (top > 2) add(dv > 2, o.z);
+        if (top > 3) add(dv == 4, o.w);
+        if (top > 4) {
+            int k = dv == 5 ? o.w & 255 : 0;
+            const int4 *m = tab + (dv == 5 ? o.w >> 8 : 0);
+            for (; __any_sync(kFullWarp, k > 0); k -= 4, m++) {
+                const int4 e = k > 0 ? *m : o;
+                add(k > 0, e.x);
+                add(k > 1, e.y);
+                add(k > 2, e.z);
+                add(k > 3, e.w);
+            }
+        }
+        p.put((jw >> 8) * Z, s);
+        i += di;
+        r += dr;
+        if (r >= Q) {
+            r -= Q;
+            i++;
+        }
+    }
+}
+
 // Shared memory ahead of the posterior array (flags, codeword, tables; see the kernel).
 __host__ __device__ inline size_t cl_tables_bytes(int nnz)
 {
@@ -323,7 +426,7 @@ __host__ __device__ inline size_t cl_tables_bytes(int nnz)
 template <int DMAX>
 constexpr int cl_threads() { return DMAX <= 12 ? 768 : 512; }
 
-template <int DMAX, typename MsgT, bool HC>
+template <int DMAX, typename MsgT, bool HC, bool SPREAD>
 __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_threads<DMAX>(), 1)
     k_flood_cluster(const CodeDev *__restrict__ cd, const __grid_constant__ ClusterArgs a)
 {
@@ -412,13 +515,18 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
         if (tid == 0) flags[0] = flags[1] = 0;
         // load: APP = L (+0: no -0) for owned variables, messages 0 for owned edges
         const float *L = static_cast<const float *>(req.llr) + cw * N;
-        for (int r = ru; works && r < Z; r += WT)
-            for (int i = w0; i < n_cols; i += W) {
-                const int jw = cols[i];
-                const float v = __ldg(L + (jw & 255) * Z + r);
-                if (!isfinite(v)) atomicOr(cd->status, IN_NONFINITE);
-                app[(jw >> 8) * Z + r] = v + 0.0f;
-            }
+        auto load = [&](int i, int r) {
+            const int jw = cols[i];
+            const float v = __ldg(L + (jw & 255) * Z + r);
+            if (!isfinite(v)) atomicOr(cd->status, IN_NONFINITE);
+            app[(jw >> 8) * Z + r] = v + 0.0f;
+        };
+        if constexpr (SPREAD) {
+            for (int x = tid; x < n_cols * Z; x += nth) load(x / Z, x % Z);
+        } else {
+            for (int r = ru; works && r < Z; r += WT)
+                for (int i = w0; i < n_cols; i += W) load(i, r);
+        }
         for (int i = tid; i < (blk1 - blk0) * Z; i += nth) R[i] = MsgT(0.0f);
         cl_sync();
         int t = 0;
@@ -427,7 +535,12 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             const int tr = t;  // this round's flag is flags[tr & 1]
             // ---------------- check-node phase over the owned checks
             uint32_t bad = 0;
-            if (works)
+            if constexpr (SPREAD) {
+                uint32_t pbad[2] = {0, 0};
+                cl_rows_spread<DMAX, MsgT, HC>(tab, rows, n_rows, ClusterMem<MsgT>{reinterpret_cast<char *>(smem)}, Z, H,
+                                               tid, nth, Xb, Pb, pbad);
+                bad = pbad[0] | pbad[1];
+            } else if (works)
                 for (int rr = 0; rr < wt; rr += WT) {
                     PairPlace p;
                     const int r = rr + ru;
@@ -452,7 +565,22 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
             const bool conv = tr >= 1 && a.early_exit && flags[tr & 1] == 0;
             if (!__any_sync(0xffffffffu, conv)) {
                 // ---------------- variable-node phase over the owned variables
-                if (a.W4 > 0) {
+                if constexpr (SPREAD) {
+                    if (Z % 4 == 0) {
+                        const bool wide = a.wide_L;
+                        cl_cols_spread<VarQuad<MsgT>>(a.cend[q][0], ctab, tab, cols, n_cols, Z, Z / 4, tid, nth,
+                                                      [&](int r, bool ok) {
+                            return VarQuad<MsgT>{L + 4 * r, (uint32_t)(4 * SR * r), app + 4 * r, ok, wide};
+                        });
+                    } else {
+                        cl_cols_spread<VarPair<MsgT>>(a.cend[q][0], ctab, tab, cols, n_cols, Z, H, tid, nth,
+                                                      [&](int r, bool ok) {
+                            const int s = r + H < Z ? r + H : Z - 1;
+                            return VarPair<MsgT>{L + r,   L + s,   (uint32_t)(SR * r), (uint32_t)(SR * s),
+                                                 app + r, app + s, ok,                 ok && r + H < Z};
+                        });
+                    }
+                } else if (a.W4 > 0) {
                     const bool wide = a.wide_L;
                     for (int qq = 0; qq < a.wt4; qq += a.WT4) {
                         const int x = qq + ru4, xc = 4 * x < Z ? 4 * x : Z - 4;
@@ -478,13 +606,18 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
         // output: each CTA writes its variables
         uint8_t *Bo = req.bits + cw * N;
         float *Ao = req.app ? req.app + cw * N : nullptr;
-        for (int r = ru; works && r < Z; r += WT)
-            for (int i = w0; i < n_cols; i += W) {
-                const int jw = cols[i], n = (jw & 255) * Z + r;
-                const float v = app[(jw >> 8) * Z + r];
-                Bo[n] = v < 0.0f ? 1 : 0;
-                if (Ao) Ao[n] = v;
-            }
+        auto store = [&](int i, int r) {
+            const int jw = cols[i], n = (jw & 255) * Z + r;
+            const float v = app[(jw >> 8) * Z + r];
+            Bo[n] = v < 0.0f ? 1 : 0;
+            if (Ao) Ao[n] = v;
+        };
+        if constexpr (SPREAD) {
+            for (int x = tid; x < n_cols * Z; x += nth) store(x / Z, x % Z);
+        } else {
+            for (int r = ru; works && r < Z; r += WT)
+                for (int i = w0; i < n_cols; i += W) store(i, r);
+        }
         if (q == 0 && tid == 0) req.iters[cw] = t;
     }
     cl_sync();  // no CTA leaves while another may still read its shared memory
@@ -563,6 +696,22 @@ static size_t cl_plan(const CodeDev &h, int msg, ClusterArgs &a, size_t limit)
     a.wt4 = (a.Z / 4 + 31) & ~31;
     a.WT4 = a.Z % 4 ? 32 : a.wt4 <= nth ? a.wt4 : nth;
     a.W4 = a.Z % 4 ? 0 : nth / a.WT4;
+    // end to end over the threads where that leaves so few turns of the rows (about two thirds of the
+    // time) and the columns that it pays for the votes.  (GB300, FP16, us per launch, groups of whole
+    // warps / end to end: 512 codewords of a 64 x 128 code of 1024 blocks, Z = 130 2167 / 1643, Z = 136
+    // 2024 / 1486; 1024 of a 34 x 68 code, Z = 260 2065 / 1664; FP32, 64 x 128, Z = 68 1184 / 954.)
+    const int Q = a.Z % 4 ? a.H : a.Z / 4, Wc = a.W4 ? a.W4 : a.W;
+    double whole[2] = {}, spread[2] = {};  // turns of rows and columns, of the slower CTA
+    for (int q = 0; q < CLUSTER_CTAS; q++) {
+        const int n[2] = {a.row_split[q + 1] - a.row_split[q], a.ncols[q]}, w[2] = {a.W, Wc}, p[2] = {a.H, Q};
+        for (int i = 0; i < 2; i++) {
+            whole[i] = fmax(whole[i], (n[i] + w[i] - 1) / w[i]);
+            spread[i] = fmax(spread[i], (n[i] * p[i] + nth - 1) / nth);
+        }
+    }
+    const double gain = 0.65 * spread[0] / whole[0] + 0.35 * spread[1] / whole[1];
+    a.spread = gain * (1.0 + 2.1 * h.mb / h.nnz) * 1.05 < 1.0;
+    if (a.spread) a.W = a.W4 = 1;  // one list of each
     // the CTAs' lists, and the size of their tables.  A phase ends at a cluster barrier, so its
     // rows (columns) go to the groups by weight, heaviest first to the least loaded group
     size_t tables = cl_tables_bytes(h.nnz);
@@ -647,10 +796,10 @@ int cluster_supported(const CodeDev &h, int msg)
     return need > 0 && need <= cl_limit();
 }
 
-template <int DMAX, typename MsgT, bool HC>
+template <int DMAX, typename MsgT, bool HC, bool SPREAD>
 static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d, cudaStream_t s)
 {
-    cudaError_t e = ensure_smem<k_flood_cluster<DMAX, MsgT, HC>>(smem);
+    cudaError_t e = ensure_smem<k_flood_cluster<DMAX, MsgT, HC, SPREAD>>(smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CLUSTER_CTAS, 1, 1);
@@ -665,7 +814,7 @@ static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, con
     if (dev < 0 || dev >= 64) dev = 0;
     int clusters = __atomic_load_n(&cached[dev], __ATOMIC_RELAXED);
     if (clusters < 1 || __atomic_load_n(&cached_smem[dev], __ATOMIC_RELAXED) != smem) {
-        e = cudaOccupancyMaxActiveClusters(&clusters, k_flood_cluster<DMAX, MsgT, HC>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&clusters, k_flood_cluster<DMAX, MsgT, HC, SPREAD>, &cfg);
         if (e != cudaSuccess || clusters < 1) {
             cudaGetLastError();
             int nsm = 2;
@@ -680,17 +829,25 @@ static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, con
     for (int i = 0; i < a.n_req; i++)
         if (reinterpret_cast<uintptr_t>(a.reqs[i].llr) & 15) a.wide_L = 0;
     LaunchScope ls(F_SLOTS, s);
-    k_flood_cluster<DMAX, MsgT, HC><<<(unsigned)(clusters * CLUSTER_CTAS), cl_threads<DMAX>(), smem, s>>>(d, a);
+    k_flood_cluster<DMAX, MsgT, HC, SPREAD><<<(unsigned)(clusters * CLUSTER_CTAS), cl_threads<DMAX>(), smem, s>>>(d, a);
     return cudaGetLastError();
 }
 
-template <typename MsgT, bool HC>
+template <typename MsgT, bool HC, bool SPREAD>
 static cudaError_t launch_cluster_d(int dmax, ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d,
                                     cudaStream_t s)
 {
-    if (dmax <= 8) return launch_cluster<8, MsgT, HC>(a, smem, n_cw, d, s);
-    if (dmax <= 12) return launch_cluster<12, MsgT, HC>(a, smem, n_cw, d, s);
-    return launch_cluster<32, MsgT, HC>(a, smem, n_cw, d, s);
+    if (dmax <= 8) return launch_cluster<8, MsgT, HC, SPREAD>(a, smem, n_cw, d, s);
+    if (dmax <= 12) return launch_cluster<12, MsgT, HC, SPREAD>(a, smem, n_cw, d, s);
+    return launch_cluster<32, MsgT, HC, SPREAD>(a, smem, n_cw, d, s);
+}
+
+template <typename MsgT, bool HC>
+static cudaError_t launch_cluster_f(int dmax, ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d,
+                                    cudaStream_t s)
+{
+    return a.spread ? launch_cluster_d<MsgT, HC, true>(dmax, a, smem, n_cw, d, s)
+                    : launch_cluster_d<MsgT, HC, false>(dmax, a, smem, n_cw, d, s);
 }
 
 cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_decode_params &p, const HostReq *reqs,
@@ -724,10 +881,10 @@ cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     if (e != cudaSuccess) return e;
     const bool hc = p.phi_clamp < FLOOD_CLAMP_X;
     if (p.msg == LDPC_MSG_F16)
-        return hc ? launch_cluster_d<__half, true>(h.dc_max, a, smem, items, d, s)
-                  : launch_cluster_d<__half, false>(h.dc_max, a, smem, items, d, s);
-    return hc ? launch_cluster_d<float, true>(h.dc_max, a, smem, items, d, s)
-              : launch_cluster_d<float, false>(h.dc_max, a, smem, items, d, s);
+        return hc ? launch_cluster_f<__half, true>(h.dc_max, a, smem, items, d, s)
+                  : launch_cluster_f<__half, false>(h.dc_max, a, smem, items, d, s);
+    return hc ? launch_cluster_f<float, true>(h.dc_max, a, smem, items, d, s)
+              : launch_cluster_f<float, false>(h.dc_max, a, smem, items, d, s);
 }
 
 }  // namespace ldpc

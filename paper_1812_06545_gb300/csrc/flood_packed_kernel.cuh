@@ -24,15 +24,6 @@
 
 namespace ldpc {
 
-constexpr unsigned kFullWarp = 0xffffffffu;
-constexpr int kNoRow = 255;  // above any degree
-
-__device__ __forceinline__ float pick(bool c, float a, float b) { return c ? a : b; }
-__device__ __forceinline__ float2 pick(bool c, float2 a, float2 b) { return make_float2(c ? a.x : b.x, c ? a.y : b.y); }
-
-// The body that rows of degree dc share (flood_check.cuh): exact up to 8, then up to 12, 16, 24, 32.
-__device__ __forceinline__ int body_of(int dc) { return dc <= 8 ? dc : dc <= 12 ? 12 : dc <= 16 ? 16 : dc <= 24 ? 24 : dc; }
-
 // The check-node phase of one thread: list positions i, i + step, ... (back and forth, as rows_of) below mb.
 // In each turn the warp takes the first body any of its lanes is at.
 template <int DMAX, int V, typename MsgT, bool HC>
@@ -43,13 +34,9 @@ __device__ __forceinline__ void rows_spread(const int4 *__restrict__ tab, const 
     constexpr bool B2 = kSlotB2<MsgT>;
     for (;;) {
         int hd = i < mb ? rows[i] : kNoRow;
-        const int mine = body_of(hd & 255);
-        const int body = (int)__reduce_min_sync(kFullWarp, (unsigned)mine);
+        bool on;
+        const int body = vote_body(hd, on), dc = hd & 255;
         if (body == kNoRow) break;
-        const bool on = mine == body || (body > 24 && mine != kNoRow);
-        const int hs = __shfl_sync(kFullWarp, hd, __ffs(__ballot_sync(kFullWarp, on)) - 1);
-        hd = on ? hd : hs;
-        const int dc = hd & 255;
         const int4 *ed = tab + (hd >> 8);
         Place<V> q = p;
         q.own = p.own && on;
