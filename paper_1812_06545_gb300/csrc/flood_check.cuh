@@ -340,11 +340,11 @@ __device__ __forceinline__ void check_12(int dc, const int4 *__restrict__ ed, co
 
 // Degree 13..32.  Between the passes an FP32 message's word holds its edge's d (N is dead once
 // Q is formed); with FP16 messages d is formed again from APP and N, or held in registers
-// (one codeword per thread, degree <= 16).  Two codewords per thread (G = 0) run the groups
+// (G = 2: degree <= 16).  Two codewords per thread (G = 0) run the groups
 // in a loop, so that the code of all these degrees is one group's: unrolled, the bodies of a
 // mixed-code launch overflow the instruction cache (its share of stalls was 1.6 per issue).
-// One codeword per thread, the form of small batches, unrolls G groups, whose loads then
-// overlap.
+// One codeword per thread, the form of small batches, and the cluster decoder, whose loads come
+// from the other SM, unroll G groups, whose loads then overlap.
 template <int G, int V, typename MsgT, bool B2, bool HC, typename MEM, typename PL>
 __device__ __forceinline__ void check_wide(int dc, const int4 *__restrict__ ed, const MEM mem, const PL &p,
                                            float Xb, float Pb, uint32_t (&pbad)[V])

@@ -23,7 +23,9 @@
 // r + ceil(Z / 2) of the block rows that fall to its group in ascending degree, so that a warp runs
 // one straight-line body at a time (flood_check.cuh) with two rows' arithmetic packed and one read
 // of each edge descriptor.  One CTA has several times more rows than threads, so that pairing them
-// costs no parallelism.  Variable-node threads: W4 groups; a thread owns four consecutive positions
+// costs no parallelism.  Rows above degree 12 have their groups of edges unrolled, whose remote loads
+// then overlap (600 codewords of a 42 x 84 code, Z = 136, FP16: rows of 13 to 15 edges 1628 -> 1017 us, of
+// 19 to 21 2054 -> 1364).  Variable-node threads: W4 groups; a thread owns four consecutive positions
 // of its group's columns, one access per block (where Z is a multiple of 4; else its two rows'
 // positions).  Rows and columns are dealt to the groups by weight on the host, because a phase ends
 // at a cluster barrier.  Where groups of whole warps would leave too many lanes idle, rows and columns lie
@@ -205,7 +207,7 @@ __device__ __forceinline__ void cl_rows(const uint8_t *rend, const int4 *__restr
             else if constexpr (D == 12)
                 check_12<2, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
             else
-                check_wide<0, 2, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
+                check_wide<D / 8, 2, MsgT, false, HC>(hd & 255, tab + (hd >> 8), mem, p, Xb, Pb, pbad);
         }
         if constexpr (CLS + 1 < CL_CLASSES)
             cl_rows<CLS + 1, DMAX, MsgT, HC>(rend, tab, rows, mem, p, Xb, Pb, pbad, i);
@@ -351,8 +353,14 @@ __device__ __forceinline__ void cl_rows_spread(const int4 *__restrict__ tab, con
             if constexpr (DMAX > 8) {
                 if (body == 12)
                     check_12<2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
-                else if constexpr (DMAX > 12)
-                    check_wide<0, 2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
+                else if constexpr (DMAX > 12) {
+                    if (body == 16)
+                        check_wide<2, 2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
+                    else if (body == 24)
+                        check_wide<3, 2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
+                    else
+                        check_wide<4, 2, MsgT, false, HC>(dc, ed, mem, p, Xb, Pb, pbad);
+                }
             }
         }
         if (on) {
