@@ -39,6 +39,8 @@
 #include <math.h>
 #include <string.h>
 
+#include <new>
+
 #include "flood_check.cuh"
 
 namespace ldpc {
@@ -793,16 +795,27 @@ static size_t cl_limit()
     return lim > 0 ? (size_t)lim : 227 * 1024;
 }
 
-int cluster_supported(const CodeDev &h, int msg)
+struct ClusterPlan {
+    ClusterArgs a;  // all but the requests and parameters of a call
+    size_t smem;
+};
+
+// (Planned once: forming it anew took 9 us of the host, three times per call.)
+ClusterPlan *cluster_plan_create(const CodeDev &h, int msg)
 {
-    if (h.dc_max > 32 || h.mb < CLUSTER_CTAS || h.nb < CLUSTER_CTAS) return 0;
-    if ((int64_t)h.N >= (1 << 19) || (int64_t)h.E >= (1 << 20))
-        return 0;  // the packed table fields (posterior and message bases)
-    ClusterArgs a;
-    memset(&a, 0, sizeof a);
-    const size_t need = cl_plan(h, msg, a, cl_limit());
-    return need > 0 && need <= cl_limit();
+    if (h.dc_max > 32 || h.mb < CLUSTER_CTAS || h.nb < CLUSTER_CTAS) return nullptr;
+    ClusterPlan *q = new (std::nothrow) ClusterPlan;
+    if (!q) return nullptr;
+    memset(q, 0, sizeof *q);
+    q->smem = cl_plan(h, msg, q->a, cl_limit());
+    if (q->smem == 0 || q->smem > cl_limit()) {
+        delete q;
+        return nullptr;
+    }
+    return q;
 }
+
+void cluster_plan_free(ClusterPlan *plan) { delete plan; }
 
 template <int DMAX, typename MsgT, bool HC, bool SPREAD>
 static cudaError_t launch_cluster(ClusterArgs &a, size_t smem, int64_t n_cw, const CodeDev *d, cudaStream_t s)
@@ -858,14 +871,13 @@ static cudaError_t launch_cluster_f(int dmax, ClusterArgs &a, size_t smem, int64
                     : launch_cluster_d<MsgT, HC, false>(dmax, a, smem, n_cw, d, s);
 }
 
-cudaError_t flood_cluster_decode(const CodeDev &h, const CodeDev *d, const ldpc_decode_params &p, const HostReq *reqs,
-                                 int n, void *counter, cudaStream_t s)
+cudaError_t flood_cluster_decode(const ClusterPlan &plan, const CodeDev &h, const CodeDev *d,
+                                 const ldpc_decode_params &p, const HostReq *reqs, int n, void *counter,
+                                 cudaStream_t s)
 {
     if (n < 1 || n > MULTI_MAX_REQS) return cudaErrorInvalidValue;
-    ClusterArgs a;
-    memset(&a, 0, sizeof a);
-    const size_t smem = cl_plan(h, p.msg, a, cl_limit());
-    if (smem == 0) return cudaErrorInvalidValue;
+    ClusterArgs a = plan.a;
+    const size_t smem = plan.smem;
     int64_t items = 0;
     for (int i = 0; i < n; i++) {
         if (reqs[i].n_cw <= 0) continue;

@@ -79,11 +79,14 @@ static int sm_count()
     return g_sm_count[dev];
 }
 
-static size_t max_smem_optin()
+static size_t max_smem_optin()  // (asked for once per device)
 {
+    static int cached[64];
     int dev = 0, v = 0;
     cudaGetDevice(&dev);
+    if (dev >= 0 && dev < 64 && (v = __atomic_load_n(&cached[dev], __ATOMIC_RELAXED)) > 0) return (size_t)v;
     cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (dev >= 0 && dev < 64 && v > 0) __atomic_store_n(&cached[dev], v, __ATOMIC_RELAXED);
     return v > 0 ? (size_t)v : 227 * 1024;
 }
 

@@ -235,6 +235,7 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
     memset(&c->host, 0, sizeof c->host);
     c->dev = nullptr;
     c->pool = nullptr;
+    c->cluster[0] = c->cluster[1] = nullptr;
     c->tuned_flood[0] = c->tuned_flood[1] = SCHED_UNTUNED;
     c->tuned_layered = SCHED_UNTUNED;
     CodeDev &h = c->host;
@@ -302,6 +303,11 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
         for (int v = 0; v < 4; v++)
             ldpc::flood_build_table(h, v < 2 ? LDPC_MSG_F32 : LDPC_MSG_F16, 1 + (v & 1), tab + (size_t)v * h.n_ftab);
     memcpy(img.data(), &h, sizeof h);
+    for (int f = 0; f < 2; f++) {
+        const int msg = f ? LDPC_MSG_F16 : LDPC_MSG_F32;
+        c->slots[f] = ldpc::slots_supported(h, msg);
+        c->pairs[f] = ldpc::slots_pairable(h, msg);
+    }
     if (e == cudaSuccess) e = cudaMalloc(&c->dev, img.size());
     if (e == cudaSuccess) e = cudaMemcpy(c->dev, img.data(), img.size(), cudaMemcpyHostToDevice);
     c->ftab = reinterpret_cast<int4 *>(reinterpret_cast<char *>(c->dev) + head);
@@ -310,6 +316,7 @@ ldpc_status ldpc_code_create(const int32_t *base, int32_t mb, int32_t nb, int32_
         delete c;
         return cuda_fail(e, "device code tables");
     }
+    for (int f = 0; f < 2; f++) c->cluster[f] = ldpc::cluster_plan_create(h, f ? LDPC_MSG_F16 : LDPC_MSG_F32);
     c->sms = 0;
     if (cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) cudaGetLastError();
     c->pool = ldpc::pool_acquire(c->device);
@@ -322,6 +329,7 @@ void ldpc_code_destroy(ldpc_code *c)
     if (!c) return;
     if (c->dev) cudaFree(c->dev);
     ldpc::pool_release(c->device, c->pool);
+    for (ldpc::ClusterPlan *q : c->cluster) ldpc::cluster_plan_free(q);
     delete c;
 }
 
@@ -334,6 +342,8 @@ ldpc_status ldpc_code_info(const ldpc_code *c, int32_t *N, int32_t *K, int32_t *
     if (E) *E = c->host.E;
     return LDPC_OK;
 }
+
+static int msg_index(const ldpc_decode_params *p) { return p->msg == LDPC_MSG_F16 ? 1 : 0; }
 
 static ldpc_status check_params(const ldpc_code *c, const ldpc_decode_params *p, int llr_type)
 {
@@ -353,7 +363,7 @@ static ldpc_status check_params(const ldpc_code *c, const ldpc_decode_params *p,
         if (llr_type != LDPC_LLR_F32) return fail(LDPC_EINVAL, "flooding SPA takes fp32 LLRs");
         if (p->impl == LDPC_IMPL_PLAIN && p->msg != LDPC_MSG_F32)
             return fail(LDPC_ENOTSUP, "the plain comparator stores F32 messages");
-        if (p->impl == LDPC_IMPL_CLUSTER && !ldpc::cluster_supported(c->host, p->msg))
+        if (p->impl == LDPC_IMPL_CLUSTER && !c->cluster[msg_index(p)])
             return fail(LDPC_ENOTSUP, "code does not fit the cluster decoder");
         if (c->host.dc_max > 32) return fail(LDPC_ENOTSUP, "check degree %d > 32", c->host.dc_max);
         return LDPC_OK;
@@ -394,8 +404,8 @@ static ldpc_status check_params(const ldpc_code *c, const ldpc_decode_params *p,
 // a CTA's shared memory; LDPC_IMPL_STREAMING and the plain comparator use the HBM layout.
 static bool use_slots(const ldpc_code *c, const ldpc_decode_params *p)
 {
-    return p->sched == LDPC_SCHED_FLOODING && p->impl == LDPC_IMPL_AUTO && ldpc::slots_supported(c->host, p->msg) &&
-           c->tuned_flood[p->msg == LDPC_MSG_F16 ? 1 : 0] != SCHED_STREAMING;
+    return p->sched == LDPC_SCHED_FLOODING && p->impl == LDPC_IMPL_AUTO && c->slots[msg_index(p)] &&
+           c->tuned_flood[msg_index(p)] != SCHED_STREAMING;
 }
 
 // The cluster decoder serves flooding codes whose codeword does not fit one CTA (AUTO), or
@@ -404,8 +414,8 @@ static bool use_cluster(const ldpc_code *c, const ldpc_decode_params *p)
 {
     if (p->sched != LDPC_SCHED_FLOODING) return false;
     if (p->impl == LDPC_IMPL_CLUSTER) return true;
-    return p->impl == LDPC_IMPL_AUTO && !ldpc::slots_supported(c->host, p->msg) &&
-           ldpc::cluster_supported(c->host, p->msg) && c->tuned_flood[p->msg == LDPC_MSG_F16 ? 1 : 0] != SCHED_STREAMING;
+    return p->impl == LDPC_IMPL_AUTO && !c->slots[msg_index(p)] && c->cluster[msg_index(p)] &&
+           c->tuned_flood[msg_index(p)] != SCHED_STREAMING;
 }
 
 // The layered min-sum runs as persistent slots (work counter in the workspace) unless
@@ -512,7 +522,7 @@ ldpc_status ldpc_decode_batch(const ldpc_code *c, const ldpc_decode_params *p, c
         e = ldpc::flood_multi_decode(&rq, 1, *p, ws, s);
     } else if (use_cluster(c, p)) {
         const ldpc::HostReq rq = {c, llr, n_cw, bits, iters, app};
-        e = ldpc::flood_cluster_decode(c->host, c->dev, *p, &rq, 1, ws, s);
+        e = ldpc::flood_cluster_decode(*c->cluster[msg_index(p)], c->host, c->dev, *p, &rq, 1, ws, s);
     } else {
         ldpc::FloodWs w;
         ldpc::flood_ws_layout(c->host, n_cw, p->msg, &w, static_cast<char *>(ws));
@@ -592,7 +602,8 @@ ldpc_status ldpc_decode_multi(const ldpc_request *reqs, int32_t n_req, const ldp
                     same[nsame++] = hr[k];
                     done_req[k] = true;
                 }
-            e = ldpc::flood_cluster_decode(hr[i].code->host, hr[i].code->dev, *p, same, nsame, ws, s);
+            e = ldpc::flood_cluster_decode(*hr[i].code->cluster[msg_index(p)], hr[i].code->host, hr[i].code->dev, *p,
+                                           same, nsame, ws, s);
         }
     } else {
         e = cudaSuccess;
@@ -636,13 +647,13 @@ ldpc_status ldpc_autotune(ldpc_code *c, const ldpc_decode_params *p, const void 
     if (use_layered_spa(p)) return fail(LDPC_ENOTSUP, "layered SPA has a single schedule: nothing to tune");
     if (n_cw < 1 || !llr) return fail(LDPC_EINVAL, "autotuning needs a non-empty sample of LLRs");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    int *slot = p->sched == LDPC_SCHED_FLOODING ? &c->tuned_flood[p->msg == LDPC_MSG_F16 ? 1 : 0] : &c->tuned_layered;
+    int *slot = p->sched == LDPC_SCHED_FLOODING ? &c->tuned_flood[msg_index(p)] : &c->tuned_layered;
     int cand[3], nc = 0;
     if (p->sched == LDPC_SCHED_FLOODING) {
-        if (ldpc::slots_supported(c->host, p->msg)) {
+        if (c->slots[msg_index(p)]) {
             cand[nc++] = SCHED_SLOTS_V1;
-            if (ldpc::slots_pairable(c->host, p->msg)) cand[nc++] = SCHED_SLOTS_V2;
-        } else if (ldpc::cluster_supported(c->host, p->msg)) {
+            if (c->pairs[msg_index(p)]) cand[nc++] = SCHED_SLOTS_V2;
+        } else if (c->cluster[msg_index(p)]) {
             cand[nc++] = SCHED_SLOTS_V1;  // the cluster decoder
         }
     } else if (ldpc::layered_slots_per_cta(c->host) > 0) {

@@ -118,9 +118,14 @@ constexpr float FLOOD_CLAMP_X = 40.0f;
 
 // Flooding SPA cluster decoder (flood_cluster.cu): one codeword per two-SM cluster, for codes
 // whose codeword does not fit one CTA; every codeword of n requests of one code in one launch.
-int cluster_supported(const CodeDev &host, int msg);
-cudaError_t flood_cluster_decode(const CodeDev &host, const CodeDev *dev, const ldpc_decode_params &p,
-                                 const HostReq *reqs, int n, void *counter, cudaStream_t s);
+// The plan (how the codeword is split and dealt out) depends on the code and message type alone:
+// made when the code is created, null when the code does not fit.
+struct ClusterPlan;
+ClusterPlan *cluster_plan_create(const CodeDev &host, int msg);
+void cluster_plan_free(ClusterPlan *plan);
+cudaError_t flood_cluster_decode(const ClusterPlan &plan, const CodeDev &host, const CodeDev *dev,
+                                 const ldpc_decode_params &p, const HostReq *reqs, int n, void *counter,
+                                 cudaStream_t s);
 
 // Flooding SPA slot decoder: supported when one codeword of the code fits a CTA.
 int slots_supported(const CodeDev &host, int msg);
@@ -150,7 +155,11 @@ struct ldpc_code {
     int sms;             // SMs of the device
     cudaMemPool_t pool;  // the device's scratch pool (shared with its other codes), or null
     int4 *ftab;          // flooding slot decoder's tables: [2 * (F16) + V - 1][host.n_ftab] (flood_slots.h)
-    int tuned_flood[2];  // per message type (F32, F16)
+    // flooding decoders that serve the code, per message type (F32, F16): slots with one codeword per
+    // thread, with two, and the cluster decoder's plan (null: it does not fit)
+    bool slots[2], pairs[2];
+    ldpc::ClusterPlan *cluster[2];
+    int tuned_flood[2];
     int tuned_layered;
 };
 
