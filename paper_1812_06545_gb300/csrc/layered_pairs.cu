@@ -288,8 +288,8 @@ __device__ __forceinline__ void lpair_refill(const LayeredPairArgs &a, const Cod
 // spill; 4193 of the N = 4000 code, dmax 16: 896 326 us, 1024 353.)
 __host__ __device__ constexpr int lpairs_threads(int dmax) { return dmax <= 8 ? 1024 : dmax <= 16 ? 896 : 768; }
 
-template <int DMAX, bool SATAPP, bool TABLE>
-__global__ void __launch_bounds__(lpairs_threads(DMAX), 1)
+template <int DMAX, bool SATAPP, bool TABLE, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1)
     k_layered_pairs(const CodeDev *__restrict__ cd, const __grid_constant__ LayeredPairArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -483,12 +483,12 @@ static int lpairs_stride(int n, int Z, int bytes)
 // The tables' bytes: 16-bit offsets per (block, row), or 8-byte descriptors per block.
 static size_t lpairs_tab(const CodeDev &h, bool table) { return table ? 2 * (size_t)h.nnz * h.Z : 8 * (size_t)h.nnz; }
 
-// Thread slots of two codewords per CTA, at most cap.
-static int lpairs_fit(const CodeDev &h, int cap, bool table)
+// Thread slots of two codewords per CTA of so many threads, at most cap.
+static int lpairs_fit(const CodeDev &h, int cap, bool table, int threads)
 {
     if (h.dc_max > 32 || 4 * h.N > 65535) return 0;
     const int wt = ((h.Z + 31) / 32) * 32, V = 2;
-    int G = lpairs_threads(lpairs_dmax(h)) / wt;
+    int G = threads / wt;
     if (G > cap) G = cap;
     if (G * V > SLOTS_MAX) G = SLOTS_MAX / V;
     if (wt > 32 && G > 15) G = 15;  // named barriers
@@ -505,16 +505,16 @@ int layered_pairs_per_cta(const CodeDev &h)
     const size_t head = ((size_t)SLOTS_MAX * 16 + 16 + tables + 15) & ~(size_t)15;
     auto stride = [&](int n, int m) { return (size_t)(n + (((h.Z % m) - (n % m)) % m + m) % m); };
     if (head + stride(h.N, 32) * 4 + stride(h.E, 64) * 2 + 16 > 227 * 1024) return 0;
-    return 2 * lpairs_fit(h, SLOTS_MAX / 2, false);
+    return 2 * lpairs_fit(h, SLOTS_MAX / 2, false, lpairs_threads(lpairs_dmax(h)));
 }
 
-template <int DMAX, bool SATAPP, bool TABLE>
+template <int DMAX, bool SATAPP, bool TABLE, int THREADS = lpairs_threads(DMAX)>
 static cudaError_t launch_lpairs(const CodeDev *d, const LayeredPairArgs &a, size_t smem, int ctas, cudaStream_t s)
 {
-    cudaError_t e = ensure_smem<k_layered_pairs<DMAX, SATAPP, TABLE>>(smem);
+    cudaError_t e = ensure_smem<k_layered_pairs<DMAX, SATAPP, TABLE, THREADS>>(smem);
     if (e != cudaSuccess) return e;
     LaunchScope ls(F_LAYERED, s);
-    k_layered_pairs<DMAX, SATAPP, TABLE><<<(unsigned)ctas, a.G * a.TPG, smem, s>>>(d, a);
+    k_layered_pairs<DMAX, SATAPP, TABLE, THREADS><<<(unsigned)ctas, a.G * a.TPG, smem, s>>>(d, a);
     return cudaGetLastError();
 }
 
@@ -524,7 +524,9 @@ static cudaError_t launch_lpairs_d(const CodeDev &h, const CodeDev *d, const Lay
 {
     switch (lpairs_dmax(h)) {
     case 8: return launch_lpairs<8, SATAPP, TABLE>(d, a, smem, ctas, s);
-    case 16: return launch_lpairs<16, SATAPP, TABLE>(d, a, smem, ctas, s);
+    case 16:  // (1024 threads only where 896 hold fewer slots)
+        return a.G * a.TPG > lpairs_threads(16) ? launch_lpairs<16, SATAPP, TABLE, 1024>(d, a, smem, ctas, s)
+                                                : launch_lpairs<16, SATAPP, TABLE>(d, a, smem, ctas, s);
     case 24: return launch_lpairs<24, SATAPP, TABLE>(d, a, smem, ctas, s);
     default: return launch_lpairs<32, SATAPP, TABLE>(d, a, smem, ctas, s);
     }
@@ -558,8 +560,20 @@ cudaError_t layered_pairs_decode(const CodeDev &h, const CodeDev *d, const ldpc_
     const int64_t per_cta = (items + nsm - 1) / nsm;
     const int cap = per_cta < SLOTS_MAX ? (int)((per_cta + 1) / 2) : SLOTS_MAX / 2;
     // the offset table where it costs no thread slot
-    const int g = lpairs_fit(h, cap, false);
-    const bool table = lpairs_fit(h, cap, true) == g;
+    int threads = lpairs_threads(lpairs_dmax(h)), g = lpairs_fit(h, cap, false, threads);
+    // rows of 9 to 16 edges in 1024 threads, which spill, where their further thread slots save more than that:
+    // 896 hold one slot of Z in 449..512 and 1024 two (4 x 16 code of Z = 500, 10 iterations, 600 codewords
+    // 149 against 127 us, 12000 2842 against 2367; but Z = 250, 4000 codewords, five turns against four:
+    // 404 against 421)
+    if (threads == 896) {
+        const int wide = lpairs_fit(h, cap, false, 1024);
+        auto turns = [&](int G) { return (int)(((per_cta + 1) / 2 + G - 1) / G); };
+        if (g < 1 || 1.3 * turns(wide) < turns(g)) {
+            threads = 1024;
+            g = wide;
+        }
+    }
+    const bool table = lpairs_fit(h, cap, true, threads) == g;
     constexpr int V = 2;
     a.G = g;
     if (a.G < 1) return cudaErrorInvalidValue;
