@@ -709,7 +709,7 @@ static size_t cl_plan(const CodeDev &h, int msg, ClusterArgs &a, size_t limit)
     // end to end over the threads where that leaves so few turns of the rows (about two thirds of the
     // time) and the columns that it pays for the votes.  (GB300, FP16, us per launch, groups of whole
     // warps / end to end: 512 codewords of a 64 x 128 code of 1024 blocks, Z = 130 2167 / 1643, Z = 136
-    // 2024 / 1486; 1024 of a 34 x 68 code, Z = 260 2065 / 1664; FP32, 64 x 128, Z = 68 1184 / 954.)
+    // 2024 / 1486; 1024 of a 34 x 68 code, Z = 260 2065 / 1664; FP32, 64 x 128, Z = 68 1184 / 954, but 30 x 90, rows of 8, Z = 278, 2334 / 2737.)
     const int Q = a.Z % 4 ? a.H : a.Z / 4, Wc = a.W4 ? a.W4 : a.W;
     double whole[2] = {}, spread[2] = {};  // turns of rows and columns, of the slower CTA
     for (int q = 0; q < CLUSTER_CTAS; q++) {
@@ -720,7 +720,7 @@ static size_t cl_plan(const CodeDev &h, int msg, ClusterArgs &a, size_t limit)
         }
     }
     const double gain = 0.65 * spread[0] / whole[0] + 0.35 * spread[1] / whole[1];
-    a.spread = gain * (1.0 + 2.1 * h.mb / h.nnz) * 1.05 < 1.0;
+    a.spread = gain * (1.0 + 4.3 * h.mb / h.nnz) < 1.0;  // (rows of 9.5 edges take 1.3 to 1.45 times as long)
     if (a.spread) a.W = a.W4 = 1;  // one list of each
     // the CTAs' lists, and the size of their tables.  A phase ends at a cluster barrier, so its
     // rows (columns) go to the groups by weight, heaviest first to the least loaded group

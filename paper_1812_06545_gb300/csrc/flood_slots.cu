@@ -159,7 +159,8 @@ static SlotShape slot_shape(const CodeDev &h, int msg, int V, int dmax, size_t l
 
 // What n codewords cost an SM in a shape of V codewords per thread, as warps times check rows:
 //   a round takes ceil(mb / W) block rows of every warp, and as long as 14 more edges for the rest of it;
-//   fewer than 20 warps take as long as 20 (latency);
+//   fewer than 20 warps take as long as 20 (`least`; 8 where far fewer warps of spread rows above degree 12
+//     stand against whole ones, as such a row has many independent edges);
 //   a few times the resident codewords take whole turns of them;
 //   a row of two codewords takes 1.35 times as long as a row of one (FP16, rows above degree 12, which
 //     spill: 1.55, packed 1.9);
@@ -170,7 +171,8 @@ static SlotShape slot_shape(const CodeDev &h, int msg, int V, int dmax, size_t l
 // Measured (us, whole warps / packed / spread, 10 iterations): at widths without idle lanes, N = 768 rate 1/2,
 // FP32 675 / 711 / 881, rate 5/6 1000 / 1048 / 1190; 600 codewords of a 12 x 24 code of Z = 3 42 / 27 / 27;
 // 39 of a 46 x 92 code of Z = 9 112 / - / 54; 16588 of a rate-5/6 code of Z = 20, FP16 733 / 600 / 712.
-static double shape_cost(const CodeDev &h, int msg, const SlotShape &s, int V, int64_t n, FloodForm form, double change)
+static double shape_cost(const CodeDev &h, int msg, const SlotShape &s, int V, int64_t n, FloodForm form, double change,
+                         double least = 20.0)
 {
     const double warps = s.G / s.K * (s.TPG / 32.0), degree = (double)h.nnz / h.mb;
     double turns = (double)((n + V - 1) / V) / s.G;
@@ -182,7 +184,7 @@ static double shape_cost(const CodeDev &h, int msg, const SlotShape &s, int V, i
         if (span > s.W) span = s.W;
         rows *= 1.0 + 0.25 * (span - 1.0) * change;
     }
-    double c = (rows + 14.0 / degree) * turns * (warps > 20.0 ? warps : 20.0);
+    double c = (rows + 14.0 / degree) * turns * (warps > least ? warps : least);
     if (V == 2) c *= h.dc_max <= 12 || msg != LDPC_MSG_F16 ? 1.35 : form == FLOOD_WHOLE ? 1.55 : 1.9;
     if (form != FLOOD_WHOLE) c *= (form == FLOOD_SPREAD ? 1.0 + 2.1 / degree : 1.03) + 0.02 * (s.K - 1);
     return c;
@@ -354,7 +356,7 @@ cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, 
     }
     if (V == 2) {
         whole = shapes(2, FLOOD_WHOLE, pair);
-        if (whole == 0.0 || (one > 0.0 && one * 1.2 < whole)) {  // (clearly cheaper: fewer pairs fit than half the codewords)
+        if (whole == 0.0 || (p.msg != LDPC_MSG_F16 && one > 0.0 && one * 1.2 < whole)) {  // (too few pairs fit)
             V = 1;
             whole = tuned == SCHED_SLOTS_V2 ? shapes(1, FLOOD_WHOLE, shape) : one;
         } else {
@@ -362,20 +364,37 @@ cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, 
         }
     }
     if (whole == 0.0) return cudaErrorInvalidValue;
-    // rows end to end where a quarter of some code's warps would be idle and that is estimated 5 % cheaper
+    // rows end to end where that is estimated 5 % cheaper: packed if a quarter of some code's lanes would be
+    // idle, spread if a twentieth would be and a thread of one codeword has several rows
     out.form = FLOOD_WHOLE;
-    bool idle = false;
+    bool quarter = false, some = false, several = false;
     int64_t most = 0;  // (one codeword to an SM has nothing to be packed with)
     for (int g = 0; g < ng; g++) {
-        idle |= 4 * codes[g]->host.Z <= 3 * ((codes[g]->host.Z + 31) & ~31);
+        const int Z = codes[g]->host.Z, wt = (Z + 31) & ~31;
+        quarter |= 4 * Z <= 3 * wt;
+        some |= 20 * Z <= 19 * wt;
+        several |= shape[g].W < codes[g]->host.mb;
         most = per_sm[g] > most ? per_sm[g] : most;
     }
+    if (!quarter && (V == 2 || !several)) some = false;
     const struct { FloodForm form; int V; } other[3] = {{FLOOD_PACKED, 1}, {FLOOD_PACKED, 2}, {FLOOD_SPREAD, 1}};
-    for (int i = 0; i < 3 && idle; i++) {
+    for (int i = 0; i < 3 && some; i++) {
         SlotShape s[MULTI_MAX_GROUPS];
-        if ((tuned && other[i].V != V) || (other[i].form == FLOOD_PACKED && most < 2 * other[i].V)) continue;
+        if ((tuned && other[i].V != V) || (other[i].form == FLOOD_PACKED && (!quarter || most < 2 * other[i].V))) continue;
         const double cost = shapes(other[i].V, other[i].form, s);
-        if (cost > 0.0 && cost * (out.form ? 1.0 : 1.05) < whole) {
+        bool take = cost > 0.0 && cost * (out.form ? 1.0 : 1.05) < whole;
+        if (cost > 0.0 && !take && !out.form && V == 1 && other[i].form == FLOOD_SPREAD) {
+            double a = 0.0, b = 0.0;
+            take = true;
+            for (int g = 0; g < ng; g++) {
+                const CodeDev &h = codes[g]->host;
+                take &= h.dc_max > 12;
+                a += h.nnz / (double)h.mb * shape_cost(h, p.msg, shape[g], 1, per_sm[g], FLOOD_WHOLE, 0.0, 8.0);
+                b += h.nnz / (double)h.mb * shape_cost(h, p.msg, s[g], 1, per_sm[g], FLOOD_SPREAD, body_changes(h), 8.0);
+            }
+            take &= b * 1.3 < a;
+        }
+        if (take) {
             out.form = other[i].form;
             whole = cost;
             V = other[i].V;

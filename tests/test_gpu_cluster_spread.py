@@ -12,11 +12,11 @@ from tests.test_gpu_flood_shapes import base_of, decode
 pytestmark = pytest.mark.gpu
 
 CODES = {
-    "narrow_z66": (base_of([2, 3, 4, 5, 6, 7, 8, 8] * 8, 96, 66, 31), 66),
-    "to12_z68": (base_of([4, 9, 10, 11, 12, 12, 8, 7] * 8, 96, 68, 32), 68),
+    "narrow_z34": (base_of([2, 3, 4, 5, 6, 7, 8, 8] * 8, 72, 34, 31), 34),
+    "to12_z68": (base_of([4, 9, 10, 11, 12, 12, 8, 7] * 8, 80, 68, 32), 68),
     "wide_z65": (base_of([3, 13, 16, 17, 24, 25, 32, 12] * 6, 72, 65, 33), 65),
-    "wide_z36": (base_of([16] * 60, 120, 36, 34), 36),
-    "one_turn_z311": (base_of([13, 14, 15, 16] * 2, 17, 311, 35), 311),
+    "wide_z36": (base_of([16] * 56, 112, 36, 34), 36),
+    "one_group_z621": (base_of([13, 14, 15, 16] * 2, 17, 621, 35), 621),
 }
 
 
