@@ -128,7 +128,8 @@ ldpc_status ldpc_workspace_size(const ldpc_code *code, const ldpc_decode_params 
  *              (integer forms write their integer APP converted exactly to fp32).
  *   workspace  device scratch of >= ldpc_workspace_size() bytes, 256-byte aligned, or NULL
  *              to let the library allocate and free it stream-ordered on `stream` (the
- *              on-chip decoders take nothing for batches of up to one codeword per SM).
+ *              flooding and layered sum-product slot decoders, and the layered min-sum with
+ *              two codewords per thread, take nothing for up to one codeword per SM).
  * n_cw == 0 returns LDPC_OK with nothing launched. */
 ldpc_status ldpc_decode_batch(const ldpc_code *code, const ldpc_decode_params *p,
                               const void *llr_dev, int32_t llr_type, int64_t n_cw,

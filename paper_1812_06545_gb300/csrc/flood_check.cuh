@@ -107,7 +107,7 @@ struct OwnMem {
 // beta + d alpha), R = ln(alpha / beta) with the sign of the other edges.
 
 // d of each codeword.  HC: the upper clamp a >= phi(X) is applied; without it the clamp is
-// known not to change d (phi(X) so small that ex2 rounds e^-phi(X) to 1, see flood_slots.cu).
+// known not to change d (phi(X) so small that ex2 rounds e^-phi(X) to 1, see FLOOD_CLAMP_X).
 template <bool B2, bool HC>
 __device__ __forceinline__ float form_d(float q, float Xb, float Pb)
 {

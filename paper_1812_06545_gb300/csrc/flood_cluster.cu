@@ -61,9 +61,8 @@ struct ClusterArgs {
     // from here (neither loaded nor divided in the kernel) these are known to be warp-uniform: the
     // code's sizes, and W row groups of WT threads
     int Z, H, N, W, WT;
-    // the variable-node phase in quads: W4 groups of WT4 threads, wt4 = the warps' worth of quads
-    // of a column (W4 = 0: Z is no multiple of 4)
-    int W4, WT4, wt4, wide_L;
+    // the variable-node phase in quads: W4 groups of WT4 threads (W4 = 0: Z is no multiple of 4)
+    int W4, WT4, wide_L;
     int spread;  // rows and columns end to end over the threads instead
     int64_t n_items;
     unsigned long long *next;
@@ -492,9 +491,8 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
         for (int k = 3; dv > 4 && k < dv; k += 4) tab[x++] = make_int4(addr(k), addr(k + 1), addr(k + 2), addr(k + 3));
     }
     const uint32_t flag_0 = cl_map(flags, 0), flag_1 = cl_map(flags, 1);
-    // row groups of WT threads; when a row needs more threads than the CTA has, one group whose
-    // threads take positions ru, ru + nth, ...
-    const int wt = (H + 31) & ~31, W = a.W, WT = a.WT;
+    // row groups of WT threads (a row pair never needs more threads than a CTA has)
+    const int W = a.W, WT = a.WT;
     const int w0 = (int)__reduce_min_sync(0xffffffffu, (unsigned)(tid / WT));  // (a warp reduction: known to be uniform)
     const int ru = tid - w0 * WT;
     const bool works = w0 < W;
@@ -550,22 +548,19 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
                 cl_rows_spread<DMAX, MsgT, HC>(tab, rows, n_rows, ClusterMem<MsgT>{reinterpret_cast<char *>(smem)}, Z, H,
                                                tid, nth, Xb, Pb, pbad);
                 bad = pbad[0] | pbad[1];
-            } else if (works)
-                for (int rr = 0; rr < wt; rr += WT) {
-                    PairPlace p;
-                    const int r = rr + ru;
-                    p.own = r < H;
-                    p.r = p.own ? r : H - 1;
-                    p.own2 = p.own && p.r + H < Z;
-                    p.s = p.r + H < Z ? p.r + H : Z - 1;
-                    p.rw = p.r - Z;
-                    p.sw = p.s - Z;
-                    uint32_t pbad[2] = {0, 0};
-                    cl_rows<0, DMAX, MsgT, HC>(a.rend[q][w0], tab, rows,
-                                               ClusterMem<MsgT>{reinterpret_cast<char *>(smem)}, p, Xb, Pb, pbad,
-                                               a.rstart[q][w0]);
-                    bad |= pbad[0] | pbad[1];
-                }
+            } else if (works) {
+                PairPlace p;
+                p.own = ru < H;
+                p.r = p.own ? ru : H - 1;
+                p.own2 = p.own && p.r + H < Z;
+                p.s = p.r + H < Z ? p.r + H : Z - 1;
+                p.rw = p.r - Z;
+                p.sw = p.s - Z;
+                uint32_t pbad[2] = {0, 0};
+                cl_rows<0, DMAX, MsgT, HC>(a.rend[q][w0], tab, rows, ClusterMem<MsgT>{reinterpret_cast<char *>(smem)}, p,
+                                           Xb, Pb, pbad, a.rstart[q][w0]);
+                bad = pbad[0] | pbad[1];
+            }
             if (__any_sync(0xffffffffu, (bad & kSign) != 0) && (tid & 31) == 0) {
                 cl_st(flag_0 + 4 * (tr & 1), 1);
                 cl_st(flag_1 + 4 * (tr & 1), 1);
@@ -591,19 +586,14 @@ __global__ void __cluster_dims__(CLUSTER_CTAS, 1, 1) __launch_bounds__(cl_thread
                         });
                     }
                 } else if (a.W4 > 0) {
-                    const bool wide = a.wide_L;
-                    for (int qq = 0; qq < a.wt4; qq += a.WT4) {
-                        const int x = qq + ru4, xc = 4 * x < Z ? 4 * x : Z - 4;
-                        const VarQuad<MsgT> v{L + xc, (uint32_t)(SR * xc), app + xc, 4 * x < Z, wide};
-                        if (w4 < a.W4) cl_cols<1>(a.cend[q][w4], ctab, tab, cols, v, Z, a.cstart[q][w4]);
-                    }
+                    const int xc = 4 * ru4 < Z ? 4 * ru4 : Z - 4;
+                    const VarQuad<MsgT> v{L + xc, (uint32_t)(SR * xc), app + xc, 4 * ru4 < Z, a.wide_L != 0};
+                    if (w4 < a.W4) cl_cols<1>(a.cend[q][w4], ctab, tab, cols, v, Z, a.cstart[q][w4]);
                 } else if (works) {
-                    for (int rr = 0; rr < wt; rr += WT) {
-                        const int r = rr + ru, rc = r < H ? r : H - 1, sc = rc + H < Z ? rc + H : Z - 1;
-                        const VarPair<MsgT> v{L + rc,   L + sc,   (uint32_t)(SR * rc), (uint32_t)(SR * sc),
-                                              app + rc, app + sc, r < H,               r < H && rc + H < Z};
-                        cl_cols<1>(a.cend[q][w0], ctab, tab, cols, v, Z, a.cstart[q][w0]);
-                    }
+                    const int rc = ru < H ? ru : H - 1, sc = rc + H < Z ? rc + H : Z - 1;
+                    const VarPair<MsgT> v{L + rc,   L + sc,   (uint32_t)(SR * rc), (uint32_t)(SR * sc),
+                                          app + rc, app + sc, ru < H,              ru < H && rc + H < Z};
+                    cl_cols<1>(a.cend[q][w0], ctab, tab, cols, v, Z, a.cstart[q][w0]);
                 }
                 t++;
             }
@@ -700,11 +690,10 @@ static size_t cl_plan(const CodeDev &h, int msg, ClusterArgs &a, size_t limit)
     const int nth = h.dc_max <= 12 ? cl_threads<12>() : cl_threads<32>();
     a.Z = h.Z;
     a.H = (h.Z + 1) / 2;
-    const int wt = (a.H + 31) & ~31;
-    a.W = wt <= nth ? nth / wt : 1;
-    a.WT = wt <= nth ? wt : nth;
-    a.wt4 = (a.Z / 4 + 31) & ~31;
-    a.WT4 = a.Z % 4 ? 32 : a.wt4 <= nth ? a.wt4 : nth;
+    static_assert(Z_MAX / 2 <= cl_threads<32>(), "a row pair's threads");
+    a.WT = (a.H + 31) & ~31;
+    a.W = nth / a.WT;
+    a.WT4 = a.Z % 4 ? 32 : (a.Z / 4 + 31) & ~31;
     a.W4 = a.Z % 4 ? 0 : nth / a.WT4;
     // end to end over the threads where that leaves so few turns of the rows (about two thirds of the
     // time) and the columns that it pays for the votes.  (GB300, FP16, us per launch, groups of whole

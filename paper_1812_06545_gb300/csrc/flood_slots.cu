@@ -40,7 +40,7 @@
 //
 // What bounds it, and what the shape measured (GB300, 8192 codewords of the N = 1944 rate-1/2
 // code, 1.75 dB FP32 / 2.25 dB FP16, per launch): instruction issue and its latencies, not the
-// special-function units (0.30 of their ceiling) nor shared memory.
+// special-function units (0.35 of their ceiling) nor shared memory.
 //   one codeword per thread, lock-step over the CTA          1225 us FP32
 //   two per thread and barrier groups of three slots                        790 us FP16
 //   two per thread, two row groups, one slot per barrier       964            679

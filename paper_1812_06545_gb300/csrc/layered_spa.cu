@@ -749,7 +749,7 @@ cudaError_t layered_spa_decode(const CodeDev &h, const CodeDev *d, const ldpc_de
     const int g1 = lspa_fit(h, p.msg, 1, cap1), g2 = lspa_fit(h, p.msg, 2, cap2);
     // two codewords per thread where that holds more codewords per CTA than the threads allow one
     // to a thread: FP16 messages, rows of degree <= 8.  (8192 codewords on GB300, one against two:
-    // N = 1944 rate 1/2 FP16 507 / 467 us, 10 slots against 6 pairs; FP32 486 / 597, 7 against 3;
+    // N = 1944 rate 1/2 FP16 507 / 467 us, 10 slots against 6 pairs; FP32 502 / 626, 7 against 3;
     // rate 5/6 FP16 489 / 545: there single slots of more warps win.)
     const bool pairs = f16 && h.dc_max <= 8;
     int V = pairs && per_sm > g1 && 2 * g2 > g1 ? 2 : 1;
