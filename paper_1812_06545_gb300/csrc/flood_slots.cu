@@ -51,8 +51,6 @@
 #include <math.h>
 #include <string.h>
 
-#include <numeric>
-
 #include "flood_slots.h"
 
 namespace ldpc {
@@ -179,8 +177,8 @@ static double shape_cost(const CodeDev &h, int msg, const SlotShape &s, int V, i
     turns = turns < 8.0 ? ceil(turns) : turns + 0.5;
     double rows = (h.mb + s.W - 1) / s.W;
     if (form == FLOOD_SPREAD) {
-        const int block = s.K * h.Z;
-        double span = 1.0 + (32 - std::gcd(block, 32)) / (double)block;
+        const int block = s.K * h.Z, two = block & -block;  // (its largest power of two)
+        double span = 1.0 + (32 - (two < 32 ? two : 32)) / (double)block;
         if (span > s.W) span = s.W;
         rows *= 1.0 + 0.25 * (span - 1.0) * change;
     }
@@ -376,7 +374,7 @@ cudaError_t flood_plan(const HostReq *reqs, int n, const ldpc_decode_params &p, 
         several |= shape[g].W < codes[g]->host.mb;
         most = per_sm[g] > most ? per_sm[g] : most;
     }
-    if (!quarter && (V == 2 || !several)) some = false;
+    if (!quarter && (ng > 1 || V == 2 || !several)) some = false;  // (not worth the host's time for many codes)
     const struct { FloodForm form; int V; } other[3] = {{FLOOD_PACKED, 1}, {FLOOD_PACKED, 2}, {FLOOD_SPREAD, 1}};
     for (int i = 0; i < 3 && some; i++) {
         SlotShape s[MULTI_MAX_GROUPS];
